@@ -2,9 +2,10 @@
 // programmes in format 2 (tileprog.h).
 //
 // Per tile (persistent grid, two CTAs per SM, 256 threads each, 32 amplitudes per thread):
-//   1. one warp issues 2^(13-c) bulk copies (TMA, cp.async.bulk) of the
-//      tile's contiguous 2^c-amplitude chunks into shared memory, completing
-//      on an mbarrier;
+//   1. one warp copies the tile into shared memory (TMA), completing on an
+//      mbarrier: k_tile2 by one to a few tensor copies (tilemap.h), the L2
+//      block and batched kernels by 2^(13-c) bulk copies of its contiguous
+//      2^c-amplitude chunks;
 //   2. the pass's per-tile diagonal data (global-qubit contributions, which
 //      are constants of the tile: Sec. III-B of arxiv 2605.15098) is summed
 //      as integer phases while the copies are in flight, then turned into the
@@ -721,9 +722,16 @@ __global__ void k_slotv(const T2Args a, float2 *__restrict__ out) {
 // the rest of tile i's programme and its write-back, which goes from
 // registers straight to the global state (16-byte stores; lanes 0..7 cover
 // tile bits 1..3, so a quarter-warp writes 128 contiguous bytes).
+// The copies are tensor copies of whole runs of local bits (tilemap.h) and a
+// tile's base is one masked addition on the previous one.  With one bulk copy
+// per 2^c-amplitude chunk, the 256 of a c = 5 tile were issued lane by lane
+// by warp 0, and the other warps waited for it: random circuit n = 28, depth
+// 8: 27.5 -> 22.6 ms, a middle pass at n = 25 642 -> 555 us; with c = 9 (16
+// chunks) QPE n = 28 3.94 -> 3.89 ms.
 template <int K, int F>
 __global__ void __launch_bounds__(Geo<K>::kThreads, K == kT2Qubits ? 2 : 1)
-    k_tile2(float *__restrict__ state, const T2Args a) {
+    k_tile2(float *__restrict__ state, const T2Args a, const __grid_constant__ CUtensorMap map,
+            const __grid_constant__ TileBox box) {
     using G = Geo<K>;
     extern __shared__ __align__(1024) unsigned char sm[];
     float2 *tab = reinterpret_cast<float2 *>(sm + G::kOffTab);
@@ -749,9 +757,24 @@ __global__ void __launch_bounds__(Geo<K>::kThreads, K == kT2Qubits ? 2 : 1)
         mbar_expect_tx(bar, (uint32_t)a.nsp * 8u);
         bulk_g2s(dst, a.slotv + t * (uint64_t)a.nsp, (uint32_t)a.nsp * 8u, bar);
     };
+    // the copies of tile t, whose global bits are b, by warp 0
+    auto issue_load = [&](uint64_t t, uint64_t b, float2 *slots) {
+        if (tid == 0) {
+            fence_async_smem();
+            const uint32_t sb = slots ? (uint32_t)a.nsp * 8u : 0u;
+            mbar_expect_tx(bar, G::kTileBytes + sb);
+            if (slots) bulk_g2s(slots, a.slotv + t * (uint64_t)a.nsp, sb, bar);
+        }
+        __syncwarp();
+        tensor_tile_load(&map, box, b, sm, bar, tid);
+    };
+    // the base of the tile gridDim.x further on: an addition on the global
+    // bits alone (the ones between them pass the carries on)
+    const uint64_t step = tile_base(a, gridDim.x);
+    uint64_t base = tile_base(a, blockIdx.x);
     if ((uint64_t)blockIdx.x < a.ntiles) {
         if (!a.gen && tid < 32)
-            issue_tile_load<K>(a, sm, state, blockIdx.x, bar, tid, pre ? slotc : nullptr);
+            issue_load(blockIdx.x, base, pre ? slotc : nullptr);
         else if (a.gen && pre && tid == 0)
             issue_slots_only(blockIdx.x, slotc);
     }
@@ -759,7 +782,7 @@ __global__ void __launch_bounds__(Geo<K>::kThreads, K == kT2Qubits ? 2 : 1)
     uint32_t parity = 0, rd = 0, buf = 0;
     for (uint64_t tile = blockIdx.x; tile < a.ntiles; tile += gridDim.x) {
         const uint64_t next = tile + gridDim.x;
-        const uint64_t base = tile_base(a, tile);
+        const uint64_t next_base = ((base | ~a.gmask) + step) & a.gmask;
         // the tile's slot values while its copies are in flight, into the
         // buffer the previous tile did not use (every warp passed that tile's
         // barrier below, so none still reads the one before)
@@ -776,7 +799,7 @@ __global__ void __launch_bounds__(Geo<K>::kThreads, K == kT2Qubits ? 2 : 1)
             float2 *nsc = slotc + (buf ^ 1u) * kT2MaxSlots;
             if (!a.gen && tid < 32 && next < a.ntiles) {
                 if (!mbar_wait(rbar, (rd - 1u) & 1u)) atomicExch(a.err, 1);
-                issue_tile_load<K>(a, sm, state, next, bar, tid, pre ? nsc : nullptr);
+                issue_load(next, next_base, pre ? nsc : nullptr);
             } else if (a.gen && pre && tid == 0 && next < a.ntiles) {
                 issue_slots_only(next, nsc);
             }
@@ -784,6 +807,7 @@ __global__ void __launch_bounds__(Geo<K>::kThreads, K == kT2Qubits ? 2 : 1)
         t2_run<K, F>(a, reinterpret_cast<float4 *>(state), rbar, rd, base, sc, hook);
         parity ^= 1u;
         buf ^= 1u;
+        base = next_base;
     }
 }
 
@@ -1344,8 +1368,11 @@ sv_status t2_launch(sv_state *h, const T2Pass &p, const T2Device &d, const sv_la
     if (per_sm < 1) return fail(SV_ERR_UNSUPPORTED, "register-stage tile kernel does not fit");
     h->stats.ctas_per_sm = h->stats.ctas_per_sm ? std::min(h->stats.ctas_per_sm, per_sm) : per_sm;
     const uint64_t grid = std::min<uint64_t>(a.ntiles, (uint64_t)per_sm * h->sm_count);
+    CUtensorMap map{};
+    TileBox box{};
+    if (!a.gen) SV_TRY(tile_map(h->amps, h->n, p.k, p.slot_phys, sizeof(float2), &map, &box));
     const int slot = prof_begin(h);
-    kern<<<(unsigned)grid, threads, smem, h->stream>>>(reinterpret_cast<float *>(h->amps), a);
+    kern<<<(unsigned)grid, threads, smem, h->stream>>>(reinterpret_cast<float *>(h->amps), a, map, box);
     SV_CUDA(cudaGetLastError());
     note_launch();
     prof_end(h, slot, meta);

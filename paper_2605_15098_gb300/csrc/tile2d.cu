@@ -4,8 +4,8 @@
 //
 // Per tile (persistent grid, one CTA per SM, 256 threads, 32 amplitudes per
 // thread held as 64 FP64 registers):
-//   1. one warp issues 2^(13-c) bulk copies of the tile's 2^c-amplitude chunks
-//      into shared memory (128 KiB), completing on an mbarrier;
+//   1. one warp copies the tile into shared memory (128 KiB) by one to a few
+//      tensor copies (tilemap.h), completing on an mbarrier;
 //   2. the tile's slot values (its global-qubit phase terms, Sec. III-B) are
 //      summed as exact 64-bit phases while the copies are in flight and
 //      turned into e^{2 pi i u / 2^64} from three FP64-generated tables;
@@ -551,24 +551,6 @@ __device__ __forceinline__ uint64_t tile_base_d(const T2Args &a, uint64_t tile) 
     return b;
 }
 
-__device__ __forceinline__ void issue_tile_load_d(const T2Args &a, unsigned char *sm, const double2 *state,
-                                                  uint64_t tile, uint64_t *bar, int tid) {
-    const int nchunks = 1 << (kT2Qubits - a.c);
-    const uint32_t chunk_bytes = 16u << a.c;
-    const uint64_t base = tile_base_d(a, tile);
-    if (tid == 0) {
-        fence_async_smem();
-        mbar_expect_tx(bar, (uint32_t)GD::kTileBytes);
-    }
-    __syncwarp();
-    for (int j = tid; j < nchunks; j += 32) {
-        uint64_t off = 0;
-        for (int b = 0; b < kT2Qubits - a.c; b++)
-            if ((j >> b) & 1) off |= UINT64_C(1) << a.slot_phys[a.c + b];
-        bulk_g2s(sm + (size_t)j * chunk_bytes, state + base + off, chunk_bytes, bar);
-    }
-}
-
 __device__ __forceinline__ void load_programme_d(const T2Args &a, unsigned char *sm, int tid, int nthreads) {
     int4 *si = reinterpret_cast<int4 *>(sm + GD::kOffIns);
     int4 *sf = reinterpret_cast<int4 *>(sm + GD::kOffFac);
@@ -622,7 +604,9 @@ __device__ __forceinline__ void tile_slots_d(const T2Args &a, double2 *slotc, ui
 // Persistent CTA over the pass's tiles; tile i+1's copies start once tile i's
 // last stage change has read shared memory.
 template <int F>
-__global__ void __launch_bounds__(kDThreads, 1) k_tile2d(double2 *__restrict__ state, const T2Args a) {
+__global__ void __launch_bounds__(kDThreads, 1)
+    k_tile2d(double2 *__restrict__ state, const T2Args a, const __grid_constant__ CUtensorMap map,
+             const __grid_constant__ TileBox box) {
     extern __shared__ __align__(1024) unsigned char sm[];
     double2 *slotc = reinterpret_cast<double2 *>(sm + GD::kOffSlotc);
     uint64_t *bar = reinterpret_cast<uint64_t *>(sm + GD::kOffBar);
@@ -635,12 +619,24 @@ __global__ void __launch_bounds__(kDThreads, 1) k_tile2d(double2 *__restrict__ s
         fence_mbar_init();
     }
     __syncthreads();
-    if (!a.gen && tid < 32 && (uint64_t)blockIdx.x < a.ntiles)
-        issue_tile_load_d(a, sm, state, blockIdx.x, bar, tid);
+    // the copies of the tile whose global bits are b, by warp 0 (in 8-byte
+    // words: an amplitude is two)
+    auto issue_load = [&](uint64_t b) {
+        if (tid == 0) {
+            fence_async_smem();
+            mbar_expect_tx(bar, (uint32_t)GD::kTileBytes);
+        }
+        __syncwarp();
+        tensor_tile_load(&map, box, b << 1, sm, bar, tid);
+    };
+    // the base of the tile gridDim.x further on: an addition on the global bits
+    const uint64_t step = tile_base_d(a, gridDim.x);
+    uint64_t base = tile_base_d(a, blockIdx.x);
+    if (!a.gen && tid < 32 && (uint64_t)blockIdx.x < a.ntiles) issue_load(base);
     uint32_t parity = 0, rd = 0, buf = 0;
     for (uint64_t tile = blockIdx.x; tile < a.ntiles; tile += gridDim.x) {
         const uint64_t next = tile + gridDim.x;
-        const uint64_t base = tile_base_d(a, tile);
+        const uint64_t next_base = ((base | ~a.gmask) + step) & a.gmask;
         double2 *sc = slotc + buf * kT2MaxSlots;
         tile_slots_d(a, sc, base, tid);
         const bool timed_out = a.gen ? false : !mbar_wait(bar, parity);
@@ -652,12 +648,13 @@ __global__ void __launch_bounds__(kDThreads, 1) k_tile2d(double2 *__restrict__ s
         auto hook = [&]() {
             if (!a.gen && tid < 32 && next < a.ntiles) {
                 if (!mbar_wait(rbar, (rd - 1u) & 1u)) atomicExch(a.err, 1);
-                issue_tile_load_d(a, sm, state, next, bar, tid);
+                issue_load(next_base);
             }
         };
         t2d_run<F>(a, state, rbar, rd, base, sc, hook);
         parity ^= 1u;
         buf ^= 1u;
+        base = next_base;
     }
 }
 
@@ -686,8 +683,12 @@ sv_status t2d_launch(sv_state *h, const T2Pass &p, const T2Device &d, const sv_l
     if (per_sm < 1) return fail(SV_ERR_UNSUPPORTED, "complex128 register-stage kernel does not fit");
     h->stats.ctas_per_sm = h->stats.ctas_per_sm ? std::min(h->stats.ctas_per_sm, per_sm) : per_sm;
     const uint64_t grid = std::min<uint64_t>(a.ntiles, (uint64_t)per_sm * h->sm_count);
+    CUtensorMap map{};
+    TileBox box{};
+    if (!a.gen) SV_TRY(tile_map(h->amps, h->n, p.k, p.slot_phys, sizeof(double2), &map, &box));
     const int slot = prof_begin(h);
-    kern<<<(unsigned)grid, kDThreads, GD::kSmemBytes, h->stream>>>(reinterpret_cast<double2 *>(h->amps), a);
+    kern<<<(unsigned)grid, kDThreads, GD::kSmemBytes, h->stream>>>(reinterpret_cast<double2 *>(h->amps), a, map,
+                                                                   box);
     SV_CUDA(cudaGetLastError());
     note_launch();
     prof_end(h, slot, meta);

@@ -8,6 +8,7 @@
 
 #include <cstdint>
 
+#include "tilemap.h"
 #include "tileprog.h"
 
 namespace sv {
@@ -62,6 +63,32 @@ __device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint32_t by
             saddr(dst)),
         "l"(src), "r"(bytes), "r"(saddr(bar))
         : "memory");
+}
+// One box of a five-dimensional tensor (tilemap.h) into shared memory.
+__device__ __forceinline__ void tensor_g2s(void *dst, const CUtensorMap *map, const int x[kTileDims], uint64_t *bar) {
+    asm volatile(
+        "cp.async.bulk.tensor.5d.shared::cluster.global.tile.mbarrier::complete_tx::bytes "
+        "[%0], [%1, {%2, %3, %4, %5, %6}], [%7];" ::"r"(saddr(dst)),
+        "l"(map), "r"(x[0]), "r"(x[1]), "r"(x[2]), "r"(x[3]), "r"(x[4]), "r"(saddr(bar))
+        : "memory");
+}
+// The copies of the tile whose global bits are `wbase` (8-byte words), by the
+// lanes of one warp: one tensor copy for each value of the bits beyond the
+// box's dimensions.  One copy of the whole tile instead of one per chunk of
+// 2^c amplitudes: with c = 5 the 256 chunk copies of a tile, issued one lane
+// at a time with their offsets, took more instructions on the issuing warp
+// than the tile's programme (random circuit, n = 28, depth 8: see k_tile2).
+__device__ __forceinline__ void tensor_tile_load(const CUtensorMap *map, const TileBox &box, uint64_t wbase,
+                                                 unsigned char *dst, uint64_t *bar, int lane) {
+    for (int e = lane; e < (1 << box.next); e += 32) {
+        uint64_t w = wbase;
+        for (int i = 0; i < box.next; i++)
+            if ((e >> i) & 1) w |= UINT64_C(1) << box.ext[i];
+        int x[kTileDims];
+#pragma unroll
+        for (int i = 0; i < kTileDims; i++) x[i] = (int)((uint32_t)(w >> box.pos[i]) & box.mask[i]);
+        tensor_g2s(dst + (size_t)e * box.copy_bytes, map, x, bar);
+    }
 }
 __device__ __forceinline__ void bulk_s2g(void *dst, const void *src, uint32_t bytes) {
     asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst),
