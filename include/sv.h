@@ -114,7 +114,11 @@ typedef struct sv_gate {
 
 /* Execution strategy for sv_apply_circuit. */
 typedef enum {
-    SV_MODE_AUTO = 0,        /* partitioned when n is larger than a tile      */
+    SV_MODE_AUTO = 0,        /* partitioned from n = 16 up; below, the gates of
+                                the list applied in order on a state resident
+                                in shared memory (3 <= n <= 15, complex128
+                                14): one launch for hundreds of gates, with
+                                the results of SV_MODE_PERGATE              */
     SV_MODE_PERGATE = 1,     /* one HBM sweep per gate (Algorithm 1 per gate)  */
     SV_MODE_PARTITIONED = 2, /* tile passes (Sec. III-B), shared-memory tiles  */
     SV_MODE_FUSED = 3        /* partitioned + 5-qubit blocks on tensor cores   */

@@ -156,6 +156,11 @@ void prof_end(sv_state *h, int slot, const sv_launch_record &meta);
 // ---- per-gate path (pergate.cu) ---------------------------------------------
 // Apply one gate whose qubits are already PHYSICAL positions.
 sv_status pergate_apply(sv_state *h, const sv_gate &g_phys);
+// The resident kernel (small.cu): a run of such gates on a state that fits one
+// cluster's shared memory, in one launch per few hundred gates, with the
+// per-gate kernels' results.
+bool small_fits(int n, sv_dtype dt);
+sv_status small_apply(sv_state *h, const std::vector<sv_gate> &gates_phys);
 // Set the state to |0...0> (recorded only; see sv_state::basis).
 sv_status init_zero_state(sv_state *h);
 // Write a recorded basis state into the buffer (no-op when it holds the state).
