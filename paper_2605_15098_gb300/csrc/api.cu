@@ -63,6 +63,11 @@ sv_status make_handle(int n, sv_dtype dt, void *buf, size_t bytes, void *stream,
         cudaGetLastError();
         return bail(fail(SV_ERR_OOM, "cannot allocate reduction buffer"));
     }
+    // the read-outs' arrival counter (measure.cu) starts at zero
+    if (cudaMemsetAsync(static_cast<char *>(h->small) + 65536 - 64, 0, 64, h->stream) != cudaSuccess) {
+        cudaError_t e = cudaGetLastError();
+        return bail(fail(SV_ERR_CUDA, "cannot clear the reduction buffer: %s", cudaGetErrorString(e)));
+    }
     sv_status st = init_zero_state(h);
     if (st != SV_OK) return bail(st);
     *out = h;
@@ -332,17 +337,9 @@ sv_status sv_argmax(sv_handle h, uint64_t qubit_mask, uint64_t *host_idx, double
     clear_error();
     if (!h || !host_idx) return fail(SV_ERR_ARG, "NULL argument");
     SV_TRY(check_mask(h, qubit_mask));
-    // the argmax does not need the normalised vector: only max / total
     int pos[64];
     const int m = mask_positions(h, qubit_mask, pos);
-    const uint64_t len = UINT64_C(1) << m;
-    SV_TRY(ensure_probs(h, len * sizeof(double)));
-    const double *sums = nullptr;
-    int nsums = 0;
-    // the marginal stays in physical order (coalesced stores whatever the qubit map)
-    OutPerm perm{};
-    SV_TRY(marginal_device(h, pos, m, h->probs, false, &sums, &nsums, &perm));
-    return argmax_device(h, h->probs, len, host_idx, host_p, sums, nsums, &perm);
+    return argmax_device(h, pos, m, host_idx, host_p);
 }
 
 sv_status sv_sample(sv_handle h, uint64_t qubit_mask, const double *host_u, size_t shots,

@@ -198,18 +198,10 @@ struct OutPerm {
 
 // Marginal over physical positions pos[0..m-1] (output bit j <-> pos[j]),
 // renormalised, into device buffer dev_out (2^m doubles), on h->stream.
-// normalise = false leaves the sums unnormalised and returns the block sums
-// whose ordered total is the normaliser (sums_out / nsums_out may be NULL).
-// With perm_out given, the entries stay in physical order (coalesced stores
-// whatever the qubit map) and *perm_out says how to read them.
-sv_status marginal_device(sv_state *h, const int *pos, int m, double *dev_out,
-                          bool normalise = true, const double **sums_out = nullptr,
-                          int *nsums_out = nullptr, OutPerm *perm_out = nullptr);
-// Lowest output index of the maximum of dev_p (entries ordered as `perm`
-// says); with sums given, dev_p is unnormalised and *host_p is max / total.
-sv_status argmax_device(sv_state *h, const double *dev_p, uint64_t len,
-                        uint64_t *host_idx, double *host_p, const double *sums = nullptr,
-                        int nsums = 0, const OutPerm *perm = nullptr);
+sv_status marginal_device(sv_state *h, const int *pos, int m, double *dev_out);
+// Lowest output index of that marginal's maximum, and the maximum; the
+// marginal itself is not written.
+sv_status argmax_device(sv_state *h, const int *pos, int m, uint64_t *host_idx, double *host_p);
 sv_status sample_device(sv_state *h, const double *dev_p, uint64_t len,
                         const double *host_u, size_t shots, uint64_t *host_out);
 

@@ -3,13 +3,19 @@
 //
 // All sums run in a fixed order, so a call returns the same bits every time:
 //   1. partial[g][m] = sum of |amp|^2 over the g-th slice of the amplitudes
-//      that map to outcome m, summed in increasing index order;
-//   2. p[m] = sum over g of partial[g][m], in g order;
-//   3. total = fixed two-level tree over p; p[m] /= total.
+//      that map to outcome m, summed in increasing index order; slices of one
+//      thread block that share an outcome are added in a fixed tree;
+//   2. p[m] = sum over the partials in a fixed tree;
+//   3. total = block sums in a fixed tree; p[m] /= total.
+// Every read-out is one kernel over the state and at most one over the
+// partials (plus the division of a large marginal): each thread block leaves
+// its sum and its largest outcome, and the last block to finish combines them
+// in block order.
 // Sampling builds the inclusive CDF in blocks of 1024 outcomes (in-block
 // running sums in index order, block totals accumulated in block order) and
 // binary-searches the smallest i with C_i > u * C_last for each shot.
 #include <algorithm>
+#include <type_traits>
 
 #include "common.h"
 
@@ -17,6 +23,10 @@ namespace sv {
 namespace {
 
 constexpr int kRedThreads = 256;
+// Resident blocks per SM of the marginal kernels: 64 registers hold eight
+// 16-byte loads per thread in flight (128 KiB per SM); a grid that walks the
+// outcomes has exactly these blocks.
+constexpr int kRedBlocks = 4;
 
 struct MargArgs {
     int n;
@@ -28,6 +38,8 @@ struct MargArgs {
     int out_bit[34];          // logical output bit of spos[k]
     uint64_t per_group;       // enumerated rest values per group
     int groups_log2;
+    int in_order;             // the output order is the physical one
+    uint64_t flush;           // values a thread sums before it adds them to its FP64 sum
 };
 
 __device__ __forceinline__ uint64_t pdep_mask(uint64_t v, uint64_t mask) {
@@ -55,13 +67,18 @@ constexpr int kLoadBatch = 8;
 template <>
 struct ProbAcc<double> {
     using V = double2;
-    double acc = 0.0;
+    // one multiply-add per component (the FP64 pipe bounds this), into sums of
+    // half the size each: fewer roundings than adding the squared modulus
+    double re = 0.0, im = 0.0;
     __device__ static V load(const double *s, uint64_t x) {
         return reinterpret_cast<const double2 *>(s)[x];
     }
-    __device__ void add(V v) { acc += v.x * v.x + v.y * v.y; }
+    __device__ void add(V v) {
+        re = fma(v.x, v.x, re);
+        im = fma(v.y, v.y, im);
+    }
     __device__ void add(const double *s, uint64_t x) { add(load(s, x)); }
-    __device__ double value() const { return acc; }
+    __device__ double value() const { return re + im; }
 };
 
 template <>
@@ -87,194 +104,59 @@ struct ProbAcc<float> {
     __device__ double value() const { return (double)hi + (double)lo; }
 };
 
-// Layout M: outcome bit 0 is physical bit 0, so consecutive threads (consecutive
-// physical-order outcomes) read neighbouring amplitudes.
-template <typename R>
-__global__ void __launch_bounds__(kRedThreads)
-k_marg_m(const R *__restrict__ s, MargArgs a, double *__restrict__ partial) {
-    const uint64_t outcomes = UINT64_C(1) << a.m;
-    const uint64_t tid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (tid >= (outcomes << a.groups_log2)) return;
-    const uint64_t mp = tid & (outcomes - 1);
-    const uint64_t g = tid >> a.m;
-    uint64_t xm = 0, ml = 0;
-    for (int k = 0; k < a.m; k++) {
-        if ((mp >> k) & 1) {
-            xm |= UINT64_C(1) << a.spos[k];
-            ml |= UINT64_C(1) << a.out_bit[k];
-        }
-    }
-    uint64_t xr = pdep_mask(g * a.per_group, a.rest);
-    ProbAcc<R> acc;
-    uint64_t i = 0;
-    // kLoadBatch loads in flight per thread, then accumulated in order
-    for (; i + kLoadBatch <= a.per_group; i += kLoadBatch) {
-        typename ProbAcc<R>::V v[kLoadBatch];
-#pragma unroll
-        for (int k = 0; k < kLoadBatch; k++) {
-            v[k] = ProbAcc<R>::load(s, xm | xr);
-            xr = ((xr | ~a.rest) + 1) & a.rest;
-        }
-#pragma unroll
-        for (int k = 0; k < kLoadBatch; k++) acc.add(v[k]);
-    }
-    for (; i < a.per_group; i++) {
-        acc.add(s, xm | xr);
-        xr = ((xr | ~a.rest) + 1) & a.rest;
-    }
-    partial[g * outcomes + ml] = acc.value();
+__device__ __forceinline__ void add_vec(ProbAcc<float> &a, ProbAcc<float> &b, float4 v) {
+    a.add(make_float2(v.x, v.y));
+    b.add(make_float2(v.z, v.w));
+}
+__device__ __forceinline__ void add_vec(ProbAcc<float> &a, ProbAcc<float> &, float2 v) { a.add(v); }
+__device__ __forceinline__ void add_vec(ProbAcc<double> &a, ProbAcc<double> &, double2 v) { a.add(v); }
+
+// What a read-out leaves besides the marginal itself.
+struct ReadResult {
+    double total;   // sum of the marginal
+    double recip;   // 1 / total
+    double best;    // its maximum divided by the total
+    uint64_t idx;   // lowest output index of the maximum
+};
+
+// Scratch of a reduction over thread blocks, in the handle's 64 KiB area.
+constexpr int kMaxStatBlocks = 2048;
+struct Stats {
+    double *sum, *best;
+    uint64_t *idx;
+    ReadResult *res;
+    unsigned *done;  // zero between launches
+};
+constexpr size_t kStatRes = 3 * 8 * kMaxStatBlocks, kStatDone = 65536 - 64;
+static_assert(kStatRes + sizeof(ReadResult) <= kStatDone, "reduction scratch");
+
+Stats stats_of(sv_state *h) {
+    char *b = reinterpret_cast<char *>(h->small);
+    Stats s;
+    s.sum = reinterpret_cast<double *>(b);
+    s.best = s.sum + kMaxStatBlocks;
+    s.idx = reinterpret_cast<uint64_t *>(s.best + kMaxStatBlocks);
+    s.res = reinterpret_cast<ReadResult *>(b + kStatRes);
+    s.done = reinterpret_cast<unsigned *>(b + kStatDone);
+    return s;
 }
 
-// Layout M, complex64: each thread takes the two outcomes that differ in
-// physical bit 0 (one 16-byte load covers both amplitudes), each summed in
-// the same order as k_marg_m.
-__global__ void __launch_bounds__(kRedThreads)
-k_marg_m2(const float *__restrict__ s, MargArgs a, double *__restrict__ partial) {
-    const uint64_t outcomes = UINT64_C(1) << a.m;
-    const uint64_t half = outcomes >> 1;
-    const uint64_t tid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (tid >= (half << a.groups_log2)) return;
-    const uint64_t mp = (tid & (half - 1)) << 1;
-    const uint64_t g = tid >> (a.m - 1);
-    uint64_t xm = 0, ml = 0;
-    for (int k = 1; k < a.m; k++) {
-        if ((mp >> k) & 1) {
-            xm |= UINT64_C(1) << a.spos[k];
-            ml |= UINT64_C(1) << a.out_bit[k];
-        }
-    }
-    const uint64_t ml1 = ml | (UINT64_C(1) << a.out_bit[0]);
-    uint64_t xr = pdep_mask(g * a.per_group, a.rest);
-    ProbAcc<float> acc0, acc1;
-    const float4 *s4 = reinterpret_cast<const float4 *>(s);
-    uint64_t i = 0;
-    for (; i + kLoadBatch <= a.per_group; i += kLoadBatch) {
-        float4 v[kLoadBatch];
-#pragma unroll
-        for (int k = 0; k < kLoadBatch; k++) {
-            v[k] = s4[(xm | xr) >> 1];
-            xr = ((xr | ~a.rest) + 1) & a.rest;
-        }
-#pragma unroll
-        for (int k = 0; k < kLoadBatch; k++) {
-            acc0.add(make_float2(v[k].x, v[k].y));
-            acc1.add(make_float2(v[k].z, v[k].w));
-        }
-    }
-    for (; i < a.per_group; i++) {
-        const float4 v = s4[(xm | xr) >> 1];
-        acc0.add(make_float2(v.x, v.y));
-        acc1.add(make_float2(v.z, v.w));
-        xr = ((xr | ~a.rest) + 1) & a.rest;
-    }
-    partial[g * outcomes + ml] = acc0.value();
-    partial[g * outcomes + ml1] = acc1.value();
-}
-
-// Layout R: the lowest physical bits are summed over; one warp per
-// (group, outcome), lanes take the five lowest rest bits.
-template <typename R>
-__global__ void __launch_bounds__(kRedThreads)
-k_marg_r(const R *__restrict__ s, MargArgs a, double *__restrict__ partial) {
-    const uint64_t outcomes = UINT64_C(1) << a.m;
-    const uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (warp >= (outcomes << a.groups_log2)) return;
-    const uint64_t mp = warp & (outcomes - 1);
-    const uint64_t g = warp >> a.m;
-    uint64_t xm = 0, ml = 0;
-    for (int k = 0; k < a.m; k++) {
-        if ((mp >> k) & 1) {
-            xm |= UINT64_C(1) << a.spos[k];
-            ml |= UINT64_C(1) << a.out_bit[k];
-        }
-    }
-    const uint64_t lane_bits = a.rest & ~a.upper;
-    const uint64_t xl = pdep_mask((uint64_t)lane, lane_bits);
-    uint64_t xo = pdep_mask(g * a.per_group, a.upper);
-    ProbAcc<R> pa;
-    uint64_t i = 0;
-    for (; i + kLoadBatch <= a.per_group; i += kLoadBatch) {
-        typename ProbAcc<R>::V v[kLoadBatch];
-#pragma unroll
-        for (int k = 0; k < kLoadBatch; k++) {
-            v[k] = ProbAcc<R>::load(s, xm | xo | xl);
-            xo = ((xo | ~a.upper) + 1) & a.upper;
-        }
-#pragma unroll
-        for (int k = 0; k < kLoadBatch; k++) pa.add(v[k]);
-    }
-    for (; i < a.per_group; i++) {
-        pa.add(s, xm | xo | xl);
-        xo = ((xo | ~a.upper) + 1) & a.upper;
-    }
-    double acc = pa.value();
-#pragma unroll
-    for (int off = 16; off; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-    if (lane == 0) partial[g * outcomes + ml] = acc;
-}
-
-__global__ void k_sum_groups(const double *__restrict__ partial, uint64_t outcomes, int groups,
-                             double *__restrict__ out) {
-    const uint64_t m = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (m >= outcomes) return;
-    double acc = 0.0;
-    for (int g = 0; g < groups; g++) acc += partial[(uint64_t)g * outcomes + m];
-    out[m] = acc;
-}
-
-// Block sums of x[0..len) (each thread sums a strided slice, then a fixed tree).
-__global__ void __launch_bounds__(kRedThreads)
-k_block_sum(const double *__restrict__ x, uint64_t len, double *__restrict__ sums) {
-    __shared__ double sh[kRedThreads];
-    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-    double acc = 0.0;
-    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < len; i += stride)
-        acc += x[i];
-    sh[threadIdx.x] = acc;
-    __syncthreads();
-    for (int w = kRedThreads / 2; w; w >>= 1) {
-        if ((int)threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) sums[blockIdx.x] = sh[0];
-}
-
-// Total of the block sums in a fixed order (one warp: lane l sums entries
-// l, l + 32, ... in order, then a fixed shuffle tree), so every call gets the
-// same bits.
-__device__ __forceinline__ double ordered_total(const double *__restrict__ sums, int nsums) {
-    double t = 0.0;
-    for (int i = threadIdx.x & 31; i < nsums; i += 32) t += sums[i];
-#pragma unroll
-    for (int off = 16; off; off >>= 1) t += __shfl_xor_sync(0xffffffffu, t, off);
-    return t;
-}
-
-__global__ void k_total(const double *__restrict__ sums, int nsums, double *__restrict__ total) {
-    const double t = ordered_total(sums, nsums);
-    if (threadIdx.x == 0) *total = t;
-}
-
-__global__ void k_normalise(double *__restrict__ p, uint64_t len, const double *__restrict__ total) {
-    const double t = *total;
-    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < len; i += stride)
-        p[i] = p[i] / t;
-}
-
-// v[0] /= total (the same ordered total as the normalisation uses).
-__global__ void k_div_total(double *v, const double *__restrict__ sums, int nsums) {
-    const double t = ordered_total(sums, nsums);
-    if (threadIdx.x == 0) v[0] = v[0] / t;
-}
-
-// argmax: (value, lowest index) per block, then one block over the partials.
+// The larger value, the lower index among equals.  The values are sums of
+// squares or the -1 of "none" (no NaN): their bit patterns compare like
+// integers, without the FP64 pipe.
 __device__ __forceinline__ void better(double &v, uint64_t &i, double v2, uint64_t i2) {
-    if (v2 > v || (v2 == v && i2 < i)) {
+    const long long a = __double_as_longlong(v), b = __double_as_longlong(v2);
+    if (b > a || (b == a && i2 < i)) {
         v = v2;
         i = i2;
     }
+}
+
+// Whether an entry (a sum of squares, or a NaN, which never wins) reaches the
+// best so far.
+__device__ __forceinline__ bool may_beat(double v, double best) {
+    const long long b = __double_as_longlong(v);
+    return b >= __double_as_longlong(best) && b <= 0x7ff0000000000000ll;
 }
 
 // Output index of the entry at position i of a marginal ordered as p says.
@@ -285,85 +167,468 @@ __device__ __forceinline__ uint64_t output_index(uint64_t i, const OutPerm &p) {
     return r;
 }
 
-__global__ void __launch_bounds__(kRedThreads)
-k_argmax(const double *__restrict__ x, const uint64_t *__restrict__ xi, uint64_t len,
-         double *__restrict__ ov, uint64_t *__restrict__ oi, const OutPerm perm) {
-    __shared__ double sv_[kRedThreads];
-    __shared__ uint64_t si[kRedThreads];
-    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-    double v = -1.0;
-    uint64_t idx = ~UINT64_C(0);
-    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < len; i += stride) {
-        const double xv = x[i];
-        // the output index (for ties: the lowest wins) only for a candidate
-        if (xv >= v) better(v, idx, xv, xi ? xi[i] : output_index(i, perm));
-    }
-    sv_[threadIdx.x] = v;
-    si[threadIdx.x] = idx;
-    __syncthreads();
-    for (int w = kRedThreads / 2; w; w >>= 1) {
-        if ((int)threadIdx.x < w) {
-            double v2 = sv_[threadIdx.x + w];
-            uint64_t i2 = si[threadIdx.x + w];
-            double v1 = sv_[threadIdx.x];
-            uint64_t i1 = si[threadIdx.x];
-            better(v1, i1, v2, i2);
-            sv_[threadIdx.x] = v1;
-            si[threadIdx.x] = i1;
+// Sum and (with ARG) largest entry of a thread block's outcomes, by a fixed
+// tree (lanes, then warps); the results are in thread 0.
+template <bool ARG>
+__device__ __forceinline__ void block_reduce(double &sum, double &v, uint64_t &i) {
+    constexpr int kWarps = kRedThreads / 32;
+    __shared__ double s_sum[kWarps], s_v[kWarps];
+    __shared__ uint64_t s_i[kWarps];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    auto lanes = [&](int from) {
+        for (int w = from; w; w >>= 1) {
+            sum += __shfl_down_sync(0xffffffffu, sum, w);
+            if (ARG) {
+                const double v2 = __shfl_down_sync(0xffffffffu, v, w);
+                const uint64_t i2 = __shfl_down_sync(0xffffffffu, (unsigned long long)i, w);
+                better(v, i, v2, i2);
+            }
         }
-        __syncthreads();
+    };
+    lanes(16);
+    __syncthreads();  // earlier use of the arrays is over
+    if (lane == 0) {
+        s_sum[warp] = sum;
+        s_v[warp] = v;
+        s_i[warp] = i;
+    }
+    __syncthreads();
+    if (warp == 0) {
+        sum = lane < kWarps ? s_sum[lane] : 0.0;
+        v = lane < kWarps ? s_v[lane] : -1.0;
+        i = lane < kWarps ? s_i[lane] : ~UINT64_C(0);
+        lanes(kWarps / 2);
+    }
+}
+
+// Leave this block's sum and largest entry; the last block to arrive combines
+// all of them in block order into the result.
+template <bool ARG>
+__device__ __forceinline__ void finish_stats(double sum, double v, uint64_t i, const Stats &st) {
+    __shared__ bool s_last;
+    block_reduce<ARG>(sum, v, i);
+    if (gridDim.x == 1) {
+        if (threadIdx.x == 0) *st.res = ReadResult{sum, 1.0 / sum, ARG ? v / sum : 0.0, i};
+        return;
     }
     if (threadIdx.x == 0) {
-        ov[blockIdx.x] = sv_[0];
-        oi[blockIdx.x] = si[0];
+        st.sum[blockIdx.x] = sum;
+        if (ARG) {
+            st.best[blockIdx.x] = v;
+            st.idx[blockIdx.x] = i;
+        }
+        __threadfence();
+        s_last = atomicAdd(st.done, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    double t = 0.0, bv = -1.0;
+    uint64_t bi = ~UINT64_C(0);
+    for (unsigned b = threadIdx.x; b < gridDim.x; b += kRedThreads) {
+        t += __ldcg(st.sum + b);
+        if (ARG) better(bv, bi, __ldcg(st.best + b), __ldcg(reinterpret_cast<const unsigned long long *>(st.idx) + b));
+    }
+    block_reduce<ARG>(t, bv, bi);
+    if (threadIdx.x == 0) {
+        *st.res = ReadResult{t, 1.0 / t, ARG ? bv / t : 0.0, bi};
+        *st.done = 0;
     }
 }
 
-// CDF, step 1: one thread per block of 1024 outcomes.
-__global__ void k_cdf_blocks(const double *__restrict__ p, uint64_t len, double *__restrict__ cdf,
-                             double *__restrict__ btot) {
-    const uint64_t b = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const uint64_t b0 = b * 1024;
-    if (b0 >= len) return;
-    const uint64_t b1 = b0 + 1024 < len ? b0 + 1024 : len;
+// What a marginal kernel does with its sums: keep them as partials of the
+// slices (PART), write the marginal and total it (SUM), or only find its
+// total and largest entry (ARG).
+enum { MARG_PART = 0, MARG_SUM = 1, MARG_ARG = 2 };
+
+// Layout M: consecutive threads take consecutive physical-order outcomes.
+// PB = 1 (complex64 with physical bit 0 an outcome bit): the two outcomes that
+// differ in it, whose amplitudes one 16-byte load covers.  With fewer outcomes than
+// a block has threads, the block's slices of one outcome are added here, so
+// that a marginal of a few qubits leaves a thousand partials per outcome
+// instead of up to 2^18.  HBM bounds it: 512 MiB in 86 us (0.93 of the
+// measured rate); QPE n = 28's argmax, 2 GiB, 376 us against 470 us for the
+// marginal, its block sums and its argmax as kernels of their own.
+template <typename R, int PB, int MODE>
+__global__ void __launch_bounds__(kRedThreads, kRedBlocks)
+k_marg_m(const R *__restrict__ s, MargArgs a, double *__restrict__ partial, const Stats st, const OutPerm perm) {
+    using V = typename std::conditional<PB == 1, float4, typename ProbAcc<R>::V>::type;
+    __shared__ double sh[MODE == MARG_PART ? 2 * kRedThreads : 1];
+    const uint64_t outcomes = UINT64_C(1) << a.m;
+    const uint64_t per = outcomes >> PB;  // threads per slice
+    const uint64_t items = per << a.groups_log2;
+    const V *sv_ = reinterpret_cast<const V *>(s);
+    double tot = 0.0, best = -1.0;
+    uint64_t bidx = ~UINT64_C(0);
+    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+    const uint64_t tid0 = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    // the thread's outcome as physical bits; the outcome `stride` further on
+    // is an addition on those bits alone
+    uint64_t xm = pdep_mask((tid0 & (per - 1)) << PB, a.mask);
+    const uint64_t step = MODE == MARG_PART ? 0 : pdep_mask((stride & (per - 1)) << PB, a.mask);
+    for (uint64_t tid = tid0;; tid += stride, xm = ((xm | ~a.mask) + step) & a.mask) {
+        const bool in = tid < items;
+        if (MODE != MARG_PART && !in) break;
+        const uint64_t mp = (tid & (per - 1)) << PB;
+        const uint64_t g = tid >> (a.m - PB);
+        uint64_t ml = mp;
+        if (MODE != MARG_ARG && !a.in_order) {
+            ml = 0;
+            for (int k = PB; k < a.m; k++) ml |= ((mp >> k) & 1) << a.out_bit[k];
+        }
+        const uint64_t ml1 = PB ? ml | (UINT64_C(1) << a.out_bit[0]) : ml;
+        uint64_t xr = pdep_mask(g * a.per_group, a.rest);
+        ProbAcc<R> acc0, acc1;
+        double p0 = 0.0, p1 = 0.0;
+        auto flush = [&](uint64_t done) {
+            if (done & (a.flush - 1)) return;
+            if (a.flush == a.per_group) {  // one sum: nothing to add it to
+                p0 = acc0.value();
+                if (PB) p1 = acc1.value();
+                return;
+            }
+            p0 += acc0.value();
+            acc0 = ProbAcc<R>();
+            if (PB) {
+                p1 += acc1.value();
+                acc1 = ProbAcc<R>();
+            }
+        };
+        uint64_t i = in ? 0 : a.per_group;
+        // kLoadBatch loads in flight per thread, then accumulated in order
+        for (; i + kLoadBatch <= a.per_group; i += kLoadBatch) {
+            V v[kLoadBatch];
+#pragma unroll
+            for (int k = 0; k < kLoadBatch; k++) {
+                v[k] = sv_[(xm | xr) >> PB];
+                xr = ((xr | ~a.rest) + 1) & a.rest;
+            }
+            if (a.flush >= kLoadBatch) {
+#pragma unroll
+                for (int k = 0; k < kLoadBatch; k++) add_vec(acc0, acc1, v[k]);
+                flush(i + kLoadBatch);
+            } else {
+#pragma unroll
+                for (int k = 0; k < kLoadBatch; k++) {
+                    add_vec(acc0, acc1, v[k]);
+                    flush(k + 1);
+                }
+            }
+        }
+        for (; i < a.per_group; i++) {
+            const V v = sv_[(xm | xr) >> PB];
+            add_vec(acc0, acc1, v);
+            flush(i + 1);
+            xr = ((xr | ~a.rest) + 1) & a.rest;
+        }
+        if (MODE == MARG_PART) {
+            uint64_t row = g;
+            if (per < kRedThreads) {  // add the block's slices of each outcome
+                sh[threadIdx.x] = p0;
+                if (PB) sh[kRedThreads + threadIdx.x] = p1;
+                __syncthreads();
+                for (unsigned w = kRedThreads / 2; w >= per; w >>= 1) {
+                    if (threadIdx.x < w) {
+                        sh[threadIdx.x] += sh[threadIdx.x + w];
+                        if (PB) sh[kRedThreads + threadIdx.x] += sh[kRedThreads + threadIdx.x + w];
+                    }
+                    __syncthreads();
+                }
+                if (threadIdx.x >= per) return;
+                p0 = sh[threadIdx.x];
+                p1 = sh[(PB ? kRedThreads : 0) + threadIdx.x];
+                row = blockIdx.x;
+            } else if (!in) {
+                return;
+            }
+            partial[row * outcomes + ml] = p0;
+            if (PB) partial[row * outcomes + ml1] = p1;
+            return;  // one item per thread
+        }
+        if (MODE == MARG_SUM) {
+            partial[ml] = p0;
+            if (PB) partial[ml1] = p1;
+        }
+        tot += PB ? p0 + p1 : p0;
+        if (MODE == MARG_ARG) {
+            if (may_beat(p0, best)) better(best, bidx, p0, output_index(mp, perm));
+            if (PB && may_beat(p1, best)) better(best, bidx, p1, output_index(mp | 1, perm));
+        }
+    }
+    if constexpr (MODE != MARG_PART) finish_stats<MODE == MARG_ARG>(tot, best, bidx, st);
+}
+
+// Layout R: the lowest physical bits are summed over; one warp per
+// (group, outcome), lanes take the five lowest rest bits.
+template <typename R, int MODE>
+__global__ void __launch_bounds__(kRedThreads, kRedBlocks)
+k_marg_r(const R *__restrict__ s, MargArgs a, double *__restrict__ partial, const Stats st, const OutPerm perm) {
+    const uint64_t outcomes = UINT64_C(1) << a.m;
+    const int lane = threadIdx.x & 31;
+    const uint64_t items = outcomes << a.groups_log2;
+    double tot = 0.0, best = -1.0;
+    uint64_t bidx = ~UINT64_C(0);
+    for (uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; warp < items;
+         warp += ((uint64_t)gridDim.x * blockDim.x) >> 5) {
+        const uint64_t mp = warp & (outcomes - 1);
+        const uint64_t g = warp >> a.m;
+        uint64_t xm = 0, ml = 0;
+        for (int k = 0; k < a.m; k++) {
+            if ((mp >> k) & 1) {
+                xm |= UINT64_C(1) << a.spos[k];
+                ml |= UINT64_C(1) << a.out_bit[k];
+            }
+        }
+        const uint64_t lane_bits = a.rest & ~a.upper;
+        const uint64_t xl = pdep_mask((uint64_t)lane, lane_bits);
+        uint64_t xo = pdep_mask(g * a.per_group, a.upper);
+        ProbAcc<R> pa;
+        double acc = 0.0;
+        auto flush = [&](uint64_t done) {
+            if (done & (a.flush - 1)) return;
+            acc += pa.value();
+            pa = ProbAcc<R>();
+        };
+        uint64_t i = 0;
+        for (; i + kLoadBatch <= a.per_group; i += kLoadBatch) {
+            typename ProbAcc<R>::V v[kLoadBatch];
+#pragma unroll
+            for (int k = 0; k < kLoadBatch; k++) {
+                v[k] = ProbAcc<R>::load(s, xm | xo | xl);
+                xo = ((xo | ~a.upper) + 1) & a.upper;
+            }
+            if (a.flush >= kLoadBatch) {
+#pragma unroll
+                for (int k = 0; k < kLoadBatch; k++) pa.add(v[k]);
+                flush(i + kLoadBatch);
+            } else {
+#pragma unroll
+                for (int k = 0; k < kLoadBatch; k++) {
+                    pa.add(v[k]);
+                    flush(k + 1);
+                }
+            }
+        }
+        for (; i < a.per_group; i++) {
+            pa.add(s, xm | xo | xl);
+            flush(i + 1);
+            xo = ((xo | ~a.upper) + 1) & a.upper;
+        }
+#pragma unroll
+        for (int off = 16; off; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
+        if (lane == 0) {
+            if (MODE != MARG_ARG) partial[g * outcomes + ml] = acc;
+            if (MODE != MARG_PART) tot += acc;
+            if (MODE == MARG_ARG && may_beat(acc, best)) better(best, bidx, acc, output_index(mp, perm));
+        }
+    }
+    if constexpr (MODE != MARG_PART) finish_stats<MODE == MARG_ARG>(tot, best, bidx, st);
+}
+
+// x / t for many x: r = 1 / t correctly rounded, and one correction of
+// x * r by its exact remainder gives the correctly rounded quotient (P.
+// Markstein, IBM J. Res. Dev. 34, 1990) in three FP64 operations instead of a
+// division's dozens; outside the range where the remainder is exact, divide.
+__device__ __forceinline__ double divide(double x, double t, double r, bool plain) {
+    // (x >= 0: compared as integers, off the FP64 pipe)
+    if (plain || __double_as_longlong(x) < __double_as_longlong(1e-280)) return x / t;
+    const double q = x * r;
+    return fma(fma(-q, t, x), r, q);
+}
+__device__ __forceinline__ bool divide_plain(double t) { return !(t > 1e-200 && t < 1e200); }
+
+// The sum of rows first, first + step, ... of outcome m, eight at a time (an
+// FP64 addition takes about 90 cycles).
+__device__ __forceinline__ double sum_rows(const double *__restrict__ partial, uint64_t outcomes, uint64_t m,
+                                           int first, int rows, int step) {
+    double part[8] = {};
+    int g = first;
+    for (; g + 7 * step < rows; g += 8 * step) {
+        double v[8];
+#pragma unroll
+        for (int k = 0; k < 8; k++) v[k] = partial[(uint64_t)(g + k * step) * outcomes + m];
+#pragma unroll
+        for (int k = 0; k < 8; k++) part[k] += v[k];
+    }
+    for (; g < rows; g += step) part[0] += partial[(uint64_t)g * outcomes + m];
+    return ((part[0] + part[1]) + (part[2] + part[3])) + ((part[4] + part[5]) + (part[6] + part[7]));
+}
+
+// Thread t of a block holds outcome t % to and one of the block's 256 / to
+// shares of the rows; the shares are added in a fixed tree, the sum of outcome
+// o in thread o.
+__device__ __forceinline__ double block_rows(const double *__restrict__ partial, uint64_t outcomes, uint64_t m0,
+                                             int first, int rows, int step, int to) {
+    __shared__ double sh[kRedThreads];
+    const int o = threadIdx.x % to, sl = threadIdx.x / to, ns = kRedThreads / to;
+    sh[threadIdx.x] = sum_rows(partial, outcomes, m0 + o, first + sl * step, rows, ns * step);
+    __syncthreads();
+    for (int w = kRedThreads / 2; w >= to; w >>= 1) {
+        if ((int)threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
+        __syncthreads();
+    }
+    return sh[threadIdx.x];
+}
+
+// kFoldRows rows from many: row y of the result adds rows y, y + kFoldRows, ...
+// (three qubits of n = 26, 1024 rows: 4 us and 5 us for the last sums; one
+// thread per outcome took 267 us for its 2048 rows).
+constexpr int kFoldRows = 32;
+__global__ void __launch_bounds__(kRedThreads)
+k_fold_rows(const double *__restrict__ partial, uint64_t outcomes, int rows, int to, double *__restrict__ out) {
+    const uint64_t m0 = (uint64_t)blockIdx.x * to;
+    const double acc = block_rows(partial, outcomes, m0, blockIdx.y, rows, gridDim.y, to);
+    if ((int)threadIdx.x < to) out[blockIdx.y * outcomes + m0 + threadIdx.x] = acc;
+}
+
+// p[m] = the sum of its partials; then as MODE says.  With `norm` and one
+// block the marginal is divided by its total here.
+template <int MODE>
+__global__ void __launch_bounds__(kRedThreads)
+k_sum_groups(const double *__restrict__ partial, uint64_t outcomes, int rows, int to, double *__restrict__ out,
+             const Stats st, const OutPerm perm, bool norm) {
+    const uint64_t m0 = (uint64_t)blockIdx.x * to, m = m0 + threadIdx.x;
+    const bool mine = (int)threadIdx.x < to;
+    double acc = block_rows(partial, outcomes, m0, 0, rows, 1, to);
+    if (!mine) acc = 0.0;
+    if (mine && MODE == MARG_SUM && !(norm && gridDim.x == 1)) out[m] = acc;
+    const bool cand = mine && may_beat(acc, -1.0);
+    finish_stats<MODE == MARG_ARG>(acc, cand ? acc : -1.0, cand ? output_index(m, perm) : ~UINT64_C(0), st);
+    if (MODE == MARG_SUM && norm && gridDim.x == 1) {
+        __syncthreads();
+        if (mine) out[m] = divide(acc, st.res->total, st.res->recip, divide_plain(st.res->total));
+    }
+}
+
+__global__ void __launch_bounds__(kRedThreads)
+k_normalise(double *__restrict__ p, uint64_t len, const ReadResult *__restrict__ res) {
+    const double t = res->total, r = res->recip;
+    const bool plain = divide_plain(t);
+    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+    double2 *p2 = reinterpret_cast<double2 *>(p);
+    const bool pairs = (reinterpret_cast<uintptr_t>(p) & 15) == 0;
+    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < len / 2; i += stride) {
+        double2 v = pairs ? p2[i] : make_double2(p[2 * i], p[2 * i + 1]);
+        v.x = divide(v.x, t, r, plain);
+        v.y = divide(v.y, t, r, plain);
+        if (pairs) p2[i] = v;
+        else {
+            p[2 * i] = v.x;
+            p[2 * i + 1] = v.y;
+        }
+    }
+}
+
+// CDF, step 1: the running sums of each block of 1024 outcomes, in index
+// order: one lane per block, 32 blocks per warp.  The warp loads 32 outcomes
+// of each of its blocks at a time (whole 256-byte rows, the next ones while it
+// adds), and each lane keeps its running sum at every 32nd outcome (chk)
+// and at the end (btot).  One addition after the other bounds it: 70 us for
+// 2^20 outcomes; reading them from each lane's own row and writing the whole
+// CDF took 160 us.
+constexpr int kCdfBlock = 1024, kCdfStep = 32;
+__global__ void __launch_bounds__(32)
+k_cdf_blocks(const double *__restrict__ p, uint64_t len, double *__restrict__ chk, double *__restrict__ btot) {
+    __shared__ double sh[32][33];
+    const int lane = threadIdx.x;
+    const uint64_t b0 = (uint64_t)blockIdx.x * 32;
+    double nxt[32];
+    auto load = [&](int c) {
+#pragma unroll
+        for (int k = 0; k < 32; k++) {
+            const uint64_t i = (b0 + k) * kCdfBlock + c * kCdfStep + lane;
+            nxt[k] = i < len ? p[i] : 0.0;
+        }
+    };
+    load(0);
     double run = 0.0;
-    for (uint64_t i = b0; i < b1; i++) {
-        run += p[i];
-        cdf[i] = run;
+    const uint64_t b = b0 + lane;
+    const bool mine = b * kCdfBlock < len;
+    for (int c = 0; c < kCdfBlock / kCdfStep; c++) {
+#pragma unroll
+        for (int k = 0; k < 32; k++) sh[k][lane] = nxt[k];
+        __syncwarp();
+        if (c + 1 < kCdfBlock / kCdfStep) load(c + 1);
+        if (mine) chk[b * (kCdfBlock / kCdfStep) + c] = run;
+        double x[32];
+#pragma unroll
+        for (int k = 0; k < 32; k++) x[k] = sh[lane][k];
+#pragma unroll
+        for (int k = 0; k < 32; k++) run += x[k];  // outcomes beyond len are 0
+        __syncwarp();
     }
-    btot[b] = run;
+    if (mine) btot[b] = run;
 }
 
-// CDF, step 2: exclusive running total over blocks, in block order.
-__global__ void k_cdf_scan(double *__restrict__ btot, uint64_t nb) {
-    double before = 0.0;
-    for (uint64_t b = 0; b < nb; b++) {
-        double t = btot[b];
-        btot[b] = before;
-        before += t;
+// CDF, step 2: before[b] = running total of the blocks before b, in block
+// order; before[nb] = C_last.  One addition after the other (about 90 cycles
+// each: 48 us for 1024 blocks, 107 us when each waited for its load too); the
+// loads and stores go through shared memory, 1024 blocks at a time.
+__global__ void __launch_bounds__(kRedThreads)
+k_cdf_scan(const double *__restrict__ btot, uint64_t nb, double *__restrict__ before) {
+    __shared__ double in[1024], out[1024];
+    double run = 0.0;
+    for (uint64_t c = 0; c < nb; c += 1024) {
+        const int m = (int)(nb - c < 1024 ? nb - c : 1024);
+        for (int i = threadIdx.x; i < 1024; i += kRedThreads) in[i] = i < m ? btot[c + i] : 0.0;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            for (int i = 0; i < m; i += 16) {
+                double x[16];
+#pragma unroll
+                for (int k = 0; k < 16; k++) x[k] = in[i + k];  // zeros beyond m
+#pragma unroll
+                for (int k = 0; k < 16; k++) {
+                    out[i + k] = run;
+                    run += x[k];
+                }
+            }
+        }
+        __syncthreads();
+        for (int i = threadIdx.x; i < m; i += kRedThreads) before[c + i] = out[i];
+        __syncthreads();
     }
+    if (threadIdx.x == 0) before[nb] = run;
 }
 
-// CDF, step 3: C_i = (total before the block) + (in-block running sum).
-__global__ void k_cdf_add(double *__restrict__ cdf, uint64_t len, const double *__restrict__ before) {
-    const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < len) cdf[i] = before[i / 1024] + cdf[i];
-}
-
-__global__ void k_sample(const double *__restrict__ cdf, uint64_t len, const double *__restrict__ u,
-                         uint64_t shots, uint64_t *__restrict__ out) {
+// CDF, step 3: the smallest i with C_i > u * C_last, where C_i = (total before
+// the block) + (running sum in the block): the block by its end, the step of
+// 32 in it by the kept sums, then the outcomes of the step in order.  The CDF
+// does not decrease, so this is what a search over all of it gives.
+__global__ void k_sample(const double *__restrict__ p, uint64_t len, const double *__restrict__ before,
+                         const double *__restrict__ chk, const double *__restrict__ u, uint64_t shots,
+                         uint64_t *__restrict__ out) {
     const uint64_t s = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= shots) return;
-    const double target = u[s] * cdf[len - 1];
-    uint64_t lo = 0, hi = len - 1;  // answer in [lo, hi]
+    const uint64_t nb = (len + kCdfBlock - 1) / kCdfBlock;
+    const double target = u[s] * before[nb];
+    uint64_t lo = 0, hi = nb - 1;
     while (lo < hi) {
-        uint64_t mid = lo + (hi - lo) / 2;
-        if (cdf[mid] > target)
-            hi = mid;
-        else
-            lo = mid + 1;
+        const uint64_t mid = lo + (hi - lo) / 2;
+        if (before[mid + 1] > target) hi = mid;
+        else lo = mid + 1;
     }
-    out[s] = lo;
+    const double bb = before[lo];
+    const double *ck = chk + lo * (kCdfBlock / kCdfStep);
+    // the first step whose end exceeds the target (the last one if none of the
+    // kept sums does)
+    const uint64_t left = len - lo * kCdfBlock;
+    const int steps = left >= (uint64_t)kCdfBlock ? kCdfBlock / kCdfStep : (int)((left + kCdfStep - 1) / kCdfStep);
+    int a = 0, z = steps - 1;
+    while (a < z) {
+        const int mid = (a + z) / 2;
+        if (bb + ck[mid + 1] > target) z = mid;
+        else a = mid + 1;
+    }
+    const uint64_t i0 = lo * kCdfBlock + (uint64_t)a * kCdfStep;
+    double run = ck[a];
+    uint64_t i = i0;
+    const uint64_t i1 = i0 + kCdfStep < len ? i0 + kCdfStep : len;
+    for (; i < i1; i++) {
+        run += p[i];
+        if (bb + run > target) break;
+    }
+    out[s] = i < len ? i : len - 1;
 }
 
 unsigned blocks_for(uint64_t work, int threads) {
@@ -409,165 +674,178 @@ sv_status ensure_probs(sv_state *h, size_t bytes) {
     return SV_OK;
 }
 
-// pos[j]: physical bit of output bit j.
-sv_status marginal_device(sv_state *h, const int *pos, int m, double *dev_out, bool normalise,
-                          const double **sums_out, int *nsums_out, OutPerm *perm_out) {
+namespace {
+
+template <int MODE>
+void launch_marginal(sv_state *h, const MargArgs &a, bool layout_r, bool pairs, unsigned grid, double *partial, const Stats &st,
+                     const OutPerm &perm) {
+    if (h->dt == SV_C128) {
+        const double *s = reinterpret_cast<const double *>(h->amps);
+        if (layout_r)
+            k_marg_r<double, MODE><<<grid, kRedThreads, 0, h->stream>>>(s, a, partial, st, perm);
+        else
+            k_marg_m<double, 0, MODE><<<grid, kRedThreads, 0, h->stream>>>(s, a, partial, st, perm);
+    } else {
+        const float *s = reinterpret_cast<const float *>(h->amps);
+        if (layout_r)
+            k_marg_r<float, MODE><<<grid, kRedThreads, 0, h->stream>>>(s, a, partial, st, perm);
+        else if (pairs)
+            k_marg_m<float, 1, MODE><<<grid, kRedThreads, 0, h->stream>>>(s, a, partial, st, perm);
+        else
+            k_marg_m<float, 0, MODE><<<grid, kRedThreads, 0, h->stream>>>(s, a, partial, st, perm);
+    }
+}
+
+// pos[j]: physical bit of output bit j.  MODE MARG_SUM: the marginal and its
+// total, in dev_out; MARG_ARG: its total and largest entry only (dev_out may
+// be NULL).  *divided: the marginal was divided by its total already.
+template <int MODE>
+sv_status marginal(sv_state *h, const int *pos, int m, double *dev_out, bool norm, bool *divided) {
     SV_TRY(materialize(h));
     const int n = h->n;
     MargArgs a{};
     a.n = n;
     a.m = m;
+    OutPerm perm{};
     // outcome bits sorted by physical position
     int order[34];
     for (int j = 0; j < m; j++) order[j] = j;
     std::sort(order, order + m, [&](int x, int y) { return pos[x] < pos[y]; });
     for (int k = 0; k < m; k++) {
         a.spos[k] = pos[order[k]];
-        a.out_bit[k] = perm_out ? k : order[k];
+        // the argmax keeps partials in physical order (coalesced whatever the
+        // qubit map) and maps only its candidates
+        a.out_bit[k] = MODE == MARG_ARG ? k : order[k];
         a.mask |= UINT64_C(1) << pos[order[k]];
     }
-    if (perm_out) {
-        perm_out->m = m;
-        for (int k = 0; k < m; k++) perm_out->bit[k] = (int8_t)order[k];
+    a.in_order = 1;
+    for (int k = 0; k < m; k++) a.in_order &= a.out_bit[k] == k;
+    if (MODE == MARG_ARG) {
+        perm.m = m;
+        for (int k = 0; k < m; k++) perm.bit[k] = (int8_t)order[k];
     }
     const uint64_t all = (n == 64) ? ~UINT64_C(0) : ((UINT64_C(1) << n) - 1);
     a.rest = all & ~a.mask;
     const int rbits = n - m;
     const uint64_t outcomes = UINT64_C(1) << m;
-    const bool layout_r = (a.mask & 1) == 0 && rbits >= 5;
-    const int target_log2 = 19;  // ~5e5 threads (layout M) or lanes (layout R)
+    const bool bit0 = (a.mask & 1) != 0;
+    const bool layout_r = !bit0 && rbits >= 5;
+    // complex64 with physical bit 0 an outcome bit: two outcomes per thread
+    const bool pairs = bit0 && h->dt == SV_C64;
+    // slices per outcome: enough threads (layout M) or lanes (layout R) for the
+    // device, but at least 16 (8) vectors per thread, so that a marginal with
+    // many outcomes, or a small state's, is one launch
+    const int target_log2 = 18;
     int gl;
     if (layout_r) {
         uint64_t up = a.rest;
         for (int i = 0; i < 5; i++) up &= up - 1;  // drop the 5 lowest rest bits
         a.upper = up;
         int ubits = rbits - 5;
-        gl = std::max(0, std::min(ubits, target_log2 - 5 - m));
+        gl = std::max(0, std::min(ubits - 3, target_log2 - 5 - m));
         a.per_group = UINT64_C(1) << (ubits - gl);
     } else {
-        gl = std::max(0, std::min(rbits, target_log2 - m));
+        gl = std::max(0, std::min(rbits - 4, target_log2 - m));
         a.per_group = UINT64_C(1) << (rbits - gl);
     }
     a.groups_log2 = gl;
-    const uint64_t groups = UINT64_C(1) << gl;
-
-    double *partial = dev_out;
-    size_t need = 0;
-    if (groups > 1) need += groups * outcomes * sizeof(double);
-    const int nsum_blocks = (int)std::min<uint64_t>(1024, blocks_for(outcomes, kRedThreads));
-    const size_t sums_off = (need + 255) & ~(size_t)255;
-    need = sums_off + (nsum_blocks + 1) * sizeof(double);
-    SV_TRY(ensure_scratch(h, need));
-    if (groups > 1) partial = reinterpret_cast<double *>(h->scratch);
-    double *sums = reinterpret_cast<double *>(reinterpret_cast<char *>(h->scratch) + sums_off);
-
-    // complex64 with physical bit 0 an outcome bit: two outcomes per thread
-    const bool pairs = !layout_r && h->dt == SV_C64 && m >= 1 && a.spos[0] == 0;
-    const uint64_t work = layout_r ? (outcomes << gl) * 32 : pairs ? ((outcomes >> 1) << gl) : (outcomes << gl);
-    const unsigned grid = blocks_for(work, kRedThreads);
-    if (h->dt == SV_C128) {
-        const double *s = reinterpret_cast<const double *>(h->amps);
-        if (layout_r)
-            k_marg_r<double><<<grid, kRedThreads, 0, h->stream>>>(s, a, partial);
-        else
-            k_marg_m<double><<<grid, kRedThreads, 0, h->stream>>>(s, a, partial);
-    } else {
-        const float *s = reinterpret_cast<const float *>(h->amps);
-        if (layout_r)
-            k_marg_r<float><<<grid, kRedThreads, 0, h->stream>>>(s, a, partial);
-        else if (pairs)
-            k_marg_m2<<<grid, kRedThreads, 0, h->stream>>>(s, a, partial);
-        else
-            k_marg_m<float><<<grid, kRedThreads, 0, h->stream>>>(s, a, partial);
-    }
-    SV_CUDA(cudaGetLastError());
-    note_launch();
-    if (groups > 1) {
-        k_sum_groups<<<blocks_for(outcomes, kRedThreads), kRedThreads, 0, h->stream>>>(
-            partial, outcomes, (int)groups, dev_out);
+    // FP32 pairs carry about 2^-48 of their sum's size per addition: short
+    // sums, added up in FP64, keep the marginal's error below 1e-15 on small
+    // and mid-sized states, where the conversions cost nothing (2^19 of them
+    // or one per amplitude, whichever is less)
+    const int short_log2 = layout_r ? std::max(0, rbits - 5 - std::max(0, 14 - m)) : std::max(0, rbits - std::max(0, 19 - m));
+    a.flush = std::min(a.per_group, UINT64_C(1) << short_log2);
+    const int pb = pairs ? 1 : 0;
+    const Stats st = stats_of(h);
+    const unsigned most = (unsigned)std::min(kMaxStatBlocks, h->sm_count * kRedBlocks);
+    const uint64_t threads = layout_r ? (outcomes << gl) * 32 : (outcomes >> pb) << gl;
+    const unsigned blocks = blocks_for(threads, kRedThreads);
+    const bool fold = !layout_r && (outcomes >> pb) < kRedThreads;  // the block adds its slices
+    *divided = false;
+    if (gl == 0) {  // every thread (warp) holds whole outcomes
+        const unsigned grid = std::min(blocks, most);
+        launch_marginal<MODE>(h, a, layout_r, pairs, grid, dev_out, st, perm);
         SV_CUDA(cudaGetLastError());
-    note_launch();
+        note_launch();
+        return SV_OK;
     }
-    k_block_sum<<<nsum_blocks, kRedThreads, 0, h->stream>>>(dev_out, outcomes, sums);
+    uint64_t rows = fold ? blocks : UINT64_C(1) << gl;
+    SV_TRY(ensure_scratch(h, (rows + kFoldRows) * outcomes * sizeof(double)));
+    double *partial = reinterpret_cast<double *>(h->scratch);
+    launch_marginal<MARG_PART>(h, a, layout_r, pairs, blocks, partial, st, perm);
     SV_CUDA(cudaGetLastError());
     note_launch();
-    if (sums_out) *sums_out = sums;
-    if (nsums_out) *nsums_out = nsum_blocks;
-    if (!normalise) return SV_OK;
-    double *total = sums + nsum_blocks;
-    k_total<<<1, 32, 0, h->stream>>>(sums, nsum_blocks, total);
+    if (rows > 4 * kFoldRows && outcomes * kFoldRows <= 8192) {
+        // many partials of few outcomes: one block would read them all
+        // (8 outcomes, 2048 rows: 18 us), so more blocks add most of them
+        double *folded = partial + rows * outcomes;
+        const int to = (int)std::min<uint64_t>(outcomes, 32);
+        k_fold_rows<<<dim3((unsigned)(outcomes / to), kFoldRows), kRedThreads, 0, h->stream>>>(
+            partial, outcomes, (int)rows, to, folded);
+        SV_CUDA(cudaGetLastError());
+        note_launch();
+        partial = folded;
+        rows = kFoldRows;
+    }
+    // outcomes per block: all its threads while that fills the device
+    const int to = (int)std::min<uint64_t>(outcomes, rows <= 16 || outcomes > 32768 ? 256 : 32);
+    const unsigned grid = (unsigned)(outcomes / to);
+    k_sum_groups<MODE><<<grid, kRedThreads, 0, h->stream>>>(partial, outcomes, (int)rows, to, dev_out, st, perm, norm);
     SV_CUDA(cudaGetLastError());
     note_launch();
-    k_normalise<<<std::min<unsigned>(blocks_for(outcomes, kRedThreads), 4096), kRedThreads, 0,
-                  h->stream>>>(dev_out, outcomes, total);
+    *divided = norm && grid == 1;
+    return SV_OK;
+}
+
+}  // namespace
+
+sv_status marginal_device(sv_state *h, const int *pos, int m, double *dev_out) {
+    bool divided;
+    SV_TRY(marginal<MARG_SUM>(h, pos, m, dev_out, true, &divided));
+    if (divided) return SV_OK;
+    const uint64_t outcomes = UINT64_C(1) << m;
+    const unsigned grid = std::min<unsigned>(blocks_for((outcomes + 1) / 2, kRedThreads), (unsigned)h->sm_count * 8);
+    k_normalise<<<grid, kRedThreads, 0, h->stream>>>(dev_out, outcomes, stats_of(h).res);
     SV_CUDA(cudaGetLastError());
     note_launch();
     return SV_OK;
 }
 
-sv_status argmax_device(sv_state *h, const double *dev_p, uint64_t len, uint64_t *host_idx,
-                        double *host_p, const double *sums, int nsums, const OutPerm *perm) {
-    OutPerm ident{};
-    const OutPerm pm = perm ? *perm : ident;
-    const int nb = (int)std::min<uint64_t>(1024, blocks_for(len, kRedThreads));
-    char *base = reinterpret_cast<char *>(h->small);
-    double *bv = reinterpret_cast<double *>(base);
-    uint64_t *bi = reinterpret_cast<uint64_t *>(base + 8192);
-    double *fv = reinterpret_cast<double *>(base + 16384);
-    uint64_t *fi = reinterpret_cast<uint64_t *>(base + 16384 + 64);
-    k_argmax<<<nb, kRedThreads, 0, h->stream>>>(dev_p, nullptr, len, bv, bi, pm);
-    SV_CUDA(cudaGetLastError());
-    note_launch();
-    k_argmax<<<1, kRedThreads, 0, h->stream>>>(bv, bi, (uint64_t)nb, fv, fi, ident);
-    SV_CUDA(cudaGetLastError());
-    note_launch();
-    if (sums) {  // unnormalised marginal: p = max / total, the total in the normalisation's order
-        k_div_total<<<1, 32, 0, h->stream>>>(fv, sums, nsums);
-        SV_CUDA(cudaGetLastError());
-        note_launch();
-    }
-    double v;
-    uint64_t i;
-    SV_CUDA(cudaMemcpyAsync(&v, fv, sizeof v, cudaMemcpyDeviceToHost, h->stream));
-    SV_CUDA(cudaMemcpyAsync(&i, fi, sizeof i, cudaMemcpyDeviceToHost, h->stream));
+sv_status argmax_device(sv_state *h, const int *pos, int m, uint64_t *host_idx, double *host_p) {
+    bool divided;
+    SV_TRY(marginal<MARG_ARG>(h, pos, m, nullptr, false, &divided));
+    ReadResult r;
+    SV_CUDA(cudaMemcpyAsync(&r, stats_of(h).res, sizeof r, cudaMemcpyDeviceToHost, h->stream));
     SV_TRY(finish_sync(h));
-    *host_idx = i;
-    if (host_p) *host_p = v;
+    *host_idx = r.idx;
+    if (host_p) *host_p = r.best;
     return SV_OK;
 }
 
 sv_status sample_device(sv_state *h, const double *dev_p, uint64_t len, const double *host_u,
                         size_t shots, uint64_t *host_out) {
-    const uint64_t nb = (len + 1023) / 1024;
-    size_t off_cdf = 0;
-    size_t off_bt = (len * sizeof(double) + 255) & ~(size_t)255;
-    size_t off_u = (off_bt + nb * sizeof(double) + 255) & ~(size_t)255;
-    size_t off_o = (off_u + shots * sizeof(double) + 255) & ~(size_t)255;
-    size_t need = off_o + shots * sizeof(uint64_t);
-    SV_TRY(ensure_scratch(h, need));
+    if (!shots) return finish_sync(h);
+    const uint64_t nb = (len + kCdfBlock - 1) / kCdfBlock;
+    const size_t off_bt = nb * (kCdfBlock / kCdfStep) * sizeof(double);
+    const size_t off_be = off_bt + nb * sizeof(double);
+    const size_t off_u = off_be + (nb + 1) * sizeof(double);
+    const size_t off_o = off_u + shots * sizeof(double);
+    SV_TRY(ensure_scratch(h, off_o + shots * sizeof(uint64_t)));
     char *base = reinterpret_cast<char *>(h->scratch);
-    double *cdf = reinterpret_cast<double *>(base + off_cdf);
+    double *chk = reinterpret_cast<double *>(base);
     double *bt = reinterpret_cast<double *>(base + off_bt);
+    double *before = reinterpret_cast<double *>(base + off_be);
     double *du = reinterpret_cast<double *>(base + off_u);
     uint64_t *dout = reinterpret_cast<uint64_t *>(base + off_o);
-    k_cdf_blocks<<<blocks_for(nb, 128), 128, 0, h->stream>>>(dev_p, len, cdf, bt);
+    k_cdf_blocks<<<blocks_for(nb, 32), 32, 0, h->stream>>>(dev_p, len, chk, bt);
     SV_CUDA(cudaGetLastError());
-    note_launch();
-    k_cdf_scan<<<1, 1, 0, h->stream>>>(bt, nb);
+    k_cdf_scan<<<1, kRedThreads, 0, h->stream>>>(bt, nb, before);
     SV_CUDA(cudaGetLastError());
-    note_launch();
-    k_cdf_add<<<blocks_for(len, kRedThreads), kRedThreads, 0, h->stream>>>(cdf, len, bt);
+    SV_CUDA(cudaMemcpyAsync(du, host_u, shots * sizeof(double), cudaMemcpyHostToDevice, h->stream));
+    k_sample<<<blocks_for(shots, 64), 64, 0, h->stream>>>(dev_p, len, before, chk, du, shots, dout);
     SV_CUDA(cudaGetLastError());
-    note_launch();
-    if (shots) {
-        SV_CUDA(cudaMemcpyAsync(du, host_u, shots * sizeof(double), cudaMemcpyHostToDevice,
-                                h->stream));
-        k_sample<<<blocks_for(shots, 128), 128, 0, h->stream>>>(cdf, len, du, shots, dout);
-        SV_CUDA(cudaGetLastError());
-    note_launch();
-        SV_CUDA(cudaMemcpyAsync(host_out, dout, shots * sizeof(uint64_t), cudaMemcpyDeviceToHost,
-                                h->stream));
-    }
+    note_launch(3);
+    SV_CUDA(cudaMemcpyAsync(host_out, dout, shots * sizeof(uint64_t), cudaMemcpyDeviceToHost, h->stream));
     return finish_sync(h);
 }
 
