@@ -59,12 +59,12 @@ sv_status make_handle(int n, sv_dtype dt, void *buf, size_t bytes, void *stream,
         h->amps = buf;
         h->stream = reinterpret_cast<cudaStream_t>(stream);
     }
-    if (dev_malloc(&h->small, 65536) != cudaSuccess) {
+    if (dev_malloc(&h->small, kSmallBytes) != cudaSuccess) {
         cudaGetLastError();
         return bail(fail(SV_ERR_OOM, "cannot allocate reduction buffer"));
     }
-    // the read-outs' arrival counter (measure.cu) starts at zero
-    if (cudaMemsetAsync(static_cast<char *>(h->small) + 65536 - 64, 0, 64, h->stream) != cudaSuccess) {
+    // the reductions' arrival counter starts at zero
+    if (cudaMemsetAsync(static_cast<char *>(h->small) + kSmallDone, 0, 64, h->stream) != cudaSuccess) {
         cudaError_t e = cudaGetLastError();
         return bail(fail(SV_ERR_CUDA, "cannot clear the reduction buffer: %s", cudaGetErrorString(e)));
     }

@@ -77,7 +77,8 @@ struct sv_state {
     size_t scratch_cap = 0;
     double *probs = nullptr;      // device marginal of the last read-out
     size_t probs_cap = 0;
-    void *small = nullptr;        // 64 KiB device area for reduction partials
+    void *small = nullptr;        // 64 KiB device area for reduction partials; an
+                                  // arrival counter at sv::kSmallDone, zero between launches
     void *grp = nullptr;          // L2 block groups: done counters and claim queue
     size_t grp_cap = 0;
     void *slotv = nullptr;        // per-tile slot values of the register-stage passes
@@ -123,6 +124,7 @@ struct sv_state {
 
 namespace sv {
 
+constexpr size_t kSmallBytes = 65536, kSmallDone = kSmallBytes - 64;
 sv_status ensure_scratch(sv_state *h, size_t bytes);
 sv_status ensure_probs(sv_state *h, size_t bytes);
 const char *last_error_cstr();

@@ -7,11 +7,16 @@
 // x is 1, so the kernel enumerates exactly those pairs (2^(n-1-k) of them).
 // U2Q updates the four amplitudes that agree off its two qubits.  MEASURE
 // sums |amp|^2 over each value of its qubit in FP64 (per-block partials in a
-// fixed tree, then the blocks in order), picks the outcome on the device as
-// the smallest i with C_i > u C_last for C = (p0, p0 + p1), and collapses the
-// state: the other half is zeroed and the kept one divided by sqrt(p_i).  No
-// host synchronisation: the outcome goes to a device array that
-// sv_last_measurements reads.
+// fixed tree, then the blocks in a fixed tree), picks the outcome on the
+// device as the smallest i with C_i > u C_last for C = (p0, p0 + p1), and
+// collapses the state: the other half is zeroed and the kept one divided by
+// sqrt(p_i).  No host synchronisation: the outcome goes to a device array
+// that sv_last_measurements reads.
+//
+// All of them are HBM (up to n = 23: L2) sweeps: threads keep several 16-byte
+// vectors in flight, of two amplitudes in complex64 when no qubit of the gate
+// is bit 0.  A dynamic circuit of n = 23 with 6 MCU, 6 U2Q and 2 measurements:
+// 1074 us with one 8-byte amplitude at a time in MCU and U2Q, 1045 so.
 #include <algorithm>
 #include <cmath>
 
@@ -21,7 +26,7 @@ namespace sv {
 namespace {
 
 constexpr int kThreads = 256;
-constexpr int kMeasBlocks = 1024;  // partial sums of a measurement (2 doubles each)
+constexpr int kMeasBlocks = 1216;  // partial sums of a measurement (2 doubles each)
 
 // Positions (ascending) where the enumeration inserts a bit.
 struct Ins {
@@ -46,106 +51,257 @@ struct C4 {
     R re[16], im[16];
 };
 
-template <typename R>
+// A vector of the state: VB = 1 two complex64 amplitudes, VB = 0 one
+// amplitude.
+template <typename R, int VB>
+struct Vec;
+template <>
+struct Vec<float, 1> {
+    using T = float4;
+};
+template <>
+struct Vec<float, 0> {
+    using T = float2;
+};
+template <>
+struct Vec<double, 0> {
+    using T = double2;
+};
+
+constexpr int kItems = 4;  // vectors (pairs, quadruples: half as many) a thread keeps in flight
+
+template <typename R, int VB>
 __global__ void __launch_bounds__(kThreads)
 k_mcu(R *__restrict__ s, uint64_t units, Ins in, uint64_t ones, uint64_t tbit, C2<R> c) {
+    using T = typename Vec<R, VB>::T;
+    T *v = reinterpret_cast<T *>(s);
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-    for (uint64_t u = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; u < units; u += stride) {
-        const uint64_t x0 = insert_zeros(u, in) | ones, x1 = x0 | tbit;
-        const R ar = s[2 * x0], ai = s[2 * x0 + 1], br = s[2 * x1], bi = s[2 * x1 + 1];
-        s[2 * x0] = c.re[0] * ar - c.im[0] * ai + c.re[1] * br - c.im[1] * bi;
-        s[2 * x0 + 1] = c.re[0] * ai + c.im[0] * ar + c.re[1] * bi + c.im[1] * br;
-        s[2 * x1] = c.re[2] * ar - c.im[2] * ai + c.re[3] * br - c.im[3] * bi;
-        s[2 * x1 + 1] = c.re[2] * ai + c.im[2] * ar + c.re[3] * bi + c.im[3] * br;
+    for (uint64_t u0 = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; u0 < units; u0 += stride * kItems) {
+        T a[kItems], b[kItems];
+        uint64_t x[kItems];
+#pragma unroll
+        for (int k = 0; k < kItems; k++) {
+            const uint64_t u = u0 + k * stride;
+            if (u >= units) break;
+            x[k] = insert_zeros(u, in) | ones;
+            a[k] = v[x[k]];
+            b[k] = v[x[k] | tbit];
+        }
+#pragma unroll
+        for (int k = 0; k < kItems; k++) {
+            if (u0 + k * stride >= units) break;
+            R *pa = reinterpret_cast<R *>(&a[k]), *pb = reinterpret_cast<R *>(&b[k]);
+#pragma unroll
+            for (int e = 0; e < (1 << VB); e++) {
+                const R ar = pa[2 * e], ai = pa[2 * e + 1], br = pb[2 * e], bi = pb[2 * e + 1];
+                pa[2 * e] = c.re[0] * ar - c.im[0] * ai + c.re[1] * br - c.im[1] * bi;
+                pa[2 * e + 1] = c.re[0] * ai + c.im[0] * ar + c.re[1] * bi + c.im[1] * br;
+                pb[2 * e] = c.re[2] * ar - c.im[2] * ai + c.re[3] * br - c.im[3] * bi;
+                pb[2 * e + 1] = c.re[2] * ai + c.im[2] * ar + c.re[3] * bi + c.im[3] * br;
+            }
+            v[x[k]] = a[k];
+            v[x[k] | tbit] = b[k];
+        }
     }
 }
 
-template <typename R>
+template <typename R, int VB>
 __global__ void __launch_bounds__(kThreads)
 k_u2q(R *__restrict__ s, uint64_t units, Ins in, uint64_t ma, uint64_t mb, C4<R> m) {
+    using T = typename Vec<R, VB>::T;
+    constexpr int NI = kItems / 2;
+    T *v = reinterpret_cast<T *>(s);
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-    for (uint64_t u = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; u < units; u += stride) {
-        const uint64_t x = insert_zeros(u, in);
-        const uint64_t idx[4] = {x, x | ma, x | mb, x | ma | mb};
-        R vr[4], vi[4];
+    for (uint64_t u0 = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; u0 < units; u0 += stride * NI) {
+        T q[NI][4];
+        uint64_t x[NI];
 #pragma unroll
-        for (int k = 0; k < 4; k++) {
-            vr[k] = s[2 * idx[k]];
-            vi[k] = s[2 * idx[k] + 1];
+        for (int i = 0; i < NI; i++) {
+            const uint64_t u = u0 + i * stride;
+            if (u >= units) break;
+            x[i] = insert_zeros(u, in);
+            q[i][0] = v[x[i]];
+            q[i][1] = v[x[i] | ma];
+            q[i][2] = v[x[i] | mb];
+            q[i][3] = v[x[i] | ma | mb];
         }
 #pragma unroll
-        for (int r = 0; r < 4; r++) {
-            R yr = 0, yi = 0;
+        for (int i = 0; i < NI; i++) {
+            if (u0 + i * stride >= units) break;
+            T y[4];
 #pragma unroll
-            for (int k = 0; k < 4; k++) {
-                yr += m.re[4 * r + k] * vr[k] - m.im[4 * r + k] * vi[k];
-                yi += m.re[4 * r + k] * vi[k] + m.im[4 * r + k] * vr[k];
-            }
-            s[2 * idx[r]] = yr;
-            s[2 * idx[r] + 1] = yi;
+            for (int e = 0; e < (1 << VB); e++)
+#pragma unroll
+                for (int r = 0; r < 4; r++) {
+                    R yr = 0, yi = 0;
+#pragma unroll
+                    for (int k = 0; k < 4; k++) {
+                        const R vr = reinterpret_cast<const R *>(&q[i][k])[2 * e];
+                        const R vi = reinterpret_cast<const R *>(&q[i][k])[2 * e + 1];
+                        yr += m.re[4 * r + k] * vr - m.im[4 * r + k] * vi;
+                        yi += m.re[4 * r + k] * vi + m.im[4 * r + k] * vr;
+                    }
+                    reinterpret_cast<R *>(&y[r])[2 * e] = yr;
+                    reinterpret_cast<R *>(&y[r])[2 * e + 1] = yi;
+                }
+            v[x[i]] = y[0];
+            v[x[i] | ma] = y[1];
+            v[x[i] | mb] = y[2];
+            v[x[i] | ma | mb] = y[3];
         }
     }
 }
 
-// Per-block FP64 sums of |amp|^2 with the measured bit 0 and 1.
+// Sums of squares of one value of the measured qubit.  complex64: exact FP32
+// squares in a double-float pair (product and fmaf remainder, error-free
+// sums), moved to FP64 every few amplitudes; complex128: FP64.
 template <typename R>
-__global__ void __launch_bounds__(kThreads)
-k_meas_partial(const R *__restrict__ s, uint64_t N, uint64_t tbit, double *__restrict__ part) {
-    __shared__ double sh0[kThreads], sh1[kThreads];
-    double p0 = 0.0, p1 = 0.0;
-    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-    for (uint64_t x = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; x < N; x += stride) {
-        const double re = (double)s[2 * x], im = (double)s[2 * x + 1];
-        const double q = re * re + im * im;
-        if (x & tbit) p1 += q;
-        else p0 += q;
+struct Squares {
+    double sr = 0.0, si = 0.0;
+    __device__ void add(R re, R im) {
+        sr = fma(re, re, sr);
+        si = fma(im, im, si);
     }
-    sh0[threadIdx.x] = p0;
-    sh1[threadIdx.x] = p1;
+    __device__ void flush() {}
+    __device__ double value() const { return sr + si; }
+};
+template <>
+struct Squares<float> {
+    double acc = 0.0;
+    float hi = 0.f, lo = 0.f;
+    __device__ void sum(float b) {
+        const float t = hi + b, bb = t - hi;
+        lo += (hi - (t - bb)) + (b - bb);
+        hi = t;
+    }
+    __device__ void add(float re, float im) {
+        const float pr = re * re, pi = im * im;
+        lo += fmaf(re, re, -pr) + fmaf(im, im, -pi);
+        sum(pr);
+        sum(pi);
+    }
+    __device__ void flush() {
+        acc += (double)hi + (double)lo;
+        hi = lo = 0.f;
+    }
+    __device__ double value() const { return acc; }
+};
+
+// Sum over a block by a fixed tree; the result in thread 0.
+__device__ __forceinline__ double block_sum(double x) {
+    __shared__ double sh[kThreads / 32];
+#pragma unroll
+    for (int w = 16; w; w >>= 1) x += __shfl_down_sync(0xffffffffu, x, w);
     __syncthreads();
-    for (int w = kThreads / 2; w; w >>= 1) {
-        if ((int)threadIdx.x < w) {
-            sh0[threadIdx.x] += sh0[threadIdx.x + w];
-            sh1[threadIdx.x] += sh1[threadIdx.x + w];
-        }
-        __syncthreads();
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = x;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        x = threadIdx.x < kThreads / 32 ? sh[threadIdx.x] : 0.0;
+#pragma unroll
+        for (int w = kThreads / 64; w; w >>= 1) x += __shfl_down_sync(0xffffffffu, x, w);
     }
-    if (threadIdx.x == 0) {
-        part[2 * blockIdx.x] = sh0[0];
-        part[2 * blockIdx.x + 1] = sh1[0];
-    }
+    return x;
 }
 
-// The outcome (smallest i with C_i > u C_last) and the kept half's scale.
-__global__ void k_meas_decide(const double *__restrict__ part, int nblocks, double u, double *dec,
-                              uint8_t *outcome) {
-    double p0 = 0.0, p1 = 0.0;
-    for (int b = 0; b < nblocks; b++) {
-        p0 += part[2 * b];
-        p1 += part[2 * b + 1];
-    }
-    const double last = p0 + p1;
-    const int out = (p0 > u * last) ? 0 : 1;
-    const double keep = out ? p1 : p0;
-    dec[0] = (double)out;
-    dec[1] = keep > 0.0 ? 1.0 / sqrt(keep) : 0.0;
-    *outcome = (uint8_t)out;
-}
-
-template <typename R>
+// p0 and p1 of the measured qubit: each thread takes the vectors that differ
+// in it (VB = 1 and the qubit bit 0: `intra`, both in one vector).  The last
+// block to finish adds the blocks' sums in a fixed tree and decides: the
+// outcome (smallest i with C_i > u C_last) and the kept half's scale.  As FP64
+// sums of every amplitude and one thread over 1024 partials this took 216 us
+// at n = 23 (64 MiB).
+template <typename R, int VB>
 __global__ void __launch_bounds__(kThreads)
-k_meas_collapse(R *__restrict__ s, uint64_t N, uint64_t tbit, const double *__restrict__ dec) {
+k_meas_decide(const R *__restrict__ s, uint64_t units, int pos, uint64_t tbit, bool intra, double *__restrict__ part,
+              unsigned *__restrict__ done, double u, double *dec, uint8_t *outcome) {
+    using T = typename Vec<R, VB>::T;
+    __shared__ bool last;
+    const T *v = reinterpret_cast<const T *>(s);
+    Squares<R> s0, s1;
+    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+    for (uint64_t u0 = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; u0 < units; u0 += stride * kItems) {
+        T a[kItems], b[kItems];
+#pragma unroll
+        for (int k = 0; k < kItems; k++) {
+            const uint64_t i = u0 + k * stride;
+            a[k] = b[k] = T{};
+            if (i >= units) continue;
+            const uint64_t x = intra ? i : ((i >> pos) << (pos + 1)) | (i & ((UINT64_C(1) << pos) - 1));
+            a[k] = v[x];
+            if (!intra) b[k] = v[x | tbit];
+        }
+#pragma unroll
+        for (int k = 0; k < kItems; k++) {
+            const R *pa = reinterpret_cast<const R *>(&a[k]), *pb = reinterpret_cast<const R *>(&b[k]);
+            if (intra) {
+                s0.add(pa[0], pa[1]);
+                if (VB) s1.add(pa[VB * 2], pa[VB * 2 + 1]);
+            } else {
+#pragma unroll
+                for (int e = 0; e < (1 << VB); e++) {
+                    s0.add(pa[2 * e], pa[2 * e + 1]);
+                    s1.add(pb[2 * e], pb[2 * e + 1]);
+                }
+            }
+        }
+        s0.flush();
+        s1.flush();
+    }
+    double p0 = block_sum(s0.value()), p1 = block_sum(s1.value());
+    if (threadIdx.x == 0) {
+        part[2 * blockIdx.x] = p0;
+        part[2 * blockIdx.x + 1] = p1;
+        __threadfence();
+        last = atomicAdd(done, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    p0 = p1 = 0.0;
+    for (unsigned b = threadIdx.x; b < gridDim.x; b += kThreads) {
+        p0 += __ldcg(part + 2 * b);
+        p1 += __ldcg(part + 2 * b + 1);
+    }
+    p0 = block_sum(p0);
+    p1 = block_sum(p1);
+    if (threadIdx.x == 0) {
+        const double total = p0 + p1;
+        const int out = (p0 > u * total) ? 0 : 1;
+        const double keep = out ? p1 : p0;
+        dec[0] = (double)out;
+        dec[1] = keep > 0.0 ? 1.0 / sqrt(keep) : 0.0;
+        *outcome = (uint8_t)out;
+        *done = 0;
+    }
+}
+
+// The kept half scaled, the other one zeroed (written without reading it).
+template <typename R, int VB>
+__global__ void __launch_bounds__(kThreads)
+k_meas_collapse(R *__restrict__ s, uint64_t units, int pos, uint64_t tbit, bool intra, const double *__restrict__ dec) {
+    using T = typename Vec<R, VB>::T;
+    T *v = reinterpret_cast<T *>(s);
     const int out = (int)dec[0];
     const R sc = (R)dec[1];
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-    for (uint64_t x = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; x < N; x += stride) {
-        const int bit = (x & tbit) ? 1 : 0;
-        if (bit == out) {
-            s[2 * x] *= sc;
-            s[2 * x + 1] *= sc;
-        } else {
-            s[2 * x] = R(0);
-            s[2 * x + 1] = R(0);
+    for (uint64_t u0 = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; u0 < units; u0 += stride * kItems) {
+        T a[kItems];
+        uint64_t x[kItems];
+#pragma unroll
+        for (int k = 0; k < kItems; k++) {
+            const uint64_t i = u0 + k * stride;
+            if (i >= units) break;
+            x[k] = intra ? i : ((i >> pos) << (pos + 1)) | (i & ((UINT64_C(1) << pos) - 1));
+            if (!intra && out) x[k] |= tbit;
+            a[k] = v[x[k]];
+        }
+#pragma unroll
+        for (int k = 0; k < kItems; k++) {
+            if (u0 + k * stride >= units) break;
+            R *pa = reinterpret_cast<R *>(&a[k]);
+#pragma unroll
+            for (int e = 0; e < (2 << VB); e++) pa[e] = intra && (e >> 1) != out ? R(0) : pa[e] * sc;
+            v[x[k]] = a[k];
+            if (!intra) v[x[k] ^ tbit] = T{};
         }
     }
 }
@@ -155,10 +311,11 @@ unsigned grid_of(uint64_t units, int sm_count) {
     return (unsigned)std::max<uint64_t>(1, std::min<uint64_t>(b, (uint64_t)sm_count * 16));
 }
 
-Ins make_ins(uint64_t fixed) {
+// The bits of `fixed`, in vectors of 2^vb amplitudes.
+Ins make_ins(uint64_t fixed, int vb) {
     Ins in{};
     for (int b = 0; b < 64; b++)
-        if ((fixed >> b) & 1) in.pos[in.n++] = (int8_t)b;
+        if ((fixed >> b) & 1) in.pos[in.n++] = (int8_t)(b - vb);
     return in;
 }
 
@@ -176,10 +333,19 @@ sv_status launch_general(sv_state *h, const sv_gate *g, sv_launch_record &meta) 
             c.re[e] = (R)m.re[e];
             c.im[e] = (R)m.im[e];
         }
-        const uint64_t units = UINT64_C(1) << (n - 1 - k);
+        // complex64: two neighbouring amplitudes at a time unless bit 0 is
+        // one of the gate's
+        const int vb = sizeof(R) == 4 && !((cm | tb) & 1) ? 1 : 0;
+        const uint64_t units = UINT64_C(1) << (n - 1 - k - vb);
         meta.bytes = 2.0 * std::ldexp(1.0, -k) * (double)state_bytes(h);
         const int slot = prof_begin(h);
-        k_mcu<R><<<grid_of(units, h->sm_count), kThreads, 0, h->stream>>>(s, units, make_ins(cm | tb), cm, tb, c);
+        const unsigned grid = grid_of((units + kItems - 1) / kItems, h->sm_count);
+        if (vb) {
+            if constexpr (sizeof(R) == 4)
+                k_mcu<R, 1><<<grid, kThreads, 0, h->stream>>>(s, units, make_ins(cm | tb, 1), cm >> 1, tb >> 1, c);
+        } else {
+            k_mcu<R, 0><<<grid, kThreads, 0, h->stream>>>(s, units, make_ins(cm | tb, 0), cm, tb, c);
+        }
         SV_CUDA(cudaGetLastError());
         note_launch();
         prof_end(h, slot, meta);
@@ -191,26 +357,43 @@ sv_status launch_general(sv_state *h, const sv_gate *g, sv_launch_record &meta) 
                 m.re[4 * r + k] = (R)g[r].p[2 * k];
                 m.im[4 * r + k] = (R)g[r].p[2 * k + 1];
             }
-        const uint64_t units = N / 4;
+        const int vb = sizeof(R) == 4 && !((ma | mb) & 1) ? 1 : 0;
+        const uint64_t units = N >> (2 + vb);
         meta.bytes = 2.0 * (double)state_bytes(h);
         const int slot = prof_begin(h);
-        k_u2q<R><<<grid_of(units, h->sm_count), kThreads, 0, h->stream>>>(s, units, make_ins(ma | mb), ma, mb, m);
+        const unsigned grid = grid_of((units + 1) / 2, h->sm_count);
+        if (vb) {
+            if constexpr (sizeof(R) == 4)
+                k_u2q<R, 1><<<grid, kThreads, 0, h->stream>>>(s, units, make_ins(ma | mb, 1), ma >> 1, mb >> 1, m);
+        } else {
+            k_u2q<R, 0><<<grid, kThreads, 0, h->stream>>>(s, units, make_ins(ma | mb, 0), ma, mb, m);
+        }
         SV_CUDA(cudaGetLastError());
         note_launch();
         prof_end(h, slot, meta);
     } else {  // SV_MEASURE
         SV_TRY(ensure_meas(h, h->nmeas + 1));
-        const uint64_t tb = UINT64_C(1) << g[0].target;
         double *part = reinterpret_cast<double *>(h->small);
         double *dec = part + 2 * kMeasBlocks;
-        const int nb = (int)std::min<uint64_t>(kMeasBlocks, grid_of(N, h->sm_count));
-        meta.bytes = 3.0 * (double)state_bytes(h);  // one read to sum, one read and write to collapse
+        unsigned *done = reinterpret_cast<unsigned *>(static_cast<char *>(h->small) + kSmallDone);
+        // complex64 vectors hold two amplitudes: a measurement of bit 0 finds
+        // both halves in each vector
+        constexpr int VB = sizeof(R) == 4 ? 1 : 0;
+        const int q = g[0].target;
+        const bool intra = VB && q == 0;
+        const int pos = intra ? 0 : q - VB;
+        const uint64_t units = intra ? N >> 1 : N >> (1 + VB);
+        const uint64_t tb = intra ? 0 : UINT64_C(1) << pos;
+        const unsigned grid = grid_of((units + kItems - 1) / kItems, h->sm_count);
+        const unsigned nb = std::min<unsigned>(kMeasBlocks, grid);
+        // one read to sum; one read of the kept half and one write to collapse
+        meta.bytes = 2.5 * (double)state_bytes(h);
         const int slot = prof_begin(h);
-        k_meas_partial<R><<<nb, kThreads, 0, h->stream>>>(s, N, tb, part);
-        k_meas_decide<<<1, 1, 0, h->stream>>>(part, nb, g[0].p[0], dec, h->meas_dev + h->nmeas);
-        k_meas_collapse<R><<<grid_of(N, h->sm_count), kThreads, 0, h->stream>>>(s, N, tb, dec);
+        k_meas_decide<R, VB><<<nb, kThreads, 0, h->stream>>>(s, units, pos, tb, intra, part, done, g[0].p[0], dec,
+                                                            h->meas_dev + h->nmeas);
+        k_meas_collapse<R, VB><<<grid, kThreads, 0, h->stream>>>(s, units, pos, tb, intra, dec);
         SV_CUDA(cudaGetLastError());
-        note_launch(3);
+        note_launch(2);
         prof_end(h, slot, meta);
         h->nmeas++;
     }
@@ -225,7 +408,7 @@ int general_records(int kind) { return kind == SV_U2Q ? 4 : 1; }
 bool is_general_kind(int kind) { return kind == SV_MCU || kind == SV_U2Q || kind == SV_MEASURE; }
 
 sv_status general_apply(sv_state *h, const sv_gate *g) {
-    static_assert(2 * kMeasBlocks * sizeof(double) + 64 <= 64 * 1024, "measurement scratch fits the small area");
+    static_assert(2 * kMeasBlocks * sizeof(double) + 64 <= kSmallDone, "measurement scratch fits the small area");
     SV_TRY(materialize(h));
     SV_TRY(resolve_norm(h));
     SV_TRY(launch_check());

@@ -127,8 +127,8 @@ struct Stats {
     ReadResult *res;
     unsigned *done;  // zero between launches
 };
-constexpr size_t kStatRes = 3 * 8 * kMaxStatBlocks, kStatDone = 65536 - 64;
-static_assert(kStatRes + sizeof(ReadResult) <= kStatDone, "reduction scratch");
+constexpr size_t kStatRes = 3 * 8 * kMaxStatBlocks;
+static_assert(kStatRes + sizeof(ReadResult) <= kSmallDone, "reduction scratch");
 
 Stats stats_of(sv_state *h) {
     char *b = reinterpret_cast<char *>(h->small);
@@ -137,7 +137,7 @@ Stats stats_of(sv_state *h) {
     s.best = s.sum + kMaxStatBlocks;
     s.idx = reinterpret_cast<uint64_t *>(s.best + kMaxStatBlocks);
     s.res = reinterpret_cast<ReadResult *>(b + kStatRes);
-    s.done = reinterpret_cast<unsigned *>(b + kStatDone);
+    s.done = reinterpret_cast<unsigned *>(b + kSmallDone);
     return s;
 }
 
