@@ -284,12 +284,11 @@ sv_status sv_batch_create(const sv_batch_item *items, size_t count, const sv_con
             // the first pass generates the starting product state
             if (pass.size() == (size_t)bi.pass0) t2_set_gen(t2, cp.basis, cp.basis_h, &a);
             Off o;
-            o.ins = blob.put(t2.ins.data(), t2.ins.size() * sizeof(T2Ins));
+            o.ins = blob.put(t2.dev.data(), t2.dev.size() * sizeof(T2Ins));
             o.stages = blob.put(t2.stages.data(), t2.stages.size() * sizeof(T2Stage));
             o.layx = blob.put(t2.layx.data(), t2.layx.size() * sizeof(T2LayoutX));
             o.epi = blob.put(&t2.epi, sizeof(T2Epilogue));
             o.mats = blob.put(t2.mats.data(), t2.mats.size() * sizeof(T2Mat));
-            o.fac = blob.put(t2.fac2.data(), t2.fac2.size() * sizeof(T2Fac));
             o.statc = blob.put(t2.statc.data(), t2.statc.size() * sizeof(float));
             o.soff = blob.put(t2.soff.data(), t2.soff.size() * sizeof(int32_t));
             o.sterms = blob.put(t2.sterms.data(), t2.sterms.size() * sizeof(T2SlotTerm));
@@ -338,7 +337,6 @@ sv_status sv_batch_create(const sv_batch_item *items, size_t count, const sv_con
         pass[p].layx = reinterpret_cast<const T2LayoutX *>(dev + offs[p].layx);
         pass[p].epi = reinterpret_cast<const T2Epilogue *>(dev + offs[p].epi);
         pass[p].mats = reinterpret_cast<const float4 *>(dev + offs[p].mats);
-        pass[p].fac = reinterpret_cast<const int4 *>(dev + offs[p].fac);
         pass[p].statc = reinterpret_cast<const float2 *>(dev + offs[p].statc);
         pass[p].soff = reinterpret_cast<const int32_t *>(dev + offs[p].soff);
         pass[p].sterms = reinterpret_cast<const T2SlotTerm *>(dev + offs[p].sterms);

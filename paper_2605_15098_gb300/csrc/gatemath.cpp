@@ -122,12 +122,19 @@ uint64_t diag_turns64(const sv_gate &g, bool *exact) {
         case SV_P:
         case SV_CP: {
             *exact = false;
-            const double inv_two_pi = 0.15915494309189533576888376337251;
-            double f = g.p[0] * inv_two_pi;
-            f -= std::floor(f);  // [0, 1)
-            double scaled = std::ldexp(f, 64);
-            if (scaled >= 0x1p64) return 0;
-            return (uint64_t)scaled;
+            // p / (2 pi) as an unevaluated sum (the product, its exact
+            // remainder and the tail of 1 / (2 pi)), so that the phase is
+            // good to 2^-64 of a turn whatever the angle's size
+            const double inv_hi = 0x1.45f306dc9c883p-3, inv_lo = -0x1.6b01ec5417056p-57;
+            const double hi = g.p[0] * inv_hi;
+            const double lo = std::fma(g.p[0], inv_hi, -hi) + g.p[0] * inv_lo;
+            if (!std::isfinite(hi)) return 0;
+            auto turns = [](double x) -> uint64_t {  // x mod 1
+                if (std::fabs(x) < 0.25) return (uint64_t)(int64_t)std::llrint(std::ldexp(x, 64));
+                const double f = x - std::floor(x);
+                return f >= 1.0 ? 0 : (uint64_t)std::ldexp(f, 64);
+            };
+            return turns(hi) + turns(lo);
         }
         default:
             *exact = true;

@@ -84,7 +84,8 @@ sv_status learned_entry(sv_state *h, const std::vector<sv_gate> &gates, const sv
     const bool dbl = h->dt == SV_C128;
     const bool allow_t2 = !dbl && !(cfg.flags & SV_FLAG_GENERIC_TILE);
     const bool fused = cfg.mode == SV_MODE_FUSED;
-    const PlanOptions base = plan_options(h->n, h->dt, cfg);
+    PlanOptions base = plan_options(h->n, h->dt, cfg);
+    if (dbl) base.split_u3 = false;  // its candidates run on the generic tile kernel
     if (dbl && base.k > 13) return fail(SV_ERR_ARG, "complex128 tiles hold at most 2^13 amplitudes");
 
     // candidate planner options; the configuration's own options come first

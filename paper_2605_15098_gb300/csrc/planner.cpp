@@ -345,6 +345,16 @@ std::string build_plan_paper(const std::vector<sv_gate> &gates, const std::vecto
 
 }  // namespace
 
+// Whether the passes of a complex128 plan run on the register-stage kernel.
+// There a split U3 is two FP64 operations per amplitude and its phases join
+// the diagonal runs, against eight for the complex 2x2 (random circuit
+// n = 21, depth 10: 8.35 -> 3.38 ms); the generic tile kernel's diagonal runs
+// cost more than they save.  The error against a reference that does not round
+// phi + lambda halves (n = 20, depth 12: 4.7e-15 -> 1.7e-15).
+bool c128_register_stage(const PlanOptions &opt, int flags) {
+    return opt.n >= 13 && opt.k == 13 && opt.c >= 4 && opt.merge_diag && !(flags & SV_FLAG_GENERIC_TILE);
+}
+
 PlanOptions plan_options(int n, sv_dtype dt, const sv_config &cfg) {
     PlanOptions opt;
     opt.n = n;
@@ -360,7 +370,7 @@ PlanOptions plan_options(int n, sv_dtype dt, const sv_config &cfg) {
     opt.search = !(cfg.flags & SV_FLAG_GREEDY_ONLY);
     if (opt.paper) opt.c = opt.k;  // the block is contiguous
     if ((cfg.flags & SV_FLAG_NARROW_FIRST) && !opt.paper) opt.first_c = 4;
-    opt.split_u3 = !dbl;
+    opt.split_u3 = !dbl || c128_register_stage(opt, cfg.flags);
     return opt;
 }
 

@@ -52,6 +52,11 @@ struct T2Pass {
     // multiplied into the generated state instead of applied at the end
     double gen_scale = 1.0;
     std::vector<T2TileTerm> tterms;
+    // format 2: the programme the kernels run (tileprog.h), its last stage
+    // change and, for the gen variant, its closing scale
+    std::vector<T2Ins> dev;
+    int dev_last_stage = -1;
+    double dev_gen_scale = 1.0;
     int nblocks = 0;
     std::vector<double> blocks64;   // fused: per block 2 x 32 x 32 (re, im), row = output index
     std::vector<float> blocks_dev;  // fused: per block kBlockFloats in the device layout
@@ -62,7 +67,7 @@ struct T2Device {
     const T2Ins *ins;
     const T2Stage *stages;
     const T2Mat *mats;
-    const void *fac;         // T2Factor (format 1) or T2Fac (format 2) records
+    const void *fac;         // format 1: T2Factor records
     const uint32_t *stat;    // format 1
     const float *statc;      // format 2
     const T2Slot *slots;     // format 2
@@ -78,17 +83,16 @@ struct T2Device {
 struct T2Args {
     uint64_t gmask, ntiles;
     int c, nins;
-    int nfac, nrows, nslots, nmats, nstages;  // factor records, static rows, slots, matrix records, stages
+    int nrows, nslots, nmats, nstages;  // static rows, slots, matrix records, stages
     int last_stage;  // index of the last T2_STAGE instruction
     int slot_phys[kMaxTileQubits];
     // the tile's physical base index: tile index bits [gs[r], gs[r] + gl[r])
     // go to physical bits gd[r].. (runs of the global bits)
     int ngr;
     int8_t gs[32], gd[32], gl[32];
-    const int4 *ins;       // T2Ins records
+    const int4 *ins;       // T2Ins records (device form)
     const int4 *stages;    // T2Stage records
     const float4 *mats;    // T2Mat records (two float4 each)
-    const int4 *fac;       // T2Fac records
     const float2 *statc;   // static complex rows (threads entries each)
     const int32_t *soff;   // slot term ranges
     const T2SlotTerm *sterms;
@@ -118,6 +122,13 @@ struct T2Args {
     // computes its own
     const float2 *slotv;
     int nsp;
+};
+
+// A pass's instructions as a launch parameter: the step loop reads them at a
+// uniform index from the parameter bank, so that every branch on them is
+// uniform.
+struct T2Prog {
+    int4 ins[kT2DevIns];
 };
 
 // Bytes of the per-tile slot values of a complex64 register-stage pass

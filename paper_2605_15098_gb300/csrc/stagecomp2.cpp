@@ -240,10 +240,17 @@ struct P64 {
     using Ph = uint64_t;
     using V = double;
     static Ph ph(uint64_t t64) { return t64; }
+    // cos and sin of 2 pi u / 2^64: the angle's rounding (up to 4e-16) is
+    // carried along and corrected to first order
     static void ex(Ph u, V *re, V *im) {
-        const double ang = 2.0 * M_PI * ((double)(int64_t)u * 0x1p-64);
-        *re = std::cos(ang);
-        *im = std::sin(ang);
+        const int64_t v = (int64_t)u;
+        const double h = (double)(v & ~INT64_C(0x7ff)), l = (double)(v & 0x7ff);  // both exact
+        const double two_pi = 0x1.921fb54442d18p+2 * 0x1p-64, tail = 0x1.1a62633145c07p-52 * 0x1p-64;
+        const double ang = h * two_pi;
+        const double err = std::fma(h, two_pi, -ang) + (h * tail + l * two_pi);
+        const double c = std::cos(ang), s = std::sin(ang);
+        *re = c - err * s;
+        *im = s + err * c;
     }
     static bool real(const double *m) { return m[1] == 0.0 && m[3] == 0.0 && m[5] == 0.0 && m[7] == 0.0; }
     // entries x of a phased butterfly on register bit j (bit j of x set)
@@ -293,6 +300,125 @@ struct P64 {
         o->sterms64.push_back({(int16_t)g0, (int16_t)g1, 0, th});
     }
 };
+
+// An unevaluated FP64 sum hi + lo.
+struct DD {
+    double hi, lo;
+};
+// x (1 + k^2), rounded to about 2^-104.
+DD times_one_plus_square(DD x, double k) {
+    const double q = k * k, qe = std::fma(k, k, -q);
+    const double f = 1.0 + q, fe = (q - (f - 1.0)) + qe;
+    const double p = x.hi * f;
+    const double e = std::fma(x.hi, f, -p) + (x.hi * fe + x.lo * f);
+    return {p + e, e - ((p + e) - p)};
+}
+// 1 / sqrt(x), with one correction step on the exact residual.
+double inverse_root(DD x) {
+    const double y = 1.0 / std::sqrt(x.hi);
+    const double t = x.hi * y, te = std::fma(x.hi, y, -t);
+    const double r = std::fma(-t, y, 1.0) - (te * y + x.lo * y * y);
+    return y + 0.5 * y * r;
+}
+
+// The device form of a compiled programme (tileprog.h).
+void lower(T2Pass *o, bool gen) {
+    // complex128 rotations [[1, -k], [k, 1]] and [[k, -1], [1, k]] grow the
+    // norm by sqrt(1 + k^2) for the k as rounded; the product of these and of
+    // the Hadamards' sqrt(2) is formed beyond FP64 and rounded once
+    DD grown{1.0, 0.0};
+    bool negative = (o->sign_flips & 1) != 0, rotated = false;
+    o->dev.clear();
+    auto rotation = [&](size_t i) { return i < o->ins.size() && o->ins[i].op == T2_ROT; };
+    double scale = 1.0;
+    bool scaled = false;
+    float hi = 0.f, lo = 0.f;
+    for (size_t i = 0; i < o->ins.size(); i++) {
+        const T2Ins &in = o->ins[i];
+        if (rotation(i)) {
+            T2Ins g{};
+            g.op = T2_ROT;
+            g.hd = kT2HdRots;
+            g.aux = in.aux;
+            int mask = 0, order = 0, count = 0, sine = 0;
+            for (; rotation(i) && !((mask >> o->ins[i].idx) & 1) && o->ins[i].aux == in.aux + count; i++, count++) {
+                const int j = o->ins[i].idx;
+                mask |= 1 << j;
+                order |= count << (3 * j);
+                if (o->wide) {
+                    const double *m = &o->mats64[8 * (size_t)o->ins[i].aux];
+                    if (m[4] != 0.0) sine |= 1 << j;
+                    grown = times_one_plus_square(grown, m[2]);
+                    negative ^= m[4] != 0.0 && m[1] < 0.0;
+                    rotated = true;
+                }
+            }
+            i--;
+            g.cidx = (int16_t)mask;
+            g.e0 = (int16_t)order;
+            g.idx = (int8_t)sine;
+            o->dev.push_back(g);
+            continue;
+        }
+        if (in.op == T2_DIAG) {
+            for (int e = in.e0; e < in.e1; e++) {
+                const T2Fac &f = o->fac2[e];
+                T2Ins d{};
+                d.op = T2_DIAG;
+                if (f.w0 & kFacTable) {
+                    d.hd = kT2HdTable;
+                    d.cidx = (int16_t)((f.w0 >> 10) & 0xfu);
+                    d.aux = f.row;
+                } else {
+                    d.hd = kT2HdFactor;
+                    d.idx = (int8_t)((f.w0 & 0xffu) ? 1 + __builtin_ctz(f.w0 & 0xffu) : 0);
+                    d.cidx = f.slot;
+                    d.e0 = (int16_t)f.row;
+                    d.e1 = f.dslot;
+                    d.aux = (int32_t)((f.w0 >> kFacDynShift) & 0x1ffu);
+                }
+                o->dev.push_back(d);
+            }
+            continue;
+        }
+        if (in.op == T2_SCALE) {  // the last step; taken up below
+            scaled = true;
+            if (o->wide) {
+                scale = o->mats64[8 * (size_t)in.aux];
+            } else {
+                hi = o->mats[in.aux].m[0];
+                lo = o->mats[in.aux].m[1];
+            }
+            continue;
+        }
+        if (in.op == T2_STAGE) o->dev_last_stage = (int)o->dev.size();
+        o->dev.push_back(in);
+    }
+    o->dev_gen_scale = o->gen_scale;
+    if (rotated) {
+        grown.hi = std::ldexp(grown.hi, o->n_h & ~1);
+        grown.lo = std::ldexp(grown.lo, o->n_h & ~1);
+        if (o->n_h & 1) grown = times_one_plus_square(grown, 1.0);
+        scale = inverse_root(grown) * (negative ? -1.0 : 1.0);
+        scaled = true;
+        o->dev_gen_scale = scale;
+    }
+    if (gen || !scaled) return;
+    T2Ins c{};
+    c.op = T2_SCALE;
+    c.hd = kT2HdScale;
+    int32_t words[2];  // e0 and e1, aux
+    if (o->wide) {
+        std::memcpy(words, &scale, sizeof scale);
+    } else {
+        std::memcpy(&words[0], &lo, sizeof lo);
+        std::memcpy(&words[1], &hi, sizeof hi);
+    }
+    c.e0 = (int16_t)(words[0] & 0xffff);
+    c.e1 = (int16_t)((uint32_t)words[0] >> 16);
+    c.aux = words[1];
+    o->dev.push_back(c);
+}
 
 template <class P>
 std::string compile_fmt2(const TilePass &tp, T2Pass *out, bool gen) {
@@ -392,7 +518,7 @@ std::string compile_fmt2(const TilePass &tp, T2Pass *out, bool gen) {
             // an uncontrolled rotation [[c, -s], [s, c]] runs as three shears;
             // with c < 0 it is -1 times the rotation by c' = -c, s' = -s, and
             // the sign joins the pass's closing scale
-            double rot_t = 0.0, rot_s = 0.0;
+            double rot_t = 0.0, rot_s = 0.0, rot_c = 0.0;
             if (in.op == T2_RGATE && op.type == TOP_GATE) {
                 const double c = op.m[0], s = op.m[4];
                 if (op.m[6] == c && op.m[2] == -s && std::fabs(c * c + s * s - 1.0) <= 1e-12) {
@@ -400,6 +526,7 @@ std::string compile_fmt2(const TilePass &tp, T2Pass *out, bool gen) {
                     const double cc = flip ? -c : c, ss = flip ? -s : s;
                     rot_t = -ss / (1.0 + cc);
                     rot_s = ss;
+                    rot_c = cc;
                     if (flip) out->sign_flips++;
                     in.op = T2_ROT;
                 }
@@ -431,6 +558,11 @@ std::string compile_fmt2(const TilePass &tp, T2Pass *out, bool gen) {
                 double m[8] = {};
                 m[0] = rot_t;
                 m[1] = rot_s;
+                // the unnormalised form: its coefficient, and whether it is
+                // divided by the sine
+                const bool by_sine = std::fabs(rot_s) > rot_c;
+                m[2] = by_sine ? rot_c / rot_s : rot_s / rot_c;
+                m[4] = by_sine ? 1.0 : 0.0;
                 in.aux = P::push_mat(out, m);
             } else if (in.op == T2_GATE || in.op == T2_RGATE) {
                 in.aux = P::push_mat(out, op.m);
@@ -739,6 +871,7 @@ std::string compile_fmt2(const TilePass &tp, T2Pass *out, bool gen) {
             // every step is linear: the pass that generates its starting
             // state generates it times the closing scale instead
             out->gen_scale = s;
+            lower(out, gen);
             return "";
         }
         T2Ins in{};
@@ -748,6 +881,7 @@ std::string compile_fmt2(const TilePass &tp, T2Pass *out, bool gen) {
         out->ins.push_back(in);
     }
     if (P::nmats(out) > (size_t)kT2SmemMats) return "more matrix records than the kernel's shared-memory copy";
+    lower(out, gen);
     return "";
 }
 

@@ -308,13 +308,13 @@ struct T2Off {
 
 T2Off put_t2(Blob &blob, const T2Pass &t) {
     T2Off o;
-    o.ins = blob.put_vec(t.ins);
+    o.ins = t.format == 2 ? blob.put_vec(t.dev) : blob.put_vec(t.ins);
     o.stages = blob.put_vec(t.stages);
     o.layx = blob.put_vec(t.layx);
     o.epi = blob.put(&t.epi, sizeof(T2Epilogue));
     // a complex128 programme's FP64 records take the places of the FP32 ones
     o.mats = t.wide ? blob.put_vec(t.mats64) : blob.put_vec(t.mats);
-    o.fac = t.format == 2 ? blob.put_vec(t.fac2) : blob.put_vec(t.factors);
+    if (t.format != 2) o.fac = blob.put_vec(t.factors);  // format 2: in the steps
     o.stat = blob.put_vec(t.stat);
     o.statc = t.wide ? blob.put_vec(t.statc64) : blob.put_vec(t.statc);
     o.slots = blob.put_vec(t.slots);

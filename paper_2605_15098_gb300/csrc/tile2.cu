@@ -21,6 +21,7 @@
 // one multiplication by 2^(-h/2), exact for even h, so the norm carries no
 // bias from a rounded 1/sqrt(2).
 #include <algorithm>
+#include <cstring>
 
 #include "common.h"
 #include "plan.h"
@@ -48,9 +49,8 @@ struct Geo {
     static constexpr size_t kOffTab = kTileBytes;
     static constexpr size_t kOffRows = kOffTab + (size_t)kTabEntries * 8;
     static constexpr size_t kOffMats = kOffRows + (size_t)kT2SmemRows * kThreads * 8;
-    static constexpr size_t kOffFac = kOffMats + (size_t)kT2SmemMats * sizeof(T2Mat);
-    static constexpr size_t kOffIns = kOffFac + (size_t)kT2SmemFactors * 16;
-    static constexpr size_t kOffSlotc = kOffIns + (size_t)kT2SmemIns * 16;  // two buffers
+    static constexpr size_t kOffIns = kOffMats + (size_t)kT2SmemMats * sizeof(T2Mat);
+    static constexpr size_t kOffSlotc = kOffIns + (size_t)kT2DevIns * 16;  // two buffers
     static constexpr size_t kOffLay = kOffSlotc + 2 * (size_t)kT2MaxSlots * 8;
     static constexpr size_t kOffEpi = kOffLay + (size_t)kT2SmemStages * sizeof(T2LayoutX);
     static constexpr size_t kOffOnes = kOffEpi + sizeof(T2Epilogue);  // the identity phase table
@@ -118,7 +118,7 @@ struct LayoutS {
 // path in the loop costs registers and instructions in all the others).
 constexpr int kFeatX = 1, kFeatR = 2, kFeatU = 4, kFeatAll = 7;
 
-// Gate KIND (0..4: H, X, real 2x2, shear rotation, general 2x2) on register
+// Gate KIND (0, 1, 2, 4: H, X, real 2x2, general 2x2) on register
 // bit SLOT (0..4).  Kinds outside the instantiation's set F compile to
 // nothing: the host never launches them there.
 template <int F, int KIND, int SLOT, int NP>
@@ -136,7 +136,6 @@ __device__ __forceinline__ void run_gate(RegsN<NP> &r, const float4 *mrec, uint3
         if constexpr (KIND == 0) reg_h2<SLOT>(r, qm);
         else if constexpr (KIND == 1) reg_x2<SLOT>(r, qm);
         else if constexpr (KIND == 2) reg_r2<SLOT>(r, qm, m);
-        else if constexpr (KIND == 3) reg_rot<SLOT>(r, qm, m);
         else reg_u2<SLOT>(r, qm, m);
     }
 }
@@ -311,6 +310,12 @@ __device__ __forceinline__ void reg_hph_s(RegsN<NP> &r, uint32_t qm, const float
     }
 }
 
+// The programme's instructions, copied to shared memory (L2 block and batched
+// kernels, whose CTAs change programmes).
+struct SmemIns {
+    __device__ int4 operator()(int pc) const { return reinterpret_cast<const int4 *>(t2_dyn_smem + G13::kOffIns)[pc]; }
+};
+
 // `rbar`: mbarrier that every warp arrives at once it has read a stage's
 // layout from shared memory (count: the CTA's warps); `rd` counts this
 // thread's arrivals.  A stage change waits for the phase of the previous read
@@ -319,66 +324,52 @@ __device__ __forceinline__ void reg_hph_s(RegsN<NP> &r, uint32_t qm, const float
 // index; `slotc`: the tile's slot values.  After the last stage change has
 // read shared memory, `hook()` runs (the callers start the next tile's bulk
 // copies there, once rbar shows every warp's reads done).
-template <int K, int F, typename Hook>
-__device__ __forceinline__ void t2_run(const T2Args &a, float4 *gstate, uint64_t *rbar, uint32_t &rd,
+template <int K, int F, typename Ins, typename Hook>
+__device__ __forceinline__ void t2_run(const T2Args &a, Ins ins, float4 *gstate, uint64_t *rbar, uint32_t &rd,
                                        uint64_t base, const float2 *slotc, Hook hook) {
     using G = Geo<K>;
-    // the programme: copied to shared memory by k_tile2 (once per CTA) and
-    // k_batch (once per pass); static rows and layouts beyond the copy stay
-    // in global memory
-    const int4 *ins = reinterpret_cast<const int4 *>(t2_dyn_smem + G::kOffIns);
-    const int4 *fac = reinterpret_cast<const int4 *>(t2_dyn_smem + G::kOffFac);
+    // the programme: its steps come from `ins`; its records are copied to
+    // shared memory by k_tile2 (once per CTA) and k_batch (once per pass);
+    // static rows and layouts beyond the copy stay in global memory
     const float2 *rows = reinterpret_cast<const float2 *>(t2_dyn_smem + G::kOffRows);
     const float4 *M = reinterpret_cast<const float4 *>(t2_dyn_smem + G::kOffMats);
     const T2LayoutX *lays = reinterpret_cast<const T2LayoutX *>(t2_dyn_smem + G::kOffLay);
     const float4 *ones = reinterpret_cast<const float4 *>(t2_dyn_smem + G::kOffOnes);
     float4 *tile4 = reinterpret_cast<float4 *>(t2_dyn_smem);
     const int tid = threadIdx.x;
-    auto layout = [&](int st) -> const T2LayoutX * { return st < kT2SmemStages ? lays + st : a.layx + st; };
+    // a layout's positions; each source its own load instructions
+    auto layout_s = [&](int st) -> LayoutS {
+        if (st < kT2SmemStages) return LayoutS(lays + st, tid);
+        return LayoutS(a.layx + st, tid);
+    };
     RegsN<kNP2> r;
     int stage = 0;
     bool live = false;
-    // a per-thread factor: static row x tile slot x one slot per dynamic thread bit set
-    auto thread_factor = [&](const int4 fd) -> float2 {
-        const uint32_t w0 = (uint32_t)fd.x;
-        const int sl = (int16_t)(fd.y & 0xffff), dsl = (int16_t)((uint32_t)fd.y >> 16);
+    auto static_row = [&](int row) -> float2 {
+        return row < kT2SmemRows ? rows[row * G::kThreads + tid] : __ldg(a.statc + (size_t)row * G::kThreads + tid);
+    };
+    // a per-thread factor (a Factor step): static row x tile slot x one slot
+    // per dynamic thread bit set
+    auto thread_factor = [&](const int4 w) -> float2 {
+        const int sl = (int16_t)(w.y & 0xffff), row = (int16_t)(w.z & 0xffff), dsl = (int16_t)(w.z >> 16);
         float2 f = make_float2(1.f, 0.f);
-        if (fd.z >= 0)
-            f = fd.z < kT2SmemRows ? rows[fd.z * G::kThreads + tid]
-                                   : __ldg(a.statc + (size_t)fd.z * G::kThreads + tid);
+        if (row >= 0) f = static_row(row);
         if (sl >= 0) f = cx(f, slotc[sl]);
-        const uint32_t dmask = (w0 >> kFacDynShift) & 0x1ffu;
-        uint32_t dm = dmask & (uint32_t)tid;
-        while (dm) {
-            const int t = __ffs(dm) - 1;
-            dm &= dm - 1;
-            f = cx(f, slotc[dsl + __popc(dmask & ((1u << t) - 1u))]);
+        int k = dsl;
+        for (uint32_t dm = (uint32_t)w.w; dm; dm &= dm - 1, k++) {
+            const float2 g = cx(f, slotc[k]);
+            if ((tid >> (__ffs(dm) - 1)) & 1) f = g;
         }
         return f;
     };
-    // the run of a phased butterfly: its table (or the identity) and its factor
-    auto hph_run = [&](const int4 w, const float4 *&T, float2 &ph) {
-        const int e0 = (int16_t)(w.z & 0xffff), e1 = (int16_t)(w.z >> 16);
-        T = ones;
-        ph = make_float2(1.f, 0.f);
-        for (int e = e0; e < e1; e++) {
-            const int4 fd = fac[e];
-            if ((uint32_t)fd.x & kFacTable)
-                T = M + 2 * fd.z;
-            else
-                ph = thread_factor(fd);
-        }
-    };
-    // the same from the step itself: its table, static row and slot are
-    // independent loads (no factor record first)
+    // the run of a phased butterfly, from the step itself: its table (or the
+    // identity), static row and slot are independent loads
     auto hph_direct = [&](const int4 w, const float4 *&T, float2 &ph) {
         const int trec = (int)((uint32_t)w.w & 0xffffu) - 1, row = (int)((uint32_t)w.w >> 16) - 1;
         const int sl = (int16_t)(w.y & 0xffff);
         T = trec >= 0 ? M + 2 * trec : ones;
         ph = make_float2(1.f, 0.f);
-        if (row >= 0)
-            ph = row < kT2SmemRows ? rows[row * G::kThreads + tid]
-                                   : __ldg(a.statc + (size_t)row * G::kThreads + tid);
+        if (row >= 0) ph = static_row(row);
         if (sl >= 0) ph = cx(ph, slotc[sl]);
     };
     // loop bounds in registers: `a` may live in memory the compiler cannot
@@ -386,24 +377,53 @@ __device__ __forceinline__ void t2_run(const T2Args &a, float4 *gstate, uint64_t
     // indexes its passes' arguments)
     const int nins = a.nins, last_stage = a.last_stage;
     for (int pc = 0; pc < nins; pc++) {
-        const int4 w = ins[pc];
+        const int4 w = ins(pc);
         // all ones at run time (the handler code is below 256), opaque to the
         // compiler (see reg_h2)
         const uint32_t qm = ~((uint32_t)w.y >> 24);
         const float4 *mrec = M + 2 * w.w;
-        // one switch on the handler code the stage compiler set (tileprog.h)
-        switch (((uint32_t)w.y >> 16) & 0xffu) {
+        const uint32_t hd = ((uint32_t)w.y >> 16) & 0xffu;  // the handler code (tileprog.h)
+        if constexpr ((F & kFeatR) != 0) {
+            if (hd == kT2HdRots) {
+                const uint32_t mask = (uint32_t)w.y & 31u, order = (uint32_t)w.z;
+                const float2 *rec = reinterpret_cast<const float2 *>(mrec);
+#define SV_ROT(J)                                                   \
+    if (mask & (1u << J)) {                                         \
+        const float2 ts = rec[4 * ((order >> (3 * J)) & 7u)];       \
+        reg_rot<J>(r, ts.x, ts.y);                                  \
+    }
+                SV_ROT(1)
+                SV_ROT(2)
+                SV_ROT(3)
+                SV_ROT(4)
+                SV_ROT(0)
+#undef SV_ROT
+                continue;
+            }
+        }
+        if (hd == kT2HdTable) {
+            const uint32_t pb = (uint32_t)w.y & 0xfu;  // thread-bit predicate
+            if (!pb || ((tid >> (pb - 1)) & 1)) apply_table_s(r, mrec, qm);
+            continue;
+        }
+        if (hd == kT2HdFactor) {
+            const float2 ff = thread_factor(w);
+            const int j = (w.x >> 16) & 0xff;
+            apply_factor_bit(r, j ? 1 << (j - 1) : 0, ff.x, ff.y);
+            continue;
+        }
+        switch (hd) {
             case kT2HdStage: {
                 if (live) {
                     // every warp has read the previous layout before any overwrites it
                     if (!mbar_wait(rbar, (rd - 1u) & 1u)) atomicExch(a.err, 1);
-                    const LayoutS L(layout(stage), tid);
+                    const LayoutS L = layout_s(stage);
 #pragma unroll
                     for (int q = 0; q < kNP2; q++)
                         tile4[L.idx(q)] = make_float4(r.re[q].x, r.re[q].y, r.im[q].x, r.im[q].y);
                     __syncthreads();
                     stage = w.w;
-                    const LayoutS L2(layout(stage), tid);
+                    const LayoutS L2 = layout_s(stage);
 #pragma unroll
                     for (int q = 0; q < kNP2; q++) {
                         const float4 v = tile4[L2.idx(q)];
@@ -411,8 +431,8 @@ __device__ __forceinline__ void t2_run(const T2Args &a, float4 *gstate, uint64_t
                         r.im[q] = make_float2(v.z, v.w);
                     }
                 } else {
-                    stage = w.w;
-                    const Layout2 L(layout(stage), tid);
+                    stage = w.w;  // 0
+                    const Layout2 L(lays, tid);
                     if (a.gen) {
                         // the product state H^{hq}|b>, generated instead of
                         // read: +-v where the index agrees with b off the
@@ -467,8 +487,7 @@ __device__ __forceinline__ void t2_run(const T2Args &a, float4 *gstate, uint64_t
                 continue;
             }
             case kT2HdScale: {
-                const float4 mm = mrec[0];
-                const float hi = mm.x, lo = mm.y;
+                const float hi = __int_as_float(w.w), lo = __int_as_float(w.z);
                 if (lo == 0.f) {  // an even number of Hadamards: an exact power of two
 #pragma unroll
                     for (int q = 0; q < kNP2; q++) {
@@ -484,32 +503,12 @@ __device__ __forceinline__ void t2_run(const T2Args &a, float4 *gstate, uint64_t
                 }
                 continue;
             }
-            case kT2HdDiag: {
-                const int e0 = (int16_t)(w.z & 0xffff), e1 = (int16_t)(w.z >> 16);
-                for (int e = e0; e < e1; e++) {
-                    const int4 fd = fac[e];
-                    const uint32_t w0 = (uint32_t)fd.x;
-                    if (w0 & kFacTable) {
-                        const int pb = (int)((w0 >> 10) & 0xfu);  // thread-bit predicate
-                        if (pb && !((tid >> (pb - 1)) & 1)) continue;
-                        apply_table_s(r, M + 2 * fd.z, qm);
-                        continue;
-                    }
-                    const float2 ff = thread_factor(fd);
-                    apply_factor_bit(r, (int)(w0 & 0xffu), ff.x, ff.y);
-                }
-                continue;
-            }
 #define SV_HPH_CASE(J)                                              \
     case kT2Handler + 8 * 5 + J: {                                  \
         const float4 *T;                                            \
         float2 ph;                                                  \
-        const int8_t hc = (int8_t)(w.x >> 24);                      \
-        if (hc == kT2HphDirect || hc == kT2HphShared)               \
-            hph_direct(w, T, ph);                                   \
-        else                                                        \
-            hph_run(w, T, ph);                                      \
-        reg_hph_s<J>(r, qm, T, T != ones, ph.x, ph.y, hc == kT2HphShared); \
+        hph_direct(w, T, ph);                                       \
+        reg_hph_s<J>(r, qm, T, T != ones, ph.x, ph.y, (int8_t)(w.x >> 24) == kT2HphShared); \
         continue;                                                   \
     }
             SV_HPH_CASE(0)
@@ -527,7 +526,6 @@ __device__ __forceinline__ void t2_run(const T2Args &a, float4 *gstate, uint64_t
             SV_GATE_CASES(0)
             SV_GATE_CASES(1)
             SV_GATE_CASES(2)
-            SV_GATE_CASES(3)
             SV_GATE_CASES(4)
 #undef SV_GATE_CASES
             default: break;
@@ -646,13 +644,11 @@ template <int K>
 __device__ __forceinline__ void load_programme(const T2Args &a, unsigned char *sm, int tid, int nthreads) {
     using G = Geo<K>;
     int4 *si = reinterpret_cast<int4 *>(sm + G::kOffIns);
-    int4 *sf = reinterpret_cast<int4 *>(sm + G::kOffFac);
     float2 *sr = reinterpret_cast<float2 *>(sm + G::kOffRows);
     float4 *smat = reinterpret_cast<float4 *>(sm + G::kOffMats);
     int4 *slay = reinterpret_cast<int4 *>(sm + G::kOffLay);
     int4 *sepi = reinterpret_cast<int4 *>(sm + G::kOffEpi);
     for (int i = tid; i < a.nins; i += nthreads) si[i] = __ldg(a.ins + i);
-    for (int i = tid; i < a.nfac; i += nthreads) sf[i] = __ldg(a.fac + i);
     for (int i = tid; i < 2 * a.nmats; i += nthreads) smat[i] = __ldg(a.mats + i);
     const int nl = min(a.nstages, kT2SmemStages) * (int)(sizeof(T2LayoutX) / 16);
     for (int i = tid; i < nl; i += nthreads) slay[i] = __ldg(reinterpret_cast<const int4 *>(a.layx) + i);
@@ -728,10 +724,17 @@ __global__ void k_slotv(const T2Args a, float2 *__restrict__ out) {
 // by warp 0, and the other warps waited for it: random circuit n = 28, depth
 // 8: 27.5 -> 22.6 ms, a middle pass at n = 25 642 -> 555 us; with c = 9 (16
 // chunks) QPE n = 28 3.94 -> 3.89 ms.
+// The steps are read from the launch parameters in the device form of
+// tileprog.h (rotations grouped, a diagonal factor's record in its step):
+// 22.6 -> 20.8 ms, the middle pass 501 us, QPE n = 28 3.79 -> 3.70 ms.  Issue
+// bounds such a pass: per tile and warp (instructions executed, by regression
+// over the passes of eight circuits of n = 24) 409 for the tile itself, 174 a
+// stage change, 51 a rotation (48 multiply-adds) and 65 a group of them, 128
+// a phase table, 154 a thread factor, 112 a register-bit factor.
 template <int K, int F>
 __global__ void __launch_bounds__(Geo<K>::kThreads, K == kT2Qubits ? 2 : 1)
     k_tile2(float *__restrict__ state, const T2Args a, const __grid_constant__ CUtensorMap map,
-            const __grid_constant__ TileBox box) {
+            const __grid_constant__ TileBox box, const __grid_constant__ T2Prog prog) {
     using G = Geo<K>;
     extern __shared__ __align__(1024) unsigned char sm[];
     float2 *tab = reinterpret_cast<float2 *>(sm + G::kOffTab);
@@ -804,7 +807,8 @@ __global__ void __launch_bounds__(Geo<K>::kThreads, K == kT2Qubits ? 2 : 1)
                 issue_slots_only(next, nsc);
             }
         };
-        t2_run<K, F>(a, reinterpret_cast<float4 *>(state), rbar, rd, base, sc, hook);
+        t2_run<K, F>(a, [&](int pc) { return prog.ins[pc]; }, reinterpret_cast<float4 *>(state), rbar, rd, base, sc,
+                     hook);
         parity ^= 1u;
         buf ^= 1u;
         base = next_base;
@@ -936,7 +940,7 @@ __global__ void __launch_bounds__(kT2Threads, 2)
                 }
             }
         };
-        t2_run<kT2Qubits, F>(a, reinterpret_cast<float4 *>(state), rbar, rd, base, sc, hook);
+        t2_run<kT2Qubits, F>(a, SmemIns(), reinterpret_cast<float4 *>(state), rbar, rd, base, sc, hook);
         sig = p + 1 < G.npass ? (long long)b * G.npass + p : -1;
         if (!a.gen) parity ^= 1u;
         buf ^= 1u;
@@ -1021,7 +1025,7 @@ __global__ void __launch_bounds__(kT2Threads, 2) k_batch(float *__restrict__ sta
                     issue_tile_load<kT2Qubits>(a, sm, state, tile + 1, bar, tid);
                 }
             };
-            t2_run<kT2Qubits, F>(a, reinterpret_cast<float4 *>(state), rbar, rd, base, sc, hook);
+            t2_run<kT2Qubits, F>(a, SmemIns(), reinterpret_cast<float4 *>(state), rbar, rd, base, sc, hook);
             buf ^= 1u;
         }
         // the next pass's bulk copies (and the read-out) see this pass's stores
@@ -1248,13 +1252,12 @@ void t2_fill_args(const T2Pass &p, const T2Device &d, int n, T2Args *a) {
     a->gmask = p.gmask;
     a->ntiles = UINT64_C(1) << (n - p.k);
     a->c = p.c;
-    a->nins = (int)p.ins.size();
-    a->nfac = (int)p.fac2.size();
+    a->nins = (int)p.dev.size();
     a->nrows = (int)((p.wide ? p.statc64.size() : p.statc.size()) / (2 * (size_t)p.threads));
     a->nslots = (int)p.slots.size();
     a->nmats = (int)(p.wide ? p.mats64.size() / 8 : p.mats.size());
     a->nstages = (int)p.stages.size();
-    a->last_stage = p.last_stage;
+    a->last_stage = p.dev_last_stage;
     for (int s = 0; s < p.k; s++) a->slot_phys[s] = p.slot_phys[s];
     // runs of the global bits: tile index bit i is the i-th lowest set bit of gmask
     a->ngr = 0;
@@ -1277,7 +1280,6 @@ void t2_fill_args(const T2Pass &p, const T2Device &d, int n, T2Args *a) {
     a->ins = reinterpret_cast<const int4 *>(d.ins);
     a->stages = reinterpret_cast<const int4 *>(d.stages);
     a->mats = reinterpret_cast<const float4 *>(d.mats);
-    a->fac = reinterpret_cast<const int4 *>(d.fac);
     a->statc = reinterpret_cast<const float2 *>(d.statc);
     a->soff = d.soff;
     a->sterms = d.sterms;
@@ -1324,7 +1326,7 @@ void t2_set_gen(const T2Pass &p, int64_t gen_basis, uint64_t basis_h, T2Args *a)
     a->gen_ghmask = basis_h & p.gmask;
     const int both = __builtin_popcount(p.gen_hmask & hq_local);
     const int hq_only = __builtin_popcountll(basis_h) - both;
-    a->gen_val64 = std::pow(2.0, 0.5 * (both - hq_only)) * p.gen_scale;
+    a->gen_val64 = std::pow(2.0, 0.5 * (both - hq_only)) * p.dev_gen_scale;
     a->gen_val = (float)a->gen_val64;
 }
 
@@ -1371,8 +1373,10 @@ sv_status t2_launch(sv_state *h, const T2Pass &p, const T2Device &d, const sv_la
     CUtensorMap map{};
     TileBox box{};
     if (!a.gen) SV_TRY(tile_map(h->amps, h->n, p.k, p.slot_phys, sizeof(float2), &map, &box));
+    T2Prog prog;
+    std::memcpy(prog.ins, p.dev.data(), p.dev.size() * sizeof(T2Ins));
     const int slot = prof_begin(h);
-    kern<<<(unsigned)grid, threads, smem, h->stream>>>(reinterpret_cast<float *>(h->amps), a, map, box);
+    kern<<<(unsigned)grid, threads, smem, h->stream>>>(reinterpret_cast<float *>(h->amps), a, map, box, prog);
     SV_CUDA(cudaGetLastError());
     note_launch();
     prof_end(h, slot, meta);

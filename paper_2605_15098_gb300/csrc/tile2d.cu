@@ -16,11 +16,17 @@
 //      and 32-entry FP64 tables; once the last stage change has read shared
 //      memory, the next tile's copies start;
 //   4. each thread writes its amplitudes from registers (16-byte stores).
+// The FP64 pipe bounds it (81-83 % busy): U3 gates run as P RY P with the
+// phases merged into the diagonal runs and RY divided by its cosine or sine
+// (two operations per amplitude instead of eight for the complex 2x2), phased
+// butterflies in six operations per pair instead of eight.  Random circuit
+// n = 21, depth 10: 8.35 -> 3.38 ms; QPE n = 24: 4.07 -> 3.06 ms.
 // Hadamards are unnormalised ([[1,1],[1,-1]]) with one multiplication by
-// 2^(-h/2) at the end of the pass; every per-amplitude operation is FP64, so
+// 2^(-h/2) (and the rotations' divisors) at the end of the pass; every per-amplitude operation is FP64, so
 // the arithmetic per touched amplitude is that of the gates' definitions
 // with the diagonal runs' phases merged exactly in integers.
 #include <algorithm>
+#include <cstring>
 
 #include "common.h"
 #include "plan.h"
@@ -44,9 +50,7 @@ struct GD {
     static constexpr size_t kTileBytes = (size_t)16 << kT2Qubits;
     static constexpr size_t kOffRows = kTileBytes;
     static constexpr size_t kOffMats = kOffRows + (size_t)kT2SmemRows * kDThreads * 16;
-    static constexpr size_t kOffFac = kOffMats + (size_t)kT2SmemMats * 64;
-    static constexpr size_t kOffIns = kOffFac + (size_t)kT2SmemFactors * 16;
-    static constexpr size_t kOffSlotc = kOffIns + (size_t)kT2SmemIns * 16;  // two buffers
+    static constexpr size_t kOffSlotc = kOffMats + (size_t)kT2SmemMats * 64;  // two buffers
     static constexpr size_t kOffLay = kOffSlotc + 2 * (size_t)kT2MaxSlots * 16;
     static constexpr size_t kOffEpi = kOffLay + (size_t)kT2SmemStages * sizeof(T2LayoutX);
     static constexpr size_t kOffOnes = kOffEpi + sizeof(T2Epilogue);  // the identity table
@@ -183,23 +187,26 @@ __device__ __forceinline__ void d_r(RegsD &r, uint32_t qm, const double *m) {
     }
 }
 
-// Rotation [[c, -s], [s, c]] as three shears a += t b, b += s a, a += t b
-// (m[0] = t, m[1] = s), the same factorisation as the complex64 kernel.
-template <int J>
-__device__ __forceinline__ void d_rot(RegsD &r, uint32_t qm, const double *m) {
-    const double t = m[0], s = m[1];
+// Rotation divided by its cosine, [[1, -k], [k, 1]], or (SINE) by its sine,
+// [[k, -1], [1, k]]; |k| <= 1 and the divisors are in the closing scale.
+// Two multiply-adds per output component pair: three shears, as the complex64
+// kernel runs, would take three, and the FP64 pipe bounds this kernel.
+template <int J, bool SINE>
+__device__ __forceinline__ void d_rot(RegsD &r, double k) {
 #pragma unroll
-    for (int g4 = 0; g4 < 4; g4++) {
-        if (!((qm >> g4) & 1)) continue;
-#pragma unroll
-        for (int i = 0; i < 4; i++) {
-            const int a = lo_of<J>(4 * g4 + i), b = a | (1 << J);
-            r.re[a] = fma(r.re[b], t, r.re[a]);
-            r.im[a] = fma(r.im[b], t, r.im[a]);
-            r.re[b] = fma(r.re[a], s, r.re[b]);
-            r.im[b] = fma(r.im[a], s, r.im[b]);
-            r.re[a] = fma(r.re[b], t, r.re[a]);
-            r.im[a] = fma(r.im[b], t, r.im[a]);
+    for (int g = 0; g < 16; g++) {
+        const int a = lo_of<J>(g), b = a | (1 << J);
+        const double ar = r.re[a], ai = r.im[a], br = r.re[b], bi = r.im[b];
+        if constexpr (SINE) {
+            r.re[a] = fma(k, ar, -br);
+            r.im[a] = fma(k, ai, -bi);
+            r.re[b] = fma(k, br, ar);
+            r.im[b] = fma(k, bi, ai);
+        } else {
+            r.re[a] = fma(-k, br, ar);
+            r.im[a] = fma(-k, bi, ai);
+            r.re[b] = fma(k, ar, br);
+            r.im[b] = fma(k, ai, bi);
         }
     }
 }
@@ -257,6 +264,17 @@ __device__ __forceinline__ void d_factor_bit(RegsD &r, int mask, double2 f) {
     }
 }
 
+// The butterfly (a + m b, a - m b) in six FP64 operations: the sum by
+// multiply-adds onto a, the difference as 2a minus the sum (eight with the
+// product formed first; one rounding less in the sum).
+__device__ __forceinline__ void d_bfly(RegsD &r, int a, int b, double2 m) {
+    const double ar = r.re[a], ai = r.im[a], br = r.re[b], bi = r.im[b];
+    r.re[a] = fma(-bi, m.y, fma(br, m.x, ar));
+    r.im[a] = fma(br, m.y, fma(bi, m.x, ai));
+    r.re[b] = fma(2.0, ar, -r.re[a]);
+    r.im[b] = fma(2.0, ai, -r.im[a]);
+}
+
 // Phased Hadamard on register bit J: b <- M b with M = f T[x_b], then the
 // pair becomes (a + M b, a - M b).  Without a table (`tab` false) M = f.
 template <int J>
@@ -277,13 +295,7 @@ __device__ __forceinline__ void d_hph(RegsD &r, uint32_t qm, const double2 *T, b
                 for (int i = 0; i < 8; i++) {
                     const int a = lo_of<J>(8 * g8 + i), b = a | (1 << J);
                     const double2 m = u[b & (NV - 1)];
-                    const double br = r.re[b], bi = r.im[b];
-                    const double pr = fma(-bi, m.y, br * m.x), pi = fma(br, m.y, bi * m.x);
-                    const double ar = r.re[a], ai = r.im[a];
-                    r.re[a] = ar + pr;
-                    r.im[a] = ai + pi;
-                    r.re[b] = ar - pr;
-                    r.im[b] = ai - pi;
+                    d_bfly(r, a, b, m);
                 }
             }
             return;
@@ -296,13 +308,7 @@ __device__ __forceinline__ void d_hph(RegsD &r, uint32_t qm, const double2 *T, b
         for (int i = 0; i < 8; i++) {
             const int a = lo_of<J>(8 * g8 + i), b = a | (1 << J);
             const double2 m = tab ? cxd(f, T[b]) : f;
-            const double br = r.re[b], bi = r.im[b];
-            const double pr = fma(-bi, m.y, br * m.x), pi = fma(br, m.y, bi * m.x);
-            const double ar = r.re[a], ai = r.im[a];
-            r.re[a] = ar + pr;
-            r.im[a] = ai + pi;
-            r.re[b] = ar - pr;
-            r.im[b] = ai - pi;
+            d_bfly(r, a, b, m);
         }
     }
 }
@@ -318,8 +324,6 @@ __device__ __forceinline__ void d_gate(RegsD &r, const double *m, uint32_t qm) {
         d_x<SLOT>(r, qm);
     } else if constexpr (KIND == 2) {
         d_r<SLOT>(r, qm, m);
-    } else if constexpr (KIND == 3) {
-        d_rot<SLOT>(r, qm, m);
     } else {
         d_u<SLOT>(r, qm, m);
     }
@@ -328,11 +332,9 @@ __device__ __forceinline__ void d_gate(RegsD &r, const double *m, uint32_t qm) {
 extern __shared__ __align__(1024) unsigned char t2d_smem[];
 
 // One tile of the pass: stages, gates, runs, and the write-back.
-template <int F, typename Hook>
-__device__ __forceinline__ void t2d_run(const T2Args &a, double2 *gstate, uint64_t *rbar, uint32_t &rd, uint64_t base,
+template <int F, typename Ins, typename Hook>
+__device__ __forceinline__ void t2d_run(const T2Args &a, Ins ins, double2 *gstate, uint64_t *rbar, uint32_t &rd, uint64_t base,
                                         const double2 *slotc, Hook hook) {
-    const int4 *ins = reinterpret_cast<const int4 *>(t2d_smem + GD::kOffIns);
-    const int4 *fac = reinterpret_cast<const int4 *>(t2d_smem + GD::kOffFac);
     const double2 *rows = reinterpret_cast<const double2 *>(t2d_smem + GD::kOffRows);
     const double2 *M = reinterpret_cast<const double2 *>(t2d_smem + GD::kOffMats);  // 4 per record
     const T2LayoutX *lays = reinterpret_cast<const T2LayoutX *>(t2d_smem + GD::kOffLay);
@@ -344,49 +346,65 @@ __device__ __forceinline__ void t2d_run(const T2Args &a, double2 *gstate, uint64
     RegsD r;
     int stage = 0;
     bool live = false;
-    auto thread_factor = [&](const int4 fd) -> double2 {
-        const uint32_t w0 = (uint32_t)fd.x;
-        const int sl = (int16_t)(fd.y & 0xffff), dsl = (int16_t)((uint32_t)fd.y >> 16);
+    auto static_row = [&](int row) -> double2 {
+        return row < kT2SmemRows ? rows[row * kDThreads + tid] : statc[(size_t)row * kDThreads + tid];
+    };
+    auto thread_factor = [&](const int4 w) -> double2 {
+        const int sl = (int16_t)(w.y & 0xffff), row = (int16_t)(w.z & 0xffff), dsl = (int16_t)(w.z >> 16);
         double2 f = make_double2(1.0, 0.0);
-        if (fd.z >= 0)
-            f = fd.z < kT2SmemRows ? rows[fd.z * kDThreads + tid] : statc[(size_t)fd.z * kDThreads + tid];
+        if (row >= 0) f = static_row(row);
         if (sl >= 0) f = cxd(f, slotc[sl]);
-        const uint32_t dmask = (w0 >> kFacDynShift) & 0x1ffu;
-        uint32_t dm = dmask & (uint32_t)tid;
-        while (dm) {
-            const int t = __ffs(dm) - 1;
-            dm &= dm - 1;
-            f = cxd(f, slotc[dsl + __popc(dmask & ((1u << t) - 1u))]);
-        }
+        int k = dsl;
+        for (uint32_t dm = (uint32_t)w.w; dm; dm &= dm - 1, k++)
+            if ((tid >> (__ffs(dm) - 1)) & 1) f = cxd(f, slotc[k]);
         return f;
     };
-    auto hph_run = [&](const int4 w, const double2 *&T, double2 &ph) {
-        const int e0 = (int16_t)(w.z & 0xffff), e1 = (int16_t)(w.z >> 16);
-        T = ones;
-        ph = make_double2(1.0, 0.0);
-        for (int e = e0; e < e1; e++) {
-            const int4 fd = fac[e];
-            if ((uint32_t)fd.x & kFacTable)
-                T = M + 4 * fd.z;
-            else
-                ph = thread_factor(fd);
-        }
-    };
-    // the same from the step itself (tileprog.h: kT2HphDirect, kT2HphShared)
+    // the run of a phased butterfly, from the step itself (tileprog.h)
     auto hph_direct = [&](const int4 w, const double2 *&T, double2 &ph) {
         const int trec = (int)((uint32_t)w.w & 0xffffu) - 1, row = (int)((uint32_t)w.w >> 16) - 1;
         const int sl = (int16_t)(w.y & 0xffff);
         T = trec >= 0 ? M + 4 * trec : ones;
         ph = make_double2(1.0, 0.0);
-        if (row >= 0) ph = row < kT2SmemRows ? rows[row * kDThreads + tid] : statc[(size_t)row * kDThreads + tid];
+        if (row >= 0) ph = static_row(row);
         if (sl >= 0) ph = cxd(ph, slotc[sl]);
     };
     const int nins = a.nins, last_stage = a.last_stage;
     for (int pc = 0; pc < nins; pc++) {
-        const int4 w = ins[pc];
+        const int4 w = ins(pc);
         const uint32_t qm = ~((uint32_t)w.y >> 24);  // all ones at run time, opaque to the compiler
         const double *mrec = reinterpret_cast<const double *>(M + 4 * w.w);
-        switch (((uint32_t)w.y >> 16) & 0xffu) {
+        const uint32_t hd = ((uint32_t)w.y >> 16) & 0xffu;
+        if constexpr ((F & 2) != 0) {  // real gates
+            if (hd == kT2HdRots) {
+                const uint32_t mask = (uint32_t)w.y & 31u, order = (uint32_t)w.z, sine = ((uint32_t)w.x >> 16) & 31u;
+#define SV_ROT(J)                                                       \
+    if (mask & (1u << J)) {                                             \
+        const double k = mrec[8 * ((order >> (3 * J)) & 7u) + 2];       \
+        if (sine & (1u << J))                                           \
+            d_rot<J, true>(r, k);                                       \
+        else                                                            \
+            d_rot<J, false>(r, k);                                      \
+    }
+                SV_ROT(0)
+                SV_ROT(1)
+                SV_ROT(2)
+                SV_ROT(3)
+                SV_ROT(4)
+#undef SV_ROT
+                continue;
+            }
+        }
+        if (hd == kT2HdTable) {
+            const uint32_t pb = (uint32_t)w.y & 0xfu;  // thread-bit predicate
+            if (!pb || ((tid >> (pb - 1)) & 1)) d_table(r, M + 4 * w.w, qm);
+            continue;
+        }
+        if (hd == kT2HdFactor) {
+            const int j = (w.x >> 16) & 0xff;
+            d_factor_bit(r, j ? 1 << (j - 1) : 0, thread_factor(w));
+            continue;
+        }
+        switch (hd) {
             case kT2HdStage: {
                 if (live) {
                     // every warp has read the previous layout before any overwrites it
@@ -437,7 +455,7 @@ __device__ __forceinline__ void t2d_run(const T2Args &a, double2 *gstate, uint64
                 continue;
             }
             case kT2HdScale: {
-                const double s = mrec[0];
+                const double s = __hiloint2double(w.w, w.z);
 #pragma unroll
                 for (int x = 0; x < kR; x++) {
                     r.re[x] *= s;
@@ -445,31 +463,12 @@ __device__ __forceinline__ void t2d_run(const T2Args &a, double2 *gstate, uint64
                 }
                 continue;
             }
-            case kT2HdDiag: {
-                const int e0 = (int16_t)(w.z & 0xffff), e1 = (int16_t)(w.z >> 16);
-                for (int e = e0; e < e1; e++) {
-                    const int4 fd = fac[e];
-                    const uint32_t w0 = (uint32_t)fd.x;
-                    if (w0 & kFacTable) {
-                        const int pb = (int)((w0 >> 10) & 0xfu);  // thread-bit predicate
-                        if (pb && !((tid >> (pb - 1)) & 1)) continue;
-                        d_table(r, M + 4 * fd.z, qm);
-                        continue;
-                    }
-                    d_factor_bit(r, (int)(w0 & 0xffu), thread_factor(fd));
-                }
-                continue;
-            }
 #define SV_HPH_CASE(J)                  \
     case kT2Handler + 8 * 5 + J: {      \
         const double2 *T;               \
         double2 ph;                     \
-        const int8_t hc = (int8_t)(w.x >> 24); \
-        if (hc == kT2HphDirect || hc == kT2HphShared) \
-            hph_direct(w, T, ph);       \
-        else                            \
-            hph_run(w, T, ph);          \
-        d_hph<J>(r, qm, T, T != ones, ph, hc == kT2HphShared); \
+        hph_direct(w, T, ph);           \
+        d_hph<J>(r, qm, T, T != ones, ph, (int8_t)(w.x >> 24) == kT2HphShared); \
         continue;                       \
     }
             SV_HPH_CASE(0)
@@ -552,16 +551,12 @@ __device__ __forceinline__ uint64_t tile_base_d(const T2Args &a, uint64_t tile) 
 }
 
 __device__ __forceinline__ void load_programme_d(const T2Args &a, unsigned char *sm, int tid, int nthreads) {
-    int4 *si = reinterpret_cast<int4 *>(sm + GD::kOffIns);
-    int4 *sf = reinterpret_cast<int4 *>(sm + GD::kOffFac);
     double2 *sr = reinterpret_cast<double2 *>(sm + GD::kOffRows);
     double2 *smat = reinterpret_cast<double2 *>(sm + GD::kOffMats);
     int4 *slay = reinterpret_cast<int4 *>(sm + GD::kOffLay);
     int4 *sepi = reinterpret_cast<int4 *>(sm + GD::kOffEpi);
     const double2 *mats = reinterpret_cast<const double2 *>(a.mats);
     const double2 *statc = reinterpret_cast<const double2 *>(a.statc);
-    for (int i = tid; i < a.nins; i += nthreads) si[i] = __ldg(a.ins + i);
-    for (int i = tid; i < a.nfac; i += nthreads) sf[i] = __ldg(a.fac + i);
     for (int i = tid; i < 4 * a.nmats; i += nthreads) smat[i] = __ldg(mats + i);
     const int nl = min(a.nstages, kT2SmemStages) * (int)(sizeof(T2LayoutX) / 16);
     for (int i = tid; i < nl; i += nthreads) slay[i] = __ldg(reinterpret_cast<const int4 *>(a.layx) + i);
@@ -606,7 +601,7 @@ __device__ __forceinline__ void tile_slots_d(const T2Args &a, double2 *slotc, ui
 template <int F>
 __global__ void __launch_bounds__(kDThreads, 1)
     k_tile2d(double2 *__restrict__ state, const T2Args a, const __grid_constant__ CUtensorMap map,
-             const __grid_constant__ TileBox box) {
+             const __grid_constant__ TileBox box, const __grid_constant__ T2Prog prog) {
     extern __shared__ __align__(1024) unsigned char sm[];
     double2 *slotc = reinterpret_cast<double2 *>(sm + GD::kOffSlotc);
     uint64_t *bar = reinterpret_cast<uint64_t *>(sm + GD::kOffBar);
@@ -651,7 +646,7 @@ __global__ void __launch_bounds__(kDThreads, 1)
                 issue_load(next_base);
             }
         };
-        t2d_run<F>(a, state, rbar, rd, base, sc, hook);
+        t2d_run<F>(a, [&](int pc) { return prog.ins[pc]; }, state, rbar, rd, base, sc, hook);
         parity ^= 1u;
         buf ^= 1u;
         base = next_base;
@@ -686,9 +681,11 @@ sv_status t2d_launch(sv_state *h, const T2Pass &p, const T2Device &d, const sv_l
     CUtensorMap map{};
     TileBox box{};
     if (!a.gen) SV_TRY(tile_map(h->amps, h->n, p.k, p.slot_phys, sizeof(double2), &map, &box));
+    T2Prog prog;
+    std::memcpy(prog.ins, p.dev.data(), p.dev.size() * sizeof(T2Ins));
     const int slot = prof_begin(h);
     kern<<<(unsigned)grid, kDThreads, GD::kSmemBytes, h->stream>>>(reinterpret_cast<double2 *>(h->amps), a, map,
-                                                                   box);
+                                                                   box, prog);
     SV_CUDA(cudaGetLastError());
     note_launch();
     prof_end(h, slot, meta);

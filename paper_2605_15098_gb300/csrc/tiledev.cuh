@@ -279,7 +279,6 @@ __device__ __forceinline__ void reg_h2(RegsN<NP> &r, uint32_t qm) {
     if constexpr (J >= 1) {
 #pragma unroll
         for (int g = 0; g < NP / 8; g++) {
-            if (!((qm >> g) & 1)) continue;
 #pragma unroll
             for (int i = 0; i < 4; i++) {
                 const int q = bfly_q<J>(4 * g + i), q1 = q | (1 << (J - 1));
@@ -292,7 +291,6 @@ __device__ __forceinline__ void reg_h2(RegsN<NP> &r, uint32_t qm) {
     } else {
 #pragma unroll
         for (int g4 = 0; g4 < NP / 4; g4++) {
-            if (!((qm >> g4) & 1)) continue;
 #pragma unroll
             for (int i = 0; i < 4; i++) {
                 const int q = 4 * g4 + i;
@@ -368,15 +366,13 @@ __device__ __forceinline__ void reg_u2(RegsN<NP> &r, uint32_t qm, const float *m
 
 // Rotation [[c, -s], [s, c]] (c >= 0) on register bit J as three in-place
 // shears: a += t b, b += s a, a += t b with t = -s / (1 + c) = (c - 1) / s
-// (m[0] = t, m[1] = s).  Their product is the rotation exactly; each shear
-// is one multiply-add per plane and no register of the pair is copied.
+// (exactly the rotation); each shear is one multiply-add per plane and no
+// register of the pair is copied.
 template <int J, int NP>
-__device__ __forceinline__ void reg_rot(RegsN<NP> &r, uint32_t qm, const float *m) {
-    const float t = m[0], s = m[1];
+__device__ __forceinline__ void reg_rot(RegsN<NP> &r, float t, float s) {
     if constexpr (J >= 1) {
 #pragma unroll
         for (int g = 0; g < NP / 8; g++) {
-            if (!((qm >> g) & 1)) continue;
 #pragma unroll
             for (int i = 0; i < 4; i++) {
                 const int q = bfly_q<J>(4 * g + i), q1 = q | (1 << (J - 1));
@@ -391,7 +387,6 @@ __device__ __forceinline__ void reg_rot(RegsN<NP> &r, uint32_t qm, const float *
     } else {
 #pragma unroll
         for (int g4 = 0; g4 < NP / 4; g4++) {
-            if (!((qm >> g4) & 1)) continue;
 #pragma unroll
             for (int i = 0; i < 4; i++) {
                 const int q = 4 * g4 + i;

@@ -206,8 +206,30 @@ struct T2SlotTerm64 {
 };
 
 // Handler codes of the non-gate steps (format 2), in the same field as the
-// gate handlers: the kernel dispatches every step with one switch.
+// gate handlers.
 constexpr int kT2HdStage = 1, kT2HdScale = 2, kT2HdDiag = 3;
+
+// The device form of a format-2 programme (T2Pass::dev), made from its steps
+// by the stage compiler.  A step cost the kernel some 30 instructions before
+// its arithmetic (fetch, decode, a chain of branches), against 48 for a
+// rotation's and 32 or 64 for a diagonal factor's, so:
+//  * consecutive rotations on distinct register bits are one step (Rots):
+//    cidx = their register bits as a mask, e0 = three bits per register bit:
+//    its record, counted from record `aux` (the records are consecutive);
+//    complex128: idx = the bits whose rotation is divided by its sine, below;
+//  * a diagonal run is one step per factor, with the factor's record in the
+//    step: Table (aux = first matrix record, cidx = thread-bit predicate) and
+//    Factor (idx = 1 + register bit or 0, cidx = slot, e0 = static row,
+//    e1 = slot of the lowest dynamic thread bit, aux = dynamic thread bits;
+//    -1 = none);
+//  * Scale holds its factor: complex64 hi in aux and lo in (e0, e1) as FP32
+//    bits, complex128 an FP64 with aux its high word.
+// complex128 rotations run unnormalised, [[1, -k], [k, 1]] with k = s / c or
+// [[k, -1], [1, k]] with k = c / s, whichever has |k| <= 1: two multiply-adds
+// per pair and component instead of three (the FP64 pipe bounds that kernel);
+// the product of the divisors joins the closing scale.
+constexpr int kT2HdRots = 4, kT2HdTable = 5, kT2HdFactor = 6;
+constexpr int kT2DevIns = 256;  // at most kT2SmemIns steps and kT2SmemFactors factors
 
 // Write-back offsets of the final layout in the global state (amplitudes),
 // relative to the tile's base: lane bits, warp bits and register bits 1..
