@@ -217,17 +217,22 @@ size_t t2_smem_bytes();
 // kernel instantiation.
 int t2_gate_kinds(const T2Pass &p);
 sv_status t2_prepare(sv_state *h);
+// Compute the slot values of these passes (n-qubit state) into out[i].
+sv_status t2_slotv(sv_state *h, const std::vector<std::pair<const T2Pass *, T2Device>> &passes,
+                   const std::vector<void *> &out);
 // gen_basis >= 0: the state is that basis state and the pass generates it
-// instead of reading the buffer.
+// instead of reading the buffer.  slotv: the pass's slot values where
+// t2_slotv computed them already, else NULL.  after_tile: the stream's last
+// operation is a register-stage pass of this call.
 sv_status t2_launch(sv_state *h, const T2Pass &p, const T2Device &d, const sv_launch_record &meta,
-                    int64_t gen_basis = -1);
+                    int64_t gen_basis = -1, const void *slotv = nullptr, bool after_tile = false);
 // The generated-state fields of a first pass that starts from the product
 // state H^{basis_h}|gen_basis> (physical qubit masks).
 void t2_set_gen(const T2Pass &p, int64_t gen_basis, uint64_t basis_h, T2Args *a);
 // The complex128 register-stage kernel (tile2d.cu): a pass compiled by
 // compile_t2v2_c128; gen_basis as for t2_launch.  Needs h->tab64.
 sv_status t2d_launch(sv_state *h, const T2Pass &p, const T2Device &d, const sv_launch_record &meta,
-                     int64_t gen_basis = -1);
+                     int64_t gen_basis = -1, bool after_tile = false);
 // One launch running the passes of an L2 block group (complex64, 2^13 tiles);
 // `need`: the gate kinds (t2_gate_kinds) of all its passes.
 sv_status t2_group_launch(sv_state *h, const GroupArgs &g, int need, const sv_launch_record &meta);

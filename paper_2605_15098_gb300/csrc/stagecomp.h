@@ -137,6 +137,23 @@ struct T2Prog {
 constexpr size_t kSlotvMaxBytes = (size_t)256 << 20;
 size_t t2_slotv_bytes(const T2Pass &p, int n);
 
+// The slot values of several passes computed in one launch (k_slotv).
+struct SlotJob {
+    uint64_t ntiles;
+    int nsp, nslots, ngr;
+    int8_t gs[32], gd[32], gl[32];
+    const int32_t *soff;
+    const T2SlotTerm *sterms;
+    float2 *out;
+};
+constexpr int kSlotJobs = 16;
+struct SlotJobs {
+    SlotJob job[kSlotJobs];
+};
+// Slot values of all passes of a call up to this many bytes: one launch before
+// the first pass; more: one per pass, into one buffer.
+constexpr size_t kSlotvTogether = (size_t)64 << 20;
+
 // Fill the counts, pointers and geometry of a format-2 pass (not gen,
 // tables or err).
 void t2_fill_args(const T2Pass &p, const T2Device &d, int n, T2Args *a);

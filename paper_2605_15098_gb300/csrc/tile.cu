@@ -352,10 +352,24 @@ struct PassUpload {
 
 constexpr size_t kPlanCacheEntries = 8;
 
-// 64-bit FNV-1a
-uint64_t fnv1a(const void *p, size_t n, uint64_t h = 0xcbf29ce484222325ull) {
+// FNV-1a's step on 64-bit words, in four lanes (a gate list is tens of
+// kilobytes; byte by byte its hash took longer than the rest of the host's
+// work for a cached programme: 30 us for QPE n = 20).  It only picks the cache
+// entries whose keys are compared.
+uint64_t key_hash(const void *p, size_t n) {
     const unsigned char *b = static_cast<const unsigned char *>(p);
-    for (size_t i = 0; i < n; i++) h = (h ^ b[i]) * 0x100000001b3ull;
+    uint64_t lane[4] = {0xcbf29ce484222325ull, 0x84222325cbf29ce4ull, 0x9e3779b97f4a7c15ull, n};
+    size_t i = 0;
+    for (; i + 32 <= n; i += 32)
+        for (int l = 0; l < 4; l++) {
+            uint64_t w;
+            std::memcpy(&w, b + i + 8 * l, 8);
+            lane[l] = (lane[l] ^ w) * 0x100000001b3ull;
+            lane[l] ^= lane[l] >> 29;
+        }
+    for (; i < n; i++) lane[0] = (lane[0] ^ b[i]) * 0x100000001b3ull;
+    uint64_t h = 0xcbf29ce484222325ull;
+    for (uint64_t l : lane) h = (h ^ l) * 0x100000001b3ull;
     return h;
 }
 
@@ -451,6 +465,7 @@ static int l2_cap(const sv_state *h, const sv_config &cfg) {
 static std::string plan_key(const sv_state *h, const std::vector<sv_gate> &gates, const sv_config &cfg,
                             const PlanOptions &opt, const PlanOverride *ov) {
     std::string k;
+    k.reserve(gates.size() * sizeof(sv_gate) + 1024);
     auto put = [&](const void *p, size_t n) { k.append(static_cast<const char *>(p), n); };
     const int head[] = {h->n, (int)h->dt, cfg.mode, (int)cfg.flags, opt.n, opt.k, opt.c,
                         opt.merge_diag, opt.relabel, opt.paper, opt.split_u3, opt.late_diag,
@@ -473,7 +488,7 @@ static sv_status compiled_plan(sv_state *h, const std::vector<sv_gate> &gates, c
     PlanOptions opt = ov ? ov->opt : plan_options(h->n, h->dt, cfg);
     if (dbl && opt.k > 13) return fail(SV_ERR_ARG, "complex128 tiles hold at most 2^13 amplitudes");
     std::string key = plan_key(h, gates, cfg, opt, ov);
-    const uint64_t hash = fnv1a(key.data(), key.size());
+    const uint64_t hash = key_hash(key.data(), key.size());
     const bool use_cache = !(cfg.flags & SV_FLAG_NO_PLAN_CACHE);
     for (size_t i = 0; use_cache && i < h->plan_cache.size(); i++) {
         const auto &e = h->plan_cache[i];
@@ -722,13 +737,22 @@ sv_status partitioned_apply(sv_state *h, const std::vector<sv_gate> &gates, cons
     }
     if (any_t2) SV_TRY(t2_prepare(h));
     if (any_t2 && dbl) SV_TRY(tab64_prepare(h));
-    if (any_t2 && !dbl) {  // the per-tile slot values of the one-level register-stage passes
+    // the per-tile slot values of the one-level register-stage passes: all of
+    // them before the first pass, or one pass's at a time
+    std::vector<size_t> slot_off(up.size(), 0);
+    size_t slots_together = 0;
+    if (any_t2 && !dbl) {
         size_t need = 0;
         for (size_t i = 0; i < up.size(); i++) {
             if (!up[i].t2 || up[i].t3 || cp->group_at[i] >= 0) continue;
-            need = std::max(need, t2_slotv_bytes(t2[i], h->n));
-            if (t2[i].genv) need = std::max(need, t2_slotv_bytes(*t2[i].genv, h->n));
+            size_t most = t2_slotv_bytes(t2[i], h->n);
+            if (t2[i].genv) most = std::max(most, t2_slotv_bytes(*t2[i].genv, h->n));
+            slot_off[i] = slots_together;
+            slots_together += (most + 255) & ~(size_t)255;
+            need = std::max(need, most);
         }
+        if (slots_together <= kSlotvTogether) need = slots_together;
+        else slots_together = 0;
         if (need > h->slotv_cap) {
             if (h->slotv) {
                 SV_CUDA(cudaStreamSynchronize(h->stream));
@@ -745,18 +769,25 @@ sv_status partitioned_apply(sv_state *h, const std::vector<sv_gate> &gates, cons
         }
     }
     if (any_t3) SV_TRY(t3_prepare(h));
+    bool slots_done = false;
+    bool after_tile = false;  // the stream's last operation is a register-stage pass of this call
 
     for (size_t i = 0; i < plan.passes.size(); i++) {
         const TilePass &p = plan.passes[i];
         if (!p.general.empty()) {  // a gate of the general set, on the per-gate path
             SV_TRY(general_apply(h, p.general.data()));
+            after_tile = false;
             continue;
         }
-        if (!p.remap_before.empty()) SV_TRY(remap_apply(h, p.remap_before));
+        if (!p.remap_before.empty()) {
+            SV_TRY(remap_apply(h, p.remap_before));
+            after_tile = false;
+        }
         if (p.ops.empty()) continue;
         if (cp->group_at[i] >= 0) {  // an L2 block group: its passes in one launch
             const int gi = cp->group_at[i];
             SV_TRY(group_apply(h, *cp, gi));
+            after_tile = false;
             i += (size_t)cp->groups[gi].count - 1;
             continue;
         }
@@ -764,7 +795,10 @@ sv_status partitioned_apply(sv_state *h, const std::vector<sv_gate> &gates, cons
                                               up[i].t3 ? PK_T3 : up[i].t2 ? PK_T2 : PK_GENERIC);
         meta.pass = h->launch_index++;
         sv_status st;
-        if (!up[i].t3) SV_TRY(resolve_norm(h));
+        if (!up[i].t3) {
+            if (h->norm_pending) after_tile = false;
+            SV_TRY(resolve_norm(h));
+        }
         // a recorded basis state: the register-stage kernel generates it in
         // its first pass; every other kernel needs it written out first
         int64_t gen = -1;
@@ -775,15 +809,36 @@ sv_status partitioned_apply(sv_state *h, const std::vector<sv_gate> &gates, cons
                 meta.generated = 1;
             } else {
                 SV_TRY(materialize(h));
+                after_tile = false;
             }
         }
         if (up[i].t2) {
             const bool g = gen >= 0;
+            if (slots_together && !slots_done && !up[i].t3) {
+                // only this pass can be generated: every later one reads the state
+                std::vector<std::pair<const T2Pass *, T2Device>> jobs;
+                std::vector<void *> out;
+                for (size_t j = i; j < up.size(); j++) {
+                    if (!up[j].t2 || up[j].t3 || cp->group_at[j] >= 0) continue;
+                    const bool gj = g && j == i;
+                    const T2Pass &tp = gj ? *t2[j].genv : t2[j];
+                    if (!t2_slotv_bytes(tp, h->n)) continue;
+                    jobs.push_back({&tp, t2_device(dev, gj ? up[j].gen : up[j].main)});
+                    out.push_back(static_cast<char *>(h->slotv) + slot_off[j]);
+                }
+                if (!jobs.empty()) SV_TRY(t2_slotv(h, jobs, out));
+                slots_done = true;
+                after_tile = false;
+            }
+            const void *sv = slots_done && t2_slotv_bytes(g ? *t2[i].genv : t2[i], h->n)
+                                 ? static_cast<char *>(h->slotv) + slot_off[i]
+                                 : nullptr;
             T2Device d = t2_device(dev, g ? up[i].gen : up[i].main);
             d.blocks = up[i].t3 ? reinterpret_cast<const float *>(dev + up[i].blocks) : nullptr;
             st = up[i].t3 ? t3_launch(h, t2[i], d, meta)
-                 : dbl    ? t2d_launch(h, g ? *t2[i].genv : t2[i], d, meta, gen)
-                          : t2_launch(h, g ? *t2[i].genv : t2[i], d, meta, gen);
+                 : dbl    ? t2d_launch(h, g ? *t2[i].genv : t2[i], d, meta, gen, after_tile)
+                          : t2_launch(h, g ? *t2[i].genv : t2[i], d, meta, gen, sv, after_tile);
+            after_tile = !up[i].t3;
             if (st == SV_OK && gen >= 0) {
                 h->basis = -1;
                 h->basis_h = 0;
@@ -807,6 +862,7 @@ sv_status partitioned_apply(sv_state *h, const std::vector<sv_gate> &gates, cons
                 a.tab64 = reinterpret_cast<const double2 *>(h->tab64);
             }
             st = dbl ? launch_pass<double>(h, a, meta) : launch_pass<float>(h, a, meta);
+            after_tile = false;
         }
         if (st != SV_OK) return st;
         h->stats.passes++;

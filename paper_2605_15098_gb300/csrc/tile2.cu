@@ -608,7 +608,8 @@ __device__ __forceinline__ void t2_run(const T2Args &a, Ins ins, float4 *gstate,
 
 // Physical base index of tile `tile`: its index bits spread over the runs of
 // the global qubits.
-__device__ __forceinline__ uint64_t tile_base(const T2Args &a, uint64_t tile) {
+template <typename A>
+__device__ __forceinline__ uint64_t tile_base(const A &a, uint64_t tile) {
     uint64_t b = 0;
     for (int i = 0; i < a.ngr; i++)
         b |= ((tile >> a.gs[i]) & ((UINT64_C(1) << a.gl[i]) - 1)) << a.gd[i];
@@ -687,10 +688,10 @@ __device__ __forceinline__ void tile_slots(const T2Args &a, const float2 *tab, f
 
 // The slot values of every tile of a pass (the same sums and table products
 // as tile_slots, one thread per tile and slot), computed before the pass so
-// that its tiles receive them with their bulk copies.
-__global__ void k_slotv(const T2Args a, float2 *__restrict__ out) {
+// that its tiles receive them with their bulk copies; blockIdx.y: the pass.
+__global__ void k_slotv(const __grid_constant__ SlotJobs jobs, const float2 *__restrict__ tab) {
+    const SlotJob &a = jobs.job[blockIdx.y];
     const uint64_t total = a.ntiles * (uint64_t)a.nsp;
-    const float2 *tab = a.tables;
     for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total;
          i += (uint64_t)gridDim.x * blockDim.x) {
         const uint64_t tile = i / (uint64_t)a.nsp;
@@ -709,7 +710,7 @@ __global__ void k_slotv(const T2Args a, float2 *__restrict__ out) {
             v = cx(cx(__ldg(tab + (u >> 24)), __ldg(tab + kTabN + ((u >> 16) & 255u))),
                    cx(__ldg(tab + 2 * kTabN + ((u >> 8) & 255u)), __ldg(tab + 3 * kTabN + (u & 255u))));
         }
-        out[i] = v;
+        a.out[i] = v;
     }
 }
 
@@ -751,6 +752,10 @@ __global__ void __launch_bounds__(Geo<K>::kThreads, K == kT2Qubits ? 2 : 1)
         fence_mbar_init();
     }
     __syncthreads();
+    // what the CTA has read so far (tables, programme) was there before the
+    // previous pass started; the state and the slot values are that pass's
+    let_next_start();
+    wait_previous();
     // precomputed slot values: tile t's arrive with its copies (a pass that
     // generates its state copies only them), into the slot buffer the previous
     // tile did not use
@@ -1330,8 +1335,39 @@ void t2_set_gen(const T2Pass &p, int64_t gen_basis, uint64_t basis_h, T2Args *a)
     a->gen_val = (float)a->gen_val64;
 }
 
+sv_status t2_slotv(sv_state *h, const std::vector<std::pair<const T2Pass *, T2Device>> &passes,
+                   const std::vector<void *> &out) {
+    for (size_t i = 0; i < passes.size();) {
+        SlotJobs jobs{};
+        uint64_t most = 0;
+        int count = 0;
+        for (; i < passes.size() && count < kSlotJobs; i++, count++) {
+            T2Args a{};
+            t2_fill_args(*passes[i].first, passes[i].second, h->n, &a);
+            SlotJob &j = jobs.job[count];
+            j.ntiles = a.ntiles;
+            j.nslots = a.nslots;
+            j.nsp = (a.nslots + 1) & ~1;
+            j.ngr = a.ngr;
+            std::memcpy(j.gs, a.gs, sizeof j.gs);
+            std::memcpy(j.gd, a.gd, sizeof j.gd);
+            std::memcpy(j.gl, a.gl, sizeof j.gl);
+            j.soff = a.soff;
+            j.sterms = a.sterms;
+            j.out = reinterpret_cast<float2 *>(out[i]);
+            most = std::max<uint64_t>(most, j.ntiles * (uint64_t)j.nsp);
+        }
+        const unsigned blocks = (unsigned)std::min<uint64_t>((most + 255) / 256, (uint64_t)h->sm_count * 8);
+        k_slotv<<<dim3(blocks, (unsigned)count), 256, 0, h->stream>>>(
+            jobs, reinterpret_cast<const float2 *>(h->t2_tables));
+        SV_CUDA(cudaGetLastError());
+        note_launch();
+    }
+    return SV_OK;
+}
+
 sv_status t2_launch(sv_state *h, const T2Pass &p, const T2Device &d, const sv_launch_record &meta,
-                    int64_t gen_basis) {
+                    int64_t gen_basis, const void *slotv, bool after_tile) {
     if (p.format != 2) return fail(SV_ERR_ARG, "internal: register-stage pass not in format 2");
     SV_TRY(launch_check());
     T2Args a{};
@@ -1340,17 +1376,18 @@ sv_status t2_launch(sv_state *h, const T2Pass &p, const T2Device &d, const sv_la
     a.tables = reinterpret_cast<const float2 *>(h->t2_tables);
     a.err = h->t2_err;
     if (p.k != 13 && p.k != 14) return fail(SV_ERR_ARG, "internal: register-stage tile of 2^%d", p.k);
-    // the tiles' slot values, computed ahead into the handle's buffer (sized
-    // by t2_slotv_bytes before the first launch of the call)
+    // the tiles' slot values, computed ahead: before the call's first pass, or
+    // now into the handle's buffer (sized by t2_slotv_bytes before the first
+    // launch of the call)
     const size_t sbytes = t2_slotv_bytes(p, h->n);
-    if (sbytes && sbytes <= h->slotv_cap) {
+    if (sbytes && !slotv && sbytes <= h->slotv_cap) {
+        SV_TRY(t2_slotv(h, {{&p, d}}, {h->slotv}));
+        slotv = h->slotv;
+        after_tile = false;
+    }
+    if (slotv) {
         a.nsp = (int)((p.slots.size() + 1) & ~(size_t)1);
-        a.slotv = reinterpret_cast<const float2 *>(h->slotv);
-        const uint64_t total = a.ntiles * (uint64_t)a.nsp;
-        const unsigned blocks = (unsigned)std::min<uint64_t>((total + 255) / 256, (uint64_t)h->sm_count * 8);
-        k_slotv<<<blocks, 256, 0, h->stream>>>(a, reinterpret_cast<float2 *>(h->slotv));
-        SV_CUDA(cudaGetLastError());
-        note_launch();
+        a.slotv = reinterpret_cast<const float2 *>(slotv);
     }
     // the smallest instantiation whose gate kinds cover the programme
     const int need = t2_gate_kinds(p);
@@ -1376,8 +1413,8 @@ sv_status t2_launch(sv_state *h, const T2Pass &p, const T2Device &d, const sv_la
     T2Prog prog;
     std::memcpy(prog.ins, p.dev.data(), p.dev.size() * sizeof(T2Ins));
     const int slot = prof_begin(h);
-    kern<<<(unsigned)grid, threads, smem, h->stream>>>(reinterpret_cast<float *>(h->amps), a, map, box, prog);
-    SV_CUDA(cudaGetLastError());
+    SV_CUDA(launch_after(kern, (unsigned)grid, threads, smem, h->stream, after_tile && slot < 0,
+                         reinterpret_cast<float *>(h->amps), a, map, box, prog));
     note_launch();
     prof_end(h, slot, meta);
     h->stats.kernels++;

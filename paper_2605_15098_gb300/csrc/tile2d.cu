@@ -614,6 +614,9 @@ __global__ void __launch_bounds__(kDThreads, 1)
         fence_mbar_init();
     }
     __syncthreads();
+    // what the CTA has read so far was there before the previous pass started
+    let_next_start();
+    wait_previous();
     // the copies of the tile whose global bits are b, by warp 0 (in 8-byte
     // words: an amplitude is two)
     auto issue_load = [&](uint64_t b) {
@@ -656,7 +659,7 @@ __global__ void __launch_bounds__(kDThreads, 1)
 }  // namespace
 
 sv_status t2d_launch(sv_state *h, const T2Pass &p, const T2Device &d, const sv_launch_record &meta,
-                     int64_t gen_basis) {
+                     int64_t gen_basis, bool after_tile) {
     if (p.format != 2 || !p.wide || p.k != kT2Qubits)
         return fail(SV_ERR_ARG, "internal: complex128 register-stage pass not compiled for it");
     SV_TRY(launch_check());
@@ -684,9 +687,8 @@ sv_status t2d_launch(sv_state *h, const T2Pass &p, const T2Device &d, const sv_l
     T2Prog prog;
     std::memcpy(prog.ins, p.dev.data(), p.dev.size() * sizeof(T2Ins));
     const int slot = prof_begin(h);
-    kern<<<(unsigned)grid, kDThreads, GD::kSmemBytes, h->stream>>>(reinterpret_cast<double2 *>(h->amps), a, map,
-                                                                   box, prog);
-    SV_CUDA(cudaGetLastError());
+    SV_CUDA(launch_after(kern, (unsigned)grid, kDThreads, GD::kSmemBytes, h->stream, after_tile && slot < 0,
+                         reinterpret_cast<double2 *>(h->amps), a, map, box, prog));
     note_launch();
     prof_end(h, slot, meta);
     h->stats.kernels++;
