@@ -316,14 +316,14 @@ struct SmemIns {
     __device__ int4 operator()(int pc) const { return reinterpret_cast<const int4 *>(t2_dyn_smem + G13::kOffIns)[pc]; }
 };
 
-// `rbar`: mbarrier that every warp arrives at once it has read a stage's
-// layout from shared memory (count: the CTA's warps); `rd` counts this
-// thread's arrivals.  A stage change waits for the phase of the previous read
-// before it overwrites the tile, so no warp overwrites data another warp has
-// not read yet, without a CTA barrier.  `base`: the tile's physical base
-// index; `slotc`: the tile's slot values.  After the last stage change has
-// read shared memory, `hook()` runs (the callers start the next tile's bulk
-// copies there, once rbar shows every warp's reads done).
+// `rbar`: mbarrier that every warp arrives at once it has read the last
+// stage's layout from shared memory (count: the CTA's warps); `rd` counts this
+// thread's arrivals.  `base`: the tile's physical base index; `slotc`: the
+// tile's slot values.  Then `hook()` runs (the callers start the next tile's
+// copies there, once rbar shows every warp's reads done).  A stage change
+// stores the tile, passes a barrier and loads it in the new layout; a thread
+// stores to the places it loaded from, so nothing waits before the stores, and
+// between layouts with the same warp bits the barrier is the warp's own.
 template <int K, int F, typename Ins, typename Hook>
 __device__ __forceinline__ void t2_run(const T2Args &a, Ins ins, float4 *gstate, uint64_t *rbar, uint32_t &rd,
                                        uint64_t base, const float2 *slotc, Hook hook) {
@@ -414,14 +414,17 @@ __device__ __forceinline__ void t2_run(const T2Args &a, Ins ins, float4 *gstate,
         }
         switch (hd) {
             case kT2HdStage: {
+                const bool local = (w.y & 1) != 0;  // within the warps (tileprog.h)
                 if (live) {
-                    // every warp has read the previous layout before any overwrites it
-                    if (!mbar_wait(rbar, (rd - 1u) & 1u)) atomicExch(a.err, 1);
+                    // a thread overwrites what it read itself; only the first
+                    // stage's read, in linear order, is another lane's
+                    __syncwarp();
                     const LayoutS L = layout_s(stage);
 #pragma unroll
                     for (int q = 0; q < kNP2; q++)
                         tile4[L.idx(q)] = make_float4(r.re[q].x, r.re[q].y, r.im[q].x, r.im[q].y);
-                    __syncthreads();
+                    if (local) __syncwarp();
+                    else __syncthreads();
                     stage = w.w;
                     const LayoutS L2 = layout_s(stage);
 #pragma unroll
@@ -480,10 +483,12 @@ __device__ __forceinline__ void t2_run(const T2Args &a, Ins ins, float4 *gstate,
                     }
                 }
                 live = true;
-                __syncwarp();
-                if ((tid & 31) == 0) mbar_arrive(rbar);
-                rd++;
-                if (pc == last_stage) hook();
+                if (pc == last_stage) {  // the next tile's copies wait for these reads
+                    __syncwarp();
+                    if ((tid & 31) == 0) mbar_arrive(rbar);
+                    rd++;
+                    hook();
+                }
                 continue;
             }
             case kT2HdScale: {

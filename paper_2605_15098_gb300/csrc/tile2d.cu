@@ -406,13 +406,16 @@ __device__ __forceinline__ void t2d_run(const T2Args &a, Ins ins, double2 *gstat
         }
         switch (hd) {
             case kT2HdStage: {
+                const bool local = (w.y & 1) != 0;  // within the warps (tileprog.h)
                 if (live) {
-                    // every warp has read the previous layout before any overwrites it
-                    if (!mbar_wait(rbar, (rd - 1u) & 1u)) atomicExch(a.err, 1);
+                    // a thread overwrites what it read itself; only the first
+                    // stage's read, in linear order, is another lane's
+                    __syncwarp();
                     const LaySD L(layout(stage), tid);
 #pragma unroll
                     for (int x = 0; x < kR; x++) tile[L.idx(x)] = make_double2(r.re[x], r.im[x]);
-                    __syncthreads();
+                    if (local) __syncwarp();
+                    else __syncthreads();
                     stage = w.w;
                     const LaySD L2(layout(stage), tid);
 #pragma unroll
@@ -448,10 +451,12 @@ __device__ __forceinline__ void t2d_run(const T2Args &a, Ins ins, double2 *gstat
                     }
                 }
                 live = true;
-                __syncwarp();
-                if ((tid & 31) == 0) mbar_arrive(rbar);
-                rd++;
-                if (pc == last_stage) hook();
+                if (pc == last_stage) {  // the next tile's copies wait for these reads
+                    __syncwarp();
+                    if ((tid & 31) == 0) mbar_arrive(rbar);
+                    rd++;
+                    hook();
+                }
                 continue;
             }
             case kT2HdScale: {

@@ -222,6 +222,8 @@ constexpr int kT2HdStage = 1, kT2HdScale = 2, kT2HdDiag = 3;
 //    Factor (idx = 1 + register bit or 0, cidx = slot, e0 = static row,
 //    e1 = slot of the lowest dynamic thread bit, aux = dynamic thread bits;
 //    -1 = none);
+//  * Stage: cidx = 1: the change stays within the warps (the layouts before and
+//    after have the same warp bits);
 //  * Scale holds its factor: complex64 hi in aux and lo in (e0, e1) as FP32
 //    bits, complex128 an FP64 with aux its high word.
 // complex128 rotations run unnormalised, [[1, -k], [k, 1]] with k = s / c or
