@@ -258,8 +258,9 @@ sv_status sv_batch_create(const sv_batch_item *items, size_t count, const sv_con
     Blob blob;
     std::vector<BatchInst> inst(count);
     std::vector<T2Args> pass;
-    struct Off { size_t ins, stages, mats, fac, statc, soff, sterms, layx, epi; };
+    struct Off { size_t ins, stages, mats, statc, soff, sterms, layx, epi; };
     std::vector<Off> offs;
+    std::vector<std::pair<const T2Pass *, size_t>> pass_of;  // each pass's programme and item
     std::vector<double> cost(count);
     uint64_t amps = 0;
     for (size_t i = 0; i < count; i++) {
@@ -293,6 +294,7 @@ sv_status sv_batch_create(const sv_batch_item *items, size_t count, const sv_con
             o.soff = blob.put(t2.soff.data(), t2.soff.size() * sizeof(int32_t));
             o.sterms = blob.put(t2.sterms.data(), t2.sterms.size() * sizeof(T2SlotTerm));
             pass.push_back(a);
+            pass_of.push_back({&t2, i});
             offs.push_back(o);
             b->total_passes++;
             b->sweep_bytes += 2.0 * 8.0 * (double)(UINT64_C(1) << cp.nphys);
@@ -321,12 +323,27 @@ sv_status sv_batch_create(const sv_batch_item *items, size_t count, const sv_con
     const size_t inst_off = blob.put(inst.data(), inst.size() * sizeof(BatchInst));
     const size_t work_off = blob.put(items4.data(), items4.size() * sizeof(int4));
     const size_t pass_off = blob.put(nullptr, pass.size() * sizeof(T2Args));
+    const size_t map_off = blob.put(nullptr, pass.size() * sizeof(CUtensorMap));
     blob.put(nullptr, 0);
     if (dev_malloc(&b->prog, blob.b.size() + 256) != cudaSuccess) {
         cudaGetLastError();
         return bail(fail(SV_ERR_OOM, "cannot allocate the batch programme (%zu bytes)", blob.b.size()));
     }
     const char *dev = reinterpret_cast<const char *>(b->prog);
+    if (dev_malloc(&b->states, amps * 8) != cudaSuccess) {
+        cudaGetLastError();
+        return bail(fail(SV_ERR_OOM, "cannot allocate batch states (%llu amplitudes)", (unsigned long long)amps));
+    }
+    std::vector<CUtensorMap> maps(pass.size());
+    for (size_t p = 0; p < pass.size(); p++) {
+        pass[p].map = reinterpret_cast<const CUtensorMap *>(dev + map_off) + p;
+        if (pass[p].gen) continue;  // reads nothing
+        const size_t i = pass_of[p].second;
+        const sv_status ts = tile_map(static_cast<char *>(static_cast<void *>(b->states)) + inst[i].state_off * 8,
+                                      inst[i].nphys, kT2Qubits, pass_of[p].first->slot_phys, 8, &maps[p], &pass[p].box);
+        if (ts != SV_OK) return bail(ts);
+    }
+    std::memcpy(blob.b.data() + map_off, maps.data(), maps.size() * sizeof(CUtensorMap));
     {
         const sv_status ts = t2_build_tables(&b->tables, &b->err, b->stream);
         if (ts != SV_OK) return bail(ts);
@@ -350,14 +367,13 @@ sv_status sv_batch_create(const sv_batch_item *items, size_t count, const sv_con
     }
     b->state_amps = amps;
     b->queue_bytes = 256 + pass.size() * sizeof(unsigned);
-    if (dev_malloc(&b->states, amps * 8) != cudaSuccess || dev_malloc(&b->queue, b->queue_bytes) != cudaSuccess ||
+    if (dev_malloc(&b->queue, b->queue_bytes) != cudaSuccess ||
         dev_malloc(&b->out_idx, count * sizeof(uint64_t)) != cudaSuccess ||
         dev_malloc(&b->out_p, count * sizeof(double)) != cudaSuccess ||
         cudaMallocHost(&b->h_idx, count * sizeof(uint64_t)) != cudaSuccess ||
         cudaMallocHost(&b->h_p, count * sizeof(double)) != cudaSuccess) {
         cudaGetLastError();
-        return bail(fail(SV_ERR_OOM, "cannot allocate batch states (%llu amplitudes)",
-                         (unsigned long long)amps));
+        return bail(fail(SV_ERR_OOM, "cannot allocate the batch queue and results"));
     }
     BatchArgs args{};
     args.inst = reinterpret_cast<const BatchInst *>(dev + inst_off);

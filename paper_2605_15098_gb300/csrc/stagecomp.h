@@ -9,6 +9,7 @@
 
 #include "l2group.h"
 #include "plan.h"
+#include "tilemap.h"
 #include "tileprog.h"
 
 namespace sv {
@@ -85,7 +86,10 @@ struct T2Args {
     int c, nins;
     int nrows, nslots, nmats, nstages;  // static rows, slots, matrix records, stages
     int last_stage;  // index of the last T2_STAGE instruction
-    int slot_phys[kMaxTileQubits];
+    // the tile's copies (tilemap.h): the tensor map, in global or parameter
+    // memory, and the box coordinates; unused by a pass that generates its state
+    const CUtensorMap *map;
+    TileBox box;
     // the tile's physical base index: tile index bits [gs[r], gs[r] + gl[r])
     // go to physical bits gd[r].. (runs of the global bits)
     int ngr;
@@ -166,6 +170,7 @@ bool t2_block_runs(T2Args *a, uint64_t gmask, uint64_t bmask, int n);
 
 // One launch of an L2 block group: its passes' arguments and the claim order.
 struct GroupArgs {
+    CUtensorMap map[kMaxGroupPasses];
     T2Args pass[kMaxGroupPasses];
     const uint32_t *segs;       // (block << 3) | pass, in claim order
     uint64_t nitems;            // segments x tiles per block

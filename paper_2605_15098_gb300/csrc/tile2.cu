@@ -2,10 +2,8 @@
 // programmes in format 2 (tileprog.h).
 //
 // Per tile (persistent grid, two CTAs per SM, 256 threads each, 32 amplitudes per thread):
-//   1. one warp copies the tile into shared memory (TMA), completing on an
-//      mbarrier: k_tile2 by one to a few tensor copies (tilemap.h), the L2
-//      block and batched kernels by 2^(13-c) bulk copies of its contiguous
-//      2^c-amplitude chunks;
+//   1. one warp copies the tile into shared memory by one to a few tensor
+//      copies (TMA; tilemap.h), completing on an mbarrier;
 //   2. the pass's per-tile diagonal data (global-qubit contributions, which
 //      are constants of the tile: Sec. III-B of arxiv 2605.15098) is summed
 //      as integer phases while the copies are in flight, then turned into the
@@ -621,15 +619,12 @@ __device__ __forceinline__ uint64_t tile_base(const A &a, uint64_t tile) {
     return b;
 }
 
-// The tile's bulk copies (warp 0); with `slots` the tile's precomputed slot
-// values come on the same barrier.
+// The copies of the tile whose global bits are `base` (warp 0); with `slots`
+// the precomputed slot values of tile `tile` come on the same barrier.
 template <int K>
-__device__ __forceinline__ void issue_tile_load(const T2Args &a, unsigned char *sm, const float *state,
-                                                uint64_t tile, uint64_t *bar, int tid,
+__device__ __forceinline__ void issue_tile_load(const T2Args &a, const CUtensorMap *map, unsigned char *sm,
+                                                uint64_t tile, uint64_t base, uint64_t *bar, int tid,
                                                 float2 *slots = nullptr) {
-    const int nchunks = 1 << (K - a.c);
-    const uint32_t chunk_bytes = 8u << a.c;
-    const uint64_t base = tile_base(a, tile);
     if (tid == 0) {
         fence_async_smem();
         const uint32_t sb = slots ? (uint32_t)a.nsp * 8u : 0u;
@@ -637,12 +632,7 @@ __device__ __forceinline__ void issue_tile_load(const T2Args &a, unsigned char *
         if (slots) bulk_g2s(slots, a.slotv + tile * (uint64_t)a.nsp, sb, bar);
     }
     __syncwarp();
-    for (int j = tid; j < nchunks; j += 32) {
-        uint64_t off = 0;
-        for (int b = 0; b < K - a.c; b++)
-            if ((j >> b) & 1) off |= UINT64_C(1) << a.slot_phys[a.c + b];
-        bulk_g2s(sm + (size_t)j * chunk_bytes, state + 2 * (base + off), chunk_bytes, bar);
-    }
+    tensor_tile_load(map, a.box, base, sm, bar, tid);
 }
 
 // The pass's programme into shared memory (sizes bounded by the stage compiler).
@@ -740,7 +730,7 @@ __global__ void k_slotv(const __grid_constant__ SlotJobs jobs, const float2 *__r
 template <int K, int F>
 __global__ void __launch_bounds__(Geo<K>::kThreads, K == kT2Qubits ? 2 : 1)
     k_tile2(float *__restrict__ state, const T2Args a, const __grid_constant__ CUtensorMap map,
-            const __grid_constant__ TileBox box, const __grid_constant__ T2Prog prog) {
+            const __grid_constant__ T2Prog prog) {
     using G = Geo<K>;
     extern __shared__ __align__(1024) unsigned char sm[];
     float2 *tab = reinterpret_cast<float2 *>(sm + G::kOffTab);
@@ -770,24 +760,13 @@ __global__ void __launch_bounds__(Geo<K>::kThreads, K == kT2Qubits ? 2 : 1)
         mbar_expect_tx(bar, (uint32_t)a.nsp * 8u);
         bulk_g2s(dst, a.slotv + t * (uint64_t)a.nsp, (uint32_t)a.nsp * 8u, bar);
     };
-    // the copies of tile t, whose global bits are b, by warp 0
-    auto issue_load = [&](uint64_t t, uint64_t b, float2 *slots) {
-        if (tid == 0) {
-            fence_async_smem();
-            const uint32_t sb = slots ? (uint32_t)a.nsp * 8u : 0u;
-            mbar_expect_tx(bar, G::kTileBytes + sb);
-            if (slots) bulk_g2s(slots, a.slotv + t * (uint64_t)a.nsp, sb, bar);
-        }
-        __syncwarp();
-        tensor_tile_load(&map, box, b, sm, bar, tid);
-    };
     // the base of the tile gridDim.x further on: an addition on the global
     // bits alone (the ones between them pass the carries on)
     const uint64_t step = tile_base(a, gridDim.x);
     uint64_t base = tile_base(a, blockIdx.x);
     if ((uint64_t)blockIdx.x < a.ntiles) {
         if (!a.gen && tid < 32)
-            issue_load(blockIdx.x, base, pre ? slotc : nullptr);
+            issue_tile_load<K>(a, &map, sm, blockIdx.x, base, bar, tid, pre ? slotc : nullptr);
         else if (a.gen && pre && tid == 0)
             issue_slots_only(blockIdx.x, slotc);
     }
@@ -812,7 +791,7 @@ __global__ void __launch_bounds__(Geo<K>::kThreads, K == kT2Qubits ? 2 : 1)
             float2 *nsc = slotc + (buf ^ 1u) * kT2MaxSlots;
             if (!a.gen && tid < 32 && next < a.ntiles) {
                 if (!mbar_wait(rbar, (rd - 1u) & 1u)) atomicExch(a.err, 1);
-                issue_load(next, next_base, pre ? nsc : nullptr);
+                issue_tile_load<K>(a, &map, sm, next, next_base, bar, tid, pre ? nsc : nullptr);
             } else if (a.gen && pre && tid == 0 && next < a.ntiles) {
                 issue_slots_only(next, nsc);
             }
@@ -915,7 +894,7 @@ __global__ void __launch_bounds__(kT2Threads, 2)
                 if (ok && rd && !mbar_wait(rbar, (rd - 1u) & 1u)) ok = false;
                 if (ok) {
                     fence_async_global();
-                    issue_tile_load<kT2Qubits>(a, sm, state, tile_of(b, t), bar, tid);
+                    issue_tile_load<kT2Qubits>(a, &G.map[p], sm, 0, tile_base(a, tile_of(b, t)), bar, tid);
                     inflight = true;
                 } else if (tid == 0) {
                     atomicExch(G.err, 1);
@@ -945,7 +924,8 @@ __global__ void __launch_bounds__(kT2Threads, 2)
                 if (ok) {
                     if (!mbar_wait(rbar, (rd - 1u) & 1u)) atomicExch(G.err, 1);
                     fence_async_global();
-                    issue_tile_load<kT2Qubits>(G.pass[np], sm, state, tile_of(nb, nt), bar, tid);
+                    issue_tile_load<kT2Qubits>(G.pass[np], &G.map[np], sm, 0, tile_base(G.pass[np], tile_of(nb, nt)), bar,
+                                               tid);
                     nissued = true;
                 }
             }
@@ -1010,7 +990,7 @@ __global__ void __launch_bounds__(kT2Threads, 2) k_batch(float *__restrict__ sta
         // straight from registers
         if (!ga.gen && tid < 32) {
             fence_async_global();
-            issue_tile_load<kT2Qubits>(ga, sm, state, t0, bar, tid);
+            issue_tile_load<kT2Qubits>(ga, ga.map, sm, t0, tile_base(ga, t0), bar, tid);
         }
         load_programme<kT2Qubits>(ga, sm, tid, blockDim.x);
         __syncthreads();
@@ -1032,7 +1012,7 @@ __global__ void __launch_bounds__(kT2Threads, 2) k_batch(float *__restrict__ sta
             auto hook = [&]() {
                 if (!a.gen && tid < 32 && tile + 1 < t0 + nt) {
                     if (!mbar_wait(rbar, (rd - 1u) & 1u)) atomicExch(B.err, 1);
-                    issue_tile_load<kT2Qubits>(a, sm, state, tile + 1, bar, tid);
+                    issue_tile_load<kT2Qubits>(a, a.map, sm, tile + 1, tile_base(a, tile + 1), bar, tid);
                 }
             };
             t2_run<kT2Qubits, F>(a, SmemIns(), reinterpret_cast<float4 *>(state), rbar, rd, base, sc, hook);
@@ -1268,7 +1248,6 @@ void t2_fill_args(const T2Pass &p, const T2Device &d, int n, T2Args *a) {
     a->nmats = (int)(p.wide ? p.mats64.size() / 8 : p.mats.size());
     a->nstages = (int)p.stages.size();
     a->last_stage = p.dev_last_stage;
-    for (int s = 0; s < p.k; s++) a->slot_phys[s] = p.slot_phys[s];
     // runs of the global bits: tile index bit i is the i-th lowest set bit of gmask
     a->ngr = 0;
     int ti = 0;
@@ -1413,13 +1392,12 @@ sv_status t2_launch(sv_state *h, const T2Pass &p, const T2Device &d, const sv_la
     h->stats.ctas_per_sm = h->stats.ctas_per_sm ? std::min(h->stats.ctas_per_sm, per_sm) : per_sm;
     const uint64_t grid = std::min<uint64_t>(a.ntiles, (uint64_t)per_sm * h->sm_count);
     CUtensorMap map{};
-    TileBox box{};
-    if (!a.gen) SV_TRY(tile_map(h->amps, h->n, p.k, p.slot_phys, sizeof(float2), &map, &box));
+    if (!a.gen) SV_TRY(tile_map(h->amps, h->n, p.k, p.slot_phys, sizeof(float2), &map, &a.box));
     T2Prog prog;
     std::memcpy(prog.ins, p.dev.data(), p.dev.size() * sizeof(T2Ins));
     const int slot = prof_begin(h);
     SV_CUDA(launch_after(kern, (unsigned)grid, threads, smem, h->stream, after_tile && slot < 0,
-                         reinterpret_cast<float *>(h->amps), a, map, box, prog));
+                         reinterpret_cast<float *>(h->amps), a, map, prog));
     note_launch();
     prof_end(h, slot, meta);
     h->stats.kernels++;

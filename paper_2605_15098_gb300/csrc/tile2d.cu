@@ -606,7 +606,7 @@ __device__ __forceinline__ void tile_slots_d(const T2Args &a, double2 *slotc, ui
 template <int F>
 __global__ void __launch_bounds__(kDThreads, 1)
     k_tile2d(double2 *__restrict__ state, const T2Args a, const __grid_constant__ CUtensorMap map,
-             const __grid_constant__ TileBox box, const __grid_constant__ T2Prog prog) {
+             const __grid_constant__ T2Prog prog) {
     extern __shared__ __align__(1024) unsigned char sm[];
     double2 *slotc = reinterpret_cast<double2 *>(sm + GD::kOffSlotc);
     uint64_t *bar = reinterpret_cast<uint64_t *>(sm + GD::kOffBar);
@@ -630,7 +630,7 @@ __global__ void __launch_bounds__(kDThreads, 1)
             mbar_expect_tx(bar, (uint32_t)GD::kTileBytes);
         }
         __syncwarp();
-        tensor_tile_load(&map, box, b << 1, sm, bar, tid);
+        tensor_tile_load(&map, a.box, b << 1, sm, bar, tid);
     };
     // the base of the tile gridDim.x further on: an addition on the global bits
     const uint64_t step = tile_base_d(a, gridDim.x);
@@ -687,13 +687,12 @@ sv_status t2d_launch(sv_state *h, const T2Pass &p, const T2Device &d, const sv_l
     h->stats.ctas_per_sm = h->stats.ctas_per_sm ? std::min(h->stats.ctas_per_sm, per_sm) : per_sm;
     const uint64_t grid = std::min<uint64_t>(a.ntiles, (uint64_t)per_sm * h->sm_count);
     CUtensorMap map{};
-    TileBox box{};
-    if (!a.gen) SV_TRY(tile_map(h->amps, h->n, p.k, p.slot_phys, sizeof(double2), &map, &box));
+    if (!a.gen) SV_TRY(tile_map(h->amps, h->n, p.k, p.slot_phys, sizeof(double2), &map, &a.box));
     T2Prog prog;
     std::memcpy(prog.ins, p.dev.data(), p.dev.size() * sizeof(T2Ins));
     const int slot = prof_begin(h);
     SV_CUDA(launch_after(kern, (unsigned)grid, kDThreads, GD::kSmemBytes, h->stream, after_tile && slot < 0,
-                         reinterpret_cast<double2 *>(h->amps), a, map, box, prog));
+                         reinterpret_cast<double2 *>(h->amps), a, map, prog));
     note_launch();
     prof_end(h, slot, meta);
     h->stats.kernels++;
