@@ -91,9 +91,18 @@ std::vector<sv_gate> fold_prefix(const sv_gate *g, size_t m, int64_t *basis, uin
     return out;
 }
 
+// Parts of an instance's read-out: 2^kBatchReadLog amplitudes each, while a
+// part has a pair of outcomes for every thread.  Only a split instance shares
+// them out, but every instance adds up its parts, so that both give the same
+// probability.
+int read_parts(const BatchInst &I) {
+    const int most = std::max(0, I.m - 9);
+    return 1 << std::max(0, std::min(I.nphys - kBatchReadLog, most));
+}
+
 // The launch's work items in claim order.  Instances of at least split_q
 // qubits (largest first) are shared out: each pass in claims of
-// kBatchClaimTiles tiles, then the read-out.  Their levels (pass 0, pass 1,
+// kBatchClaimTiles tiles, then the read-out in parts.  Their levels (pass 0, pass 1,
 // ..., read-out) are lagged: level l of the r-th large instance sits in step
 // r + l * lag, with enough claims between two levels of one instance (about
 // 2.5 grids) that the earlier level is done when the later one is claimed.
@@ -109,7 +118,7 @@ std::vector<int4> batch_work(const std::vector<BatchInst> &inst, const std::vect
     std::vector<int4> work;
     if (!large.empty()) {
         double per = 0;
-        for (int i : large) per += (double)claims(i) * inst[i].npass + 1;
+        for (int i : large) per += (double)claims(i) * inst[i].npass + inst[i].parts;
         per /= (double)large.size();
         const int lag = std::max(1, (int)std::ceil(2.5 * grid / per));
         struct Seg { long long key; int level, inst; };
@@ -123,7 +132,7 @@ std::vector<int4> batch_work(const std::vector<BatchInst> &inst, const std::vect
         for (const Seg &s : segs) {
             const BatchInst &I = inst[s.inst];
             if (s.level == I.npass) {
-                work.push_back(make_int4(s.inst, kBatchReadout, 0, 0));
+                for (int t = 0; t < I.parts; t++) work.push_back(make_int4(s.inst, kBatchReadout, t, 1));
                 continue;
             }
             const int ntiles = 1 << (I.nphys - kT2Qubits);
@@ -319,6 +328,12 @@ sv_status sv_batch_create(const sv_batch_item *items, size_t count, const sv_con
         }
         split_q = largest > 0.5 * total / grid ? 16 : 25;
     }
+    int nparts = 0;
+    for (BatchInst &I : inst) {
+        I.part0 = nparts;
+        I.parts = read_parts(I);
+        nparts += I.parts;
+    }
     const std::vector<int4> items4 = batch_work(inst, cost, split_q, grid);
     const size_t inst_off = blob.put(inst.data(), inst.size() * sizeof(BatchInst));
     const size_t work_off = blob.put(items4.data(), items4.size() * sizeof(int4));
@@ -366,8 +381,9 @@ sv_status sv_batch_create(const sv_batch_item *items, size_t count, const sv_con
         return bail(fail(SV_ERR_CUDA, "programme upload failed"));
     }
     b->state_amps = amps;
-    b->queue_bytes = 256 + pass.size() * sizeof(unsigned);
-    if (dev_malloc(&b->queue, b->queue_bytes) != cudaSuccess ||
+    b->queue_bytes = 256 + (pass.size() + count) * sizeof(unsigned);
+    const size_t parts_off = (b->queue_bytes + 255) & ~(size_t)255;
+    if (dev_malloc(&b->queue, parts_off + nparts * sizeof(BatchPart)) != cudaSuccess ||
         dev_malloc(&b->out_idx, count * sizeof(uint64_t)) != cudaSuccess ||
         dev_malloc(&b->out_p, count * sizeof(double)) != cudaSuccess ||
         cudaMallocHost(&b->h_idx, count * sizeof(uint64_t)) != cudaSuccess ||
@@ -382,6 +398,8 @@ sv_status sv_batch_create(const sv_batch_item *items, size_t count, const sv_con
     args.nwork = (int)items4.size();
     args.queue = b->queue;
     args.done = reinterpret_cast<unsigned *>(reinterpret_cast<char *>(b->queue) + 256);
+    args.rdone = args.done + pass.size();
+    args.parts = reinterpret_cast<BatchPart *>(reinterpret_cast<char *>(b->queue) + parts_off);
     args.out_idx = b->out_idx;
     args.out_p = b->out_p;
     args.err = b->err;

@@ -188,13 +188,21 @@ struct BatchInst {
     int nphys;           // qubits of the stored state (>= 13)
     int m;               // read-out qubits
     int out;             // result slot
+    int part0, parts;    // first read-out part, parts
     int pos[34];         // physical bit of read-out bit j
 };
 
 // Work items of a batched launch, in claim order: x = instance, y = kind |
-// (pass << 4), z = first tile, w = tiles.
+// (pass << 4), z = first tile, w = tiles; a read-out: z = its part.
 enum { kBatchWhole = 0, kBatchTiles = 1, kBatchReadout = 2 };
 constexpr int kBatchClaimTiles = 8;  // tiles of one claim of a split instance
+constexpr int kBatchReadLog = 17;    // amplitudes of one part of a split instance's read-out
+
+// One part of a split instance's read-out.
+struct BatchPart {
+    double best, total;
+    uint64_t idx;
+};
 
 struct BatchArgs {
     const BatchInst *inst;
@@ -202,6 +210,8 @@ struct BatchArgs {
     const int4 *work;  // work items in claim order
     int nwork;
     unsigned *done;    // per pass (index into passes): tiles finished (zero at launch)
+    unsigned *rdone;   // per instance: read-out parts finished (zero at launch)
+    BatchPart *parts;
     int *queue;
     uint64_t *out_idx;
     double *out_p;

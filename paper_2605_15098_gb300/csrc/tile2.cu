@@ -1023,8 +1023,11 @@ __global__ void __launch_bounds__(kT2Threads, 2) k_batch(float *__restrict__ sta
         __syncthreads();
         return true;
     };
-    // argmax (lowest index among ties) of the FP64 marginal over I.pos
-    auto readout = [&](const BatchInst &I, const float *state) {
+    // argmax (lowest index among ties) of the FP64 marginal over I.pos: the
+    // parts [part0, part1) of its outcomes; a CTA that has them all combines
+    // them in order, else the last part to finish does (one CTA took 200 us
+    // for the 2^20 amplitudes of a large instance)
+    auto readout = [&](const BatchInst &I, const float *state, int inst, int part0, int part1) {
         // Outcomes are visited in the order of their physical index (bit i of
         // the visit index v is the i-th lowest physical read-out qubit), so
         // that a warp's loads are contiguous whatever qubit map the passes
@@ -1057,71 +1060,130 @@ __global__ void __launch_bounds__(kT2Threads, 2) k_batch(float *__restrict__ sta
         const uint64_t rest = all & ~mask;
         const uint64_t nrest = UINT64_C(1) << (I.nphys - I.m);
         const uint64_t outcomes = UINT64_C(1) << I.m;
-        const float2 *st2 = reinterpret_cast<const float2 *>(state);
-        double best = -1.0, tot = 0.0;
-        uint64_t bidx = ~UINT64_C(0);
-        for (uint64_t v = tid; v < outcomes; v += blockDim.x) {
-            const uint64_t xy = T[v & 255] | T[256 + ((v >> 8) & 255)] | T[512 + ((v >> 16) & 255)];
-            const uint64_t y = Y[v & 255] | Y[256 + ((v >> 8) & 255)] | Y[512 + ((v >> 16) & 255)];
-            // exact FP32 squares (product + fmaf remainder) summed as a
-            // double-float pair: FP64-accurate without FP64 arithmetic
+        const int parts = I.parts;
+        double bv = -1.0, bt = 0.0;  // thread 0: the combined parts
+        uint64_t bi = ~UINT64_C(0);
+        auto combine = [&](double v2, uint64_t i2, double t2) {
+            bt += t2;
+            if (v2 > bv || (v2 == bv && i2 < bi)) {
+                bv = v2;
+                bi = i2;
+            }
+        };
+        // exact FP32 squares (product + fmaf remainder) summed as a
+        // double-float pair: FP64-accurate without FP64 arithmetic
+        struct Pair {
             float hi = 0.f, lo = 0.f;
-            auto two_sum = [&](float b) {
+            __device__ void two_sum(float b) {
                 const float t = hi + b;
                 const float bb = t - hi;
                 lo += (hi - (t - bb)) + (b - bb);
                 hi = t;
+            }
+            __device__ void add(float x, float y) {
+                const float pr = x * x, pi = y * y;
+                lo += fmaf(x, x, -pr) + fmaf(y, y, -pi);
+                two_sum(pr);
+                two_sum(pi);
+            }
+            __device__ double value() const { return (double)hi + (double)lo; }
+        };
+        bool complete = part1 - part0 == parts;
+        for (int part = part0; part < part1; part++) {
+            double best = -1.0, tot = 0.0;
+            uint64_t bidx = ~UINT64_C(0);
+            auto candidate = [&](double acc, uint64_t y) {
+                tot += acc;
+                if (acc > best || (acc == best && y < bidx)) {
+                    best = acc;
+                    bidx = y;
+                }
             };
-            // the amplitudes of outcome y in increasing index order, four
-            // independent loads in flight at a time
-            uint64_t xr = 0;
-            for (uint64_t r = 0; r < nrest; r += 4) {
-                uint64_t xs[4];
+            const uint64_t span = outcomes / (uint64_t)parts, v0 = span * (uint64_t)part;
+            if ((mask & 1) && span > 1) {
+                // physical bit 0 is an outcome bit: two outcomes per 16-byte load
+                const float4 *st4 = reinterpret_cast<const float4 *>(state);
+                for (uint64_t v = v0 + 2 * tid; v < v0 + span; v += 2 * blockDim.x) {
+                    const uint64_t xy = T[v & 255] | T[256 + ((v >> 8) & 255)] | T[512 + ((v >> 16) & 255)];
+                    const uint64_t y = Y[v & 255] | Y[256 + ((v >> 8) & 255)] | Y[512 + ((v >> 16) & 255)];
+                    Pair p0, p1;
+                    uint64_t xr = 0;
+                    for (uint64_t r = 0; r < nrest; r += 4) {
+                        float4 w[4];
 #pragma unroll
-                for (int u = 0; u < 4; u++) {
-                    xs[u] = xr;
-                    xr = ((xr | ~rest) + 1) & rest;
+                        for (int u = 0; u < 4; u++) {
+                            w[u] = r + u < nrest ? st4[(xy | xr) >> 1] : make_float4(0.f, 0.f, 0.f, 0.f);
+                            xr = ((xr | ~rest) + 1) & rest;
+                        }
+#pragma unroll
+                        for (int u = 0; u < 4; u++) {
+                            p0.add(w[u].x, w[u].y);
+                            p1.add(w[u].z, w[u].w);
+                        }
+                    }
+                    candidate(p0.value(), y);
+                    candidate(p1.value(), y | Y[1]);
                 }
-                float2 v[4];
+            } else {
+                const float2 *st2 = reinterpret_cast<const float2 *>(state);
+                for (uint64_t v = v0 + tid; v < v0 + span; v += blockDim.x) {
+                    const uint64_t xy = T[v & 255] | T[256 + ((v >> 8) & 255)] | T[512 + ((v >> 16) & 255)];
+                    const uint64_t y = Y[v & 255] | Y[256 + ((v >> 8) & 255)] | Y[512 + ((v >> 16) & 255)];
+                    Pair p0;
+                    // the amplitudes of outcome y in increasing index order, four
+                    // independent loads in flight at a time
+                    uint64_t xr = 0;
+                    for (uint64_t r = 0; r < nrest; r += 4) {
+                        float2 w[4];
 #pragma unroll
-                for (int u = 0; u < 4; u++)
-                    v[u] = r + u < nrest ? st2[xy | xs[u]] : make_float2(0.f, 0.f);
+                        for (int u = 0; u < 4; u++) {
+                            w[u] = r + u < nrest ? st2[xy | xr] : make_float2(0.f, 0.f);
+                            xr = ((xr | ~rest) + 1) & rest;
+                        }
 #pragma unroll
-                for (int u = 0; u < 4; u++) {
-                    if (r + u >= nrest) break;
-                    const float2 amp = v[u];
-                    const float pr = amp.x * amp.x, pi = amp.y * amp.y;
-                    lo += fmaf(amp.x, amp.x, -pr) + fmaf(amp.y, amp.y, -pi);
-                    two_sum(pr);
-                    two_sum(pi);
+                        for (int u = 0; u < 4; u++) p0.add(w[u].x, w[u].y);
+                    }
+                    candidate(p0.value(), y);
                 }
             }
-            const double acc = (double)hi + (double)lo;
-            tot += acc;
-            if (acc > best || (acc == best && y < bidx)) {
-                best = acc;
-                bidx = y;
-            }
-        }
-        s_val[tid] = best;
-        s_idx[tid] = bidx;
-        s_tot[tid] = tot;
-        __syncthreads();
-        for (int w = kT2Threads / 2; w; w >>= 1) {
-            if (tid < w) {
-                const double v2 = s_val[tid + w];
-                const uint64_t i2 = s_idx[tid + w];
-                if (v2 > s_val[tid] || (v2 == s_val[tid] && i2 < s_idx[tid])) {
-                    s_val[tid] = v2;
-                    s_idx[tid] = i2;
+            s_val[tid] = best;
+            s_idx[tid] = bidx;
+            s_tot[tid] = tot;
+            __syncthreads();
+            for (int w = kT2Threads / 2; w; w >>= 1) {
+                if (tid < w) {
+                    const double v2 = s_val[tid + w];
+                    const uint64_t i2 = s_idx[tid + w];
+                    if (v2 > s_val[tid] || (v2 == s_val[tid] && i2 < s_idx[tid])) {
+                        s_val[tid] = v2;
+                        s_idx[tid] = i2;
+                    }
+                    s_tot[tid] += s_tot[tid + w];
                 }
-                s_tot[tid] += s_tot[tid + w];
+                __syncthreads();
+            }
+            if (tid == 0) {
+                if (part1 - part0 == parts) {
+                    combine(s_val[0], s_idx[0], s_tot[0]);
+                } else {
+                    BatchPart *ps = B.parts + I.part0;
+                    ps[part] = {s_val[0], s_tot[0], s_idx[0]};
+                    __threadfence();
+                    if (atomicAdd(B.rdone + inst, 1u) == (unsigned)parts - 1u) {  // every part is in
+                        complete = true;
+                        __threadfence();
+                        for (int i = 0; i < parts; i++)
+                            combine(__ldcg(&ps[i].best),
+                                    __ldcg(reinterpret_cast<const unsigned long long *>(&ps[i].idx)),
+                                    __ldcg(&ps[i].total));
+                    }
+                }
             }
             __syncthreads();
         }
-        if (tid == 0) {
-            B.out_idx[I.out] = s_idx[0];
-            B.out_p[I.out] = s_tot[0] > 0.0 ? s_val[0] / s_tot[0] : 0.0;
+        if (tid == 0 && complete) {
+            B.out_idx[I.out] = bi;
+            B.out_p[I.out] = bt > 0.0 ? bv / bt : 0.0;
         }
         __syncthreads();
     };
@@ -1167,7 +1229,7 @@ __global__ void __launch_bounds__(kT2Threads, 2) k_batch(float *__restrict__ sta
             }
             continue;
         }
-        readout(I, state);
+        readout(I, state, wk.x, whole ? 0 : wk.z, whole ? I.parts : wk.z + 1);
     }
 }
 
