@@ -181,6 +181,71 @@ void pick_regs(const TilePass &tp, size_t from, bool no123, int out[4]) {
     }
 }
 
+// Order the gates between two diagonal runs (uncontrolled ones on different
+// bits commute) so that stages follow each other with fewer changes: first
+// the gates on the current register bits, last those on bits the segment
+// after the run needs soonest.  With twelve tile bits besides bit 0 and four
+// register bits, a layer of rotations then takes two stage changes instead of
+// three (random n=28 depth 8: 36 changes, 47 in list order; n=25 depth 20: 78
+// and 104).  A stage change costs a shared-memory round trip of the tile,
+// about 35 % of a random pass: n=25 5.40 -> 5.10 ms, n=28 20.1 -> 18.6 ms,
+// n=19 238 -> 232 us.  Steps before `first` stay;
+// `gen`: as for compile_fmt2.
+void order_gates(TilePass &tp, size_t first, bool gen) {
+    std::vector<TileOp> &ops = tp.ops;
+    auto is_free = [](const TileOp &op) { return op.type == TOP_GATE || op.type == TOP_H || op.type == TOP_X; };
+    int cur[4] = {-1, -1, -1, -1};  // the register bits besides bit 0
+    bool started = false;
+    auto resident = [&](int t) { return t == 0 || t == cur[0] || t == cur[1] || t == cur[2] || t == cur[3]; };
+    for (size_t i = first; i < ops.size();) {
+        if (!is_gate(ops[i].type)) {
+            i++;
+            continue;
+        }
+        size_t j = i;
+        while (j < ops.size() && is_free(ops[j])) j++;
+        if (j == i) j = i + 1;  // a controlled gate keeps its place
+        std::vector<TileOp> left(ops.begin() + (long)i, ops.begin() + (long)j), done;
+        // the next use of each bit after the segment
+        size_t use[kT2MaxQubits];
+        for (int t = 0; t < kT2MaxQubits; t++) use[t] = ops.size();
+        for (size_t e = ops.size(); e-- > j;)
+            if (is_gate(ops[e].type)) use[ops[e].slot] = e;
+        while (!left.empty()) {
+            std::vector<TileOp> rest;
+            for (const TileOp &op : left) (resident(op.slot) ? done : rest).push_back(op);
+            left.swap(rest);
+            if (left.empty()) break;
+            // the next register bits: those of the segment whose next use is
+            // farthest (the first stage of a pass that reads its tile cannot
+            // have tile bits 1..3 before any other), filled up with the next
+            // ones as pick_regs does
+            std::vector<int> bits;
+            for (const TileOp &op : left)
+                if (std::find(bits.begin(), bits.end(), op.slot) == bits.end()) bits.push_back(op.slot);
+            const bool late123 = !started && !gen;
+            std::stable_sort(bits.begin(), bits.end(), [&](int x, int y) {
+                const bool lx = late123 && x <= 3, ly = late123 && y <= 3;
+                return lx != ly ? ly : use[x] > use[y];
+            });
+            int n = 0;
+            for (int b : bits)
+                if (n < 4 && !(late123 && b <= 3)) cur[n++] = b;
+            const bool short_first = late123 && n < 4;  // pick_regs pads it with other bits
+            for (size_t e = j; e < ops.size() && n < 4 && !short_first; e++) {
+                if (!is_gate(ops[e].type) || ops[e].slot == 0) continue;
+                if (std::find(cur, cur + n, ops[e].slot) == cur + n) cur[n++] = ops[e].slot;
+            }
+            while (n < 4) cur[n++] = -1;
+            // the chosen bits' gates come next
+            std::stable_partition(left.begin(), left.end(), [&](const TileOp &op) { return resident(op.slot); });
+            started = true;
+        }
+        std::copy(done.begin(), done.end(), ops.begin() + (long)i);
+        i = j;
+    }
+}
+
 uint32_t turns32(uint64_t t64) { return (uint32_t)((t64 + (UINT64_C(1) << 31)) >> 32); }
 
 // cos and sin of 2 pi u / 2^32, evaluated in FP64 and rounded to FP32.  A
@@ -472,7 +537,8 @@ void lower(T2Pass *o, bool gen) {
 }
 
 template <class P>
-std::string compile_fmt2(const TilePass &tp, T2Pass *out, bool gen) {
+std::string compile_fmt2(const TilePass &given, T2Pass *out, bool gen) {
+    TilePass tp = given;
     using Ph = typename P::Ph;
     using V = typename P::V;
     // a tile term with its phase in the policy's width
@@ -516,6 +582,8 @@ std::string compile_fmt2(const TilePass &tp, T2Pass *out, bool gen) {
             out->n_h++;
         }
     }
+
+    order_gates(tp, first, gen);
 
     std::map<std::pair<int, int>, int> slot_of;
     std::map<std::vector<Ph>, int32_t> table_of;  // table phases -> first matrix record
