@@ -298,7 +298,7 @@ sv_status sv_batch_create(const sv_batch_item *items, size_t count, const sv_con
             o.stages = blob.put(t2.stages.data(), t2.stages.size() * sizeof(T2Stage));
             o.layx = blob.put(t2.layx.data(), t2.layx.size() * sizeof(T2LayoutX));
             o.epi = blob.put(&t2.epi, sizeof(T2Epilogue));
-            o.mats = blob.put(t2.mats.data(), t2.mats.size() * sizeof(T2Mat));
+            o.mats = blob.put(t2.dev_mats.data(), t2.dev_mats.size() * sizeof(T2Mat));
             o.statc = blob.put(t2.statc.data(), t2.statc.size() * sizeof(float));
             o.soff = blob.put(t2.soff.data(), t2.soff.size() * sizeof(int32_t));
             o.sterms = blob.put(t2.sterms.data(), t2.sterms.size() * sizeof(T2SlotTerm));

@@ -56,6 +56,7 @@ struct T2Pass {
     // format 2: the programme the kernels run (tileprog.h), its last stage
     // change and, for the gen variant, its closing scale
     std::vector<T2Ins> dev;
+    std::vector<T2Mat> dev_mats;  // complex64: its matrix records
     int dev_last_stage = -1;
     double dev_gen_scale = 1.0;
     int nblocks = 0;

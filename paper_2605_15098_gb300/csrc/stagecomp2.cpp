@@ -441,6 +441,7 @@ void lower(T2Pass *o, bool gen) {
     bool negative = (o->sign_flips & 1) != 0, rotated = false;
     o->dev.clear();
     auto rotation = [&](size_t i) { return i < o->ins.size() && o->ins[i].op == T2_ROT; };
+    o->dev_mats = o->mats;
     double scale = 1.0;
     bool scaled = false;
     float hi = 0.f, lo = 0.f;
@@ -452,10 +453,12 @@ void lower(T2Pass *o, bool gen) {
             g.hd = kT2HdRots;
             g.aux = in.aux;
             int mask = 0, order = 0, count = 0, sine = 0;
+            int32_t rec[kT2RegBits];
             for (; rotation(i) && !((mask >> o->ins[i].idx) & 1) && o->ins[i].aux == in.aux + count; i++, count++) {
                 const int j = o->ins[i].idx;
                 mask |= 1 << j;
                 order |= count << (3 * j);
+                rec[j] = o->ins[i].aux;
                 if (o->wide) {
                     const double *m = &o->mats64[8 * (size_t)o->ins[i].aux];
                     if (m[4] != 0.0) sine |= 1 << j;
@@ -465,6 +468,19 @@ void lower(T2Pass *o, bool gen) {
                 }
             }
             i--;
+            if (!o->wide) {
+                // records in the order the kernel takes the bits, each
+                // coefficient as a packed pair
+                order = 0;
+                int at = 0;
+                for (int j : {1, 2, 3, 4, 0}) {
+                    if (!((mask >> j) & 1)) continue;
+                    const float *from = o->mats[rec[j]].m;
+                    o->dev_mats[in.aux + at] = T2Mat{{from[0], from[0], from[1], from[1]}};
+                    order |= at++ << (3 * j);
+                }
+                if ((mask & 0x1e) == 0x1e) g.hd = kT2HdRots4;
+            }
             g.cidx = (int16_t)mask;
             g.e0 = (int16_t)order;
             g.idx = (int8_t)sine;

@@ -99,15 +99,18 @@ struct Layout2 {
 struct LayoutS {
     int b, p1, p2, p3, p4;
     __device__ LayoutS(const T2LayoutX *x, int tid) {
-        b = (int)x->plo[tid & 31] ^ (int)x->phi[tid >> 5];
+        b = ((int)x->plo[tid & 31] ^ (int)x->phi[tid >> 5]) << 4;
         const int4 pv = *reinterpret_cast<const int4 *>(x->ps);
-        p1 = pv.x;
-        p2 = pv.y;
-        p3 = pv.z;
-        p4 = pv.w;
+        p1 = pv.x << 4;
+        p2 = pv.y << 4;
+        p3 = pv.z << 4;
+        p4 = pv.w << 4;
     }
-    __device__ int idx(int q) const {
-        return b ^ ((q & 1) ? p1 : 0) ^ ((q & 2) ? p2 : 0) ^ ((q & 4) ? p3 : 0) ^ ((q & 8) ? p4 : 0);
+    // pair q's place in the tile at t2_dyn_smem: a byte offset, so that no
+    // access scales an index
+    __device__ float4 *at(int q) const {
+        const int o = b ^ ((q & 1) ? p1 : 0) ^ ((q & 2) ? p2 : 0) ^ ((q & 4) ? p3 : 0) ^ ((q & 8) ? p4 : 0);
+        return reinterpret_cast<float4 *>(t2_dyn_smem + o);
     }
 };
 
@@ -382,14 +385,18 @@ __device__ __forceinline__ void t2_run(const T2Args &a, Ins ins, float4 *gstate,
         const float4 *mrec = M + 2 * w.w;
         const uint32_t hd = ((uint32_t)w.y >> 16) & 0xffu;  // the handler code (tileprog.h)
         if constexpr ((F & kFeatR) != 0) {
+            if (hd == kT2HdRots4) {
+                reg_rot<1>(r, mrec[0]);
+                reg_rot<2>(r, mrec[2]);
+                reg_rot<3>(r, mrec[4]);
+                reg_rot<4>(r, mrec[6]);
+                if ((uint32_t)w.y & 1u) reg_rot<0>(r, mrec[8]);
+                continue;
+            }
             if (hd == kT2HdRots) {
                 const uint32_t mask = (uint32_t)w.y & 31u, order = (uint32_t)w.z;
-                const float2 *rec = reinterpret_cast<const float2 *>(mrec);
-#define SV_ROT(J)                                                   \
-    if (mask & (1u << J)) {                                         \
-        const float2 ts = rec[4 * ((order >> (3 * J)) & 7u)];       \
-        reg_rot<J>(r, ts.x, ts.y);                                  \
-    }
+#define SV_ROT(J) \
+    if (mask & (1u << J)) reg_rot<J>(r, mrec[2 * ((order >> (3 * J)) & 7u)]);
                 SV_ROT(1)
                 SV_ROT(2)
                 SV_ROT(3)
@@ -420,14 +427,14 @@ __device__ __forceinline__ void t2_run(const T2Args &a, Ins ins, float4 *gstate,
                     const LayoutS L = layout_s(stage);
 #pragma unroll
                     for (int q = 0; q < kNP2; q++)
-                        tile4[L.idx(q)] = make_float4(r.re[q].x, r.re[q].y, r.im[q].x, r.im[q].y);
+                        *L.at(q) = make_float4(r.re[q].x, r.re[q].y, r.im[q].x, r.im[q].y);
                     if (local) __syncwarp();
                     else __syncthreads();
                     stage = w.w;
                     const LayoutS L2 = layout_s(stage);
 #pragma unroll
                     for (int q = 0; q < kNP2; q++) {
-                        const float4 v = tile4[L2.idx(q)];
+                        const float4 v = *L2.at(q);
                         r.re[q] = make_float2(v.x, v.y);
                         r.im[q] = make_float2(v.z, v.w);
                     }
@@ -1307,7 +1314,7 @@ void t2_fill_args(const T2Pass &p, const T2Device &d, int n, T2Args *a) {
     a->nins = (int)p.dev.size();
     a->nrows = (int)((p.wide ? p.statc64.size() : p.statc.size()) / (2 * (size_t)p.threads));
     a->nslots = (int)p.slots.size();
-    a->nmats = (int)(p.wide ? p.mats64.size() / 8 : p.mats.size());
+    a->nmats = (int)(p.wide ? p.mats64.size() / 8 : p.dev_mats.size());
     a->nstages = (int)p.stages.size();
     a->last_stage = p.dev_last_stage;
     // runs of the global bits: tile index bit i is the i-th lowest set bit of gmask

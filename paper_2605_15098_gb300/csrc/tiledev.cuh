@@ -375,19 +375,20 @@ __device__ __forceinline__ void reg_u2(RegsN<NP> &r, uint32_t qm, const float *m
 // (exactly the rotation); each shear is one multiply-add per plane and no
 // register of the pair is copied.
 template <int J, int NP>
-__device__ __forceinline__ void reg_rot(RegsN<NP> &r, float t, float s) {
+__device__ __forceinline__ void reg_rot(RegsN<NP> &r, float4 ts) {
+    const float2 t = make_float2(ts.x, ts.y), s = make_float2(ts.z, ts.w);
     if constexpr (J >= 1) {
 #pragma unroll
         for (int g = 0; g < NP / 8; g++) {
 #pragma unroll
             for (int i = 0; i < 4; i++) {
                 const int q = bfly_q<J>(4 * g + i), q1 = q | (1 << (J - 1));
-                r.re[q] = fma2(r.re[q1], f2(t), r.re[q]);
-                r.im[q] = fma2(r.im[q1], f2(t), r.im[q]);
-                r.re[q1] = fma2(r.re[q], f2(s), r.re[q1]);
-                r.im[q1] = fma2(r.im[q], f2(s), r.im[q1]);
-                r.re[q] = fma2(r.re[q1], f2(t), r.re[q]);
-                r.im[q] = fma2(r.im[q1], f2(t), r.im[q]);
+                r.re[q] = fma2(r.re[q1], t, r.re[q]);
+                r.im[q] = fma2(r.im[q1], t, r.im[q]);
+                r.re[q1] = fma2(r.re[q], s, r.re[q1]);
+                r.im[q1] = fma2(r.im[q], s, r.im[q1]);
+                r.re[q] = fma2(r.re[q1], t, r.re[q]);
+                r.im[q] = fma2(r.im[q1], t, r.im[q]);
             }
         }
     } else {
@@ -397,12 +398,12 @@ __device__ __forceinline__ void reg_rot(RegsN<NP> &r, float t, float s) {
             for (int i = 0; i < 4; i++) {
                 const int q = 4 * g4 + i;
                 float2 &x = r.re[q], &y = r.im[q];
-                x.x = fmaf(x.y, t, x.x);
-                y.x = fmaf(y.y, t, y.x);
-                x.y = fmaf(x.x, s, x.y);
-                y.y = fmaf(y.x, s, y.y);
-                x.x = fmaf(x.y, t, x.x);
-                y.x = fmaf(y.y, t, y.x);
+                x.x = fmaf(x.y, t.x, x.x);
+                y.x = fmaf(y.y, t.x, y.x);
+                x.y = fmaf(x.x, s.x, x.y);
+                y.y = fmaf(y.x, s.x, y.y);
+                x.x = fmaf(x.y, t.x, x.x);
+                y.x = fmaf(y.y, t.x, y.x);
             }
         }
     }

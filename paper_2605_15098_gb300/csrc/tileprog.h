@@ -215,7 +215,9 @@ constexpr int kT2HdStage = 1, kT2HdScale = 2, kT2HdDiag = 3;
 // rotation's and 32 or 64 for a diagonal factor's, so:
 //  * consecutive rotations on distinct register bits are one step (Rots):
 //    cidx = their register bits as a mask, e0 = three bits per register bit:
-//    its record, counted from record `aux` (the records are consecutive);
+//    its record, counted from record `aux` (the records are consecutive; in
+//    complex64 each holds its two coefficients as packed pairs); Rots4: all of
+//    register bits 1..4, their records in this order, and bit 0 if cidx has it;
 //    complex128: idx = the bits whose rotation is divided by its sine, below;
 //  * a diagonal run is one step per factor, with the factor's record in the
 //    step: Table (aux = first matrix record, cidx = thread-bit predicate) and
@@ -230,7 +232,7 @@ constexpr int kT2HdStage = 1, kT2HdScale = 2, kT2HdDiag = 3;
 // [[k, -1], [1, k]] with k = c / s, whichever has |k| <= 1: two multiply-adds
 // per pair and component instead of three (the FP64 pipe bounds that kernel);
 // the product of the divisors joins the closing scale.
-constexpr int kT2HdRots = 4, kT2HdTable = 5, kT2HdFactor = 6;
+constexpr int kT2HdRots = 4, kT2HdTable = 5, kT2HdFactor = 6, kT2HdRots4 = 7;
 constexpr int kT2DevIns = 256;  // at most kT2SmemIns steps and kT2SmemFactors factors
 
 // Write-back offsets of the final layout in the global state (amplitudes),
