@@ -56,7 +56,8 @@ struct T2Pass {
     // format 2: the programme the kernels run (tileprog.h), its last stage
     // change and, for the gen variant, its closing scale
     std::vector<T2Ins> dev;
-    std::vector<T2Mat> dev_mats;  // complex64: its matrix records
+    std::vector<T2Mat> dev_mats;  // its matrix records
+    std::vector<double> dev_mats64;  // complex128
     int dev_last_stage = -1;
     double dev_gen_scale = 1.0;
     int nblocks = 0;

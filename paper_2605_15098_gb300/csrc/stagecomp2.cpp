@@ -345,6 +345,20 @@ struct P32 {
     static void push_sterm(T2Pass *o, int g0, int g1, Ph th) {
         o->sterms.push_back({(int16_t)g0, (int16_t)g1, th});
     }
+    static Ph sterm(const T2Pass *o, int32_t t) { return o->sterms[t].theta; }
+    // the device form's own records: a table, and a record of eight words
+    static size_t ndev(const T2Pass *o) { return o->dev_mats.size(); }
+    static int32_t push_dev_table(T2Pass *o, const Ph *u) {
+        o->mats.swap(o->dev_mats);
+        const int32_t m0 = push_table(o, u);
+        o->mats.swap(o->dev_mats);
+        return m0;
+    }
+    static int32_t push_words(T2Pass *o, const int32_t *words) {
+        o->dev_mats.emplace_back();
+        std::memcpy(o->dev_mats.back().m, words, 8 * sizeof(int32_t));
+        return (int32_t)o->dev_mats.size() - 1;
+    }
 };
 
 struct P64 {
@@ -410,6 +424,20 @@ struct P64 {
     static void push_sterm(T2Pass *o, int g0, int g1, Ph th) {
         o->sterms64.push_back({(int16_t)g0, (int16_t)g1, 0, th});
     }
+    static Ph sterm(const T2Pass *o, int32_t t) { return o->sterms64[t].theta; }
+    static size_t ndev(const T2Pass *o) { return o->dev_mats64.size() / 8; }
+    static int32_t push_dev_table(T2Pass *o, const Ph *u) {
+        o->mats64.swap(o->dev_mats64);
+        const int32_t m0 = push_table(o, u);
+        o->mats64.swap(o->dev_mats64);
+        return m0;
+    }
+    static int32_t push_words(T2Pass *o, const int32_t *words) {
+        double m[8] = {};
+        std::memcpy(m, words, 8 * sizeof(int32_t));
+        o->dev_mats64.insert(o->dev_mats64.end(), m, m + 8);
+        return (int32_t)(o->dev_mats64.size() / 8) - 1;
+    }
 };
 
 // An unevaluated FP64 sum hi + lo.
@@ -432,8 +460,74 @@ double inverse_root(DD x) {
     return y + 0.5 * y * r;
 }
 
+// What the device form needs beyond the programme's records.
+template <class P>
+struct LowerInfo {
+    using Ph = typename P::Ph;
+    // a register-bit factor whose static row is e^{i phi} times the sign of
+    // the parity of (thread & m), by factor
+    struct Sign {
+        Ph phi;
+        uint32_t m;
+    };
+    std::map<int, Sign> signs;
+    std::map<int32_t, std::vector<Ph>> tables;  // a table's phases, by first record
+};
+
+// The register-bit factors of diagonal run `d` that a Signs step takes
+// (tileprog.h): the factors that are signs but for a constant phase, which
+// joins the run's unpredicated table.  Emits the step and returns the factors
+// it covers; *table: factor and first record of the table to run instead.  A
+// factor by itself takes a complex product on half of the amplitudes and some
+// 80 instructions to find its row and slot; with CZ layers these were 15 % of
+// a random pass.  random n=19 222 -> 208 us, n=25 5.03 -> 4.72 ms, n=28
+// 18.5 -> 17.5 ms; complex128 n=21 3.41 -> 3.01 ms (a sign costs the FP64 pipe
+// nothing).
+template <class P>
+std::vector<int> lower_signs(T2Pass *o, const T2Ins &d, const LowerInfo<P> &info, std::pair<int, int32_t> *table) {
+    using Ph = typename P::Ph;
+    constexpr Ph half = (Ph)1 << (8 * sizeof(Ph) - 1);
+    int tab = -1;
+    for (int e = d.e0; e < d.e1; e++)
+        if ((o->fac2[e].w0 & kFacTable) && !((o->fac2[e].w0 >> 10) & 0xfu)) tab = e;
+    std::vector<int> taken;
+    std::vector<Ph> u;
+    if (tab >= 0) u = info.tables.at(o->fac2[tab].row);
+    bool changed = false;
+    int32_t words[8] = {};
+    int mask = 0;
+    for (int e = d.e0; e < d.e1; e++) {
+        const auto it = info.signs.find(e);
+        if (it == info.signs.end()) continue;
+        const T2Fac &f = o->fac2[e];
+        bool ok = !it->second.phi || tab >= 0;
+        for (int32_t t = f.slot < 0 ? 0 : o->soff[f.slot]; f.slot >= 0 && t < o->soff[f.slot + 1]; t++)
+            ok = ok && P::sterm(o, t) == half;
+        if (!ok) continue;
+        const int bit = __builtin_ctz(f.w0 & 0xffu);
+        if (it->second.phi) {
+            for (int x = 0; x < 32; x++)
+                if ((x >> bit) & 1) u[x] += it->second.phi;
+            changed = true;
+        }
+        mask |= 1 << bit;
+        words[bit] = (int32_t)(it->second.m | ((uint32_t)(uint16_t)f.slot << 16));
+        taken.push_back(e);
+    }
+    if (taken.empty() || P::ndev(o) + 1 + (changed ? 8 : 0) > (size_t)kT2SmemMats) return {};
+    T2Ins in{};
+    in.op = T2_DIAG;
+    in.hd = kT2HdSigns;
+    in.cidx = (int16_t)mask;
+    in.aux = P::push_words(o, words);
+    o->dev.push_back(in);
+    if (changed) *table = {tab, P::push_dev_table(o, u.data())};
+    return taken;
+}
+
 // The device form of a compiled programme (tileprog.h).
-void lower(T2Pass *o, bool gen) {
+template <class P>
+void lower(T2Pass *o, bool gen, const LowerInfo<P> &info) {
     // complex128 rotations [[1, -k], [k, 1]] and [[k, -1], [1, k]] grow the
     // norm by sqrt(1 + k^2) for the k as rounded; the product of these and of
     // the Hadamards' sqrt(2) is formed beyond FP64 and rounded once
@@ -442,6 +536,7 @@ void lower(T2Pass *o, bool gen) {
     o->dev.clear();
     auto rotation = [&](size_t i) { return i < o->ins.size() && o->ins[i].op == T2_ROT; };
     o->dev_mats = o->mats;
+    o->dev_mats64 = o->mats64;
     double scale = 1.0;
     bool scaled = false;
     float hi = 0.f, lo = 0.f;
@@ -488,14 +583,17 @@ void lower(T2Pass *o, bool gen) {
             continue;
         }
         if (in.op == T2_DIAG) {
+            std::pair<int, int32_t> table{-1, 0};
+            const std::vector<int> signs = lower_signs<P>(o, in, info, &table);
             for (int e = in.e0; e < in.e1; e++) {
                 const T2Fac &f = o->fac2[e];
+                if (std::find(signs.begin(), signs.end(), e) != signs.end()) continue;
                 T2Ins d{};
                 d.op = T2_DIAG;
                 if (f.w0 & kFacTable) {
                     d.hd = kT2HdTable;
                     d.cidx = (int16_t)((f.w0 >> 10) & 0xfu);
-                    d.aux = f.row;
+                    d.aux = e == table.first ? table.second : f.row;
                 } else {
                     d.hd = kT2HdFactor;
                     d.idx = (int8_t)((f.w0 & 0xffu) ? 1 + __builtin_ctz(f.w0 & 0xffu) : 0);
@@ -602,6 +700,7 @@ std::string compile_fmt2(const TilePass &given, T2Pass *out, bool gen) {
     order_gates(tp, first, gen);
 
     std::map<std::pair<int, int>, int> slot_of;
+    LowerInfo<P> info;
     std::map<std::vector<Ph>, int32_t> table_of;  // table phases -> first matrix record
     auto slot = [&](int i0, int i1) -> int {
         auto key = std::make_pair(i0, i1);
@@ -775,6 +874,7 @@ std::string compile_fmt2(const TilePass &given, T2Pass *out, bool gen) {
         // constants: (register mask, thread predicate 0 = all / t + 1) -> phase
         std::map<std::pair<int, int>, Ph> cst;
         std::vector<T2Fac> facs;
+        std::map<int, typename LowerInfo<P>::Sign> signs;  // by place in facs
         // a static row over the thread index: a constant, a constant on the
         // threads with one bit set (thread factors only: a register-bit
         // factor keeps such a row, so that the run can still become a phased
@@ -811,6 +911,18 @@ std::string compile_fmt2(const TilePass &given, T2Pass *out, bool gen) {
                 }
             }
             if (rowi < 0 && sl0 < 0 && dmask == 0) return;
+            if (mask) {
+                constexpr Ph half = (Ph)1 << (8 * sizeof(Ph) - 1);
+                typename LowerInfo<P>::Sign sg{rowi < 0 ? (Ph)0 : row[0], 0};
+                bool ok = true;
+                if (rowi >= 0) {
+                    for (int t = 0; t < TB; t++)
+                        if (row[1 << t] != row[0]) sg.m |= 1u << t;
+                    for (int tau = 0; tau < NT && ok; tau++)
+                        ok = row[tau] == (Ph)(row[0] + ((__builtin_popcount((unsigned)tau & sg.m) & 1) ? half : 0));
+                }
+                if (ok) signs[(int)facs.size()] = sg;
+            }
             T2Fac f{};
             f.w0 = (uint32_t)mask | (1u << 8) | ((uint32_t)dmask << kFacDynShift);
             f.slot = (int16_t)sl0;
@@ -871,6 +983,7 @@ std::string compile_fmt2(const TilePass &given, T2Pass *out, bool gen) {
             } else {
                 m0 = P::push_table(out, u);
                 table_of[key] = m0;
+                info.tables[m0] = key;
             }
             T2Fac f{};
             f.w0 = kFacTable | ((uint32_t)g.first << 10);
@@ -878,6 +991,7 @@ std::string compile_fmt2(const TilePass &given, T2Pass *out, bool gen) {
             f.row = m0;
             out->fac2.push_back(f);
         }
+        for (const auto &[at, sg] : signs) info.signs[(int)out->fac2.size() + at] = sg;
         out->fac2.insert(out->fac2.end(), facs.begin(), facs.end());
         in.e1 = (int16_t)out->fac2.size();
         if (out->fac2.size() > 32000) return "too many factor applications";
@@ -1028,7 +1142,7 @@ std::string compile_fmt2(const TilePass &given, T2Pass *out, bool gen) {
             // every step is linear: the pass that generates its starting
             // state generates it times the closing scale instead
             out->gen_scale = s;
-            lower(out, gen);
+            lower<P>(out, gen, info);
             return "";
         }
         T2Ins in{};
@@ -1038,7 +1152,7 @@ std::string compile_fmt2(const TilePass &given, T2Pass *out, bool gen) {
         out->ins.push_back(in);
     }
     if (P::nmats(out) > (size_t)kT2SmemMats) return "more matrix records than the kernel's shared-memory copy";
-    lower(out, gen);
+    lower<P>(out, gen, info);
     return "";
 }
 

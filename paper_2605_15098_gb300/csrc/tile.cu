@@ -313,7 +313,7 @@ T2Off put_t2(Blob &blob, const T2Pass &t) {
     o.layx = blob.put_vec(t.layx);
     o.epi = blob.put(&t.epi, sizeof(T2Epilogue));
     // a complex128 programme's FP64 records take the places of the FP32 ones
-    o.mats = t.wide ? blob.put_vec(t.mats64) : t.format == 2 ? blob.put_vec(t.dev_mats) : blob.put_vec(t.mats);
+    o.mats = t.wide ? blob.put_vec(t.dev_mats64) : t.format == 2 ? blob.put_vec(t.dev_mats) : blob.put_vec(t.mats);
     if (t.format != 2) o.fac = blob.put_vec(t.factors);  // format 2: in the steps
     o.stat = blob.put_vec(t.stat);
     o.statc = t.wide ? blob.put_vec(t.statc64) : blob.put_vec(t.statc);

@@ -417,6 +417,24 @@ __device__ __forceinline__ void t2_run(const T2Args &a, Ins ins, float4 *gstate,
             apply_factor_bit(r, j ? 1 << (j - 1) : 0, ff.x, ff.y);
             continue;
         }
+        if (hd == kT2HdSigns) {
+            const uint32_t mask = (uint32_t)w.y & 31u;
+            const int *words = reinterpret_cast<const int *>(mrec);
+#define SV_SIGN(J)                                                                     \
+    if (mask & (1u << J)) {                                                            \
+        const int v = words[J], sl = v >> 16;                                          \
+        uint32_t sg = (uint32_t)__popc(tid & v & 0xffff) << 31;                        \
+        if (sl >= 0) sg ^= __float_as_uint(slotc[sl].x) & 0x80000000u;                 \
+        reg_sign<J>(r, __uint_as_float(0x3f800000u | sg));                             \
+    }
+            SV_SIGN(1)
+            SV_SIGN(2)
+            SV_SIGN(3)
+            SV_SIGN(4)
+            SV_SIGN(0)
+#undef SV_SIGN
+            continue;
+        }
         switch (hd) {
             case kT2HdStage: {
                 const bool local = (w.y & 1) != 0;  // within the warps (tileprog.h)
@@ -1314,7 +1332,7 @@ void t2_fill_args(const T2Pass &p, const T2Device &d, int n, T2Args *a) {
     a->nins = (int)p.dev.size();
     a->nrows = (int)((p.wide ? p.statc64.size() : p.statc.size()) / (2 * (size_t)p.threads));
     a->nslots = (int)p.slots.size();
-    a->nmats = (int)(p.wide ? p.mats64.size() / 8 : p.dev_mats.size());
+    a->nmats = (int)(p.wide ? p.dev_mats64.size() / 8 : p.dev_mats.size());
     a->nstages = (int)p.stages.size();
     a->last_stage = p.dev_last_stage;
     // runs of the global bits: tile index bit i is the i-th lowest set bit of gmask

@@ -211,6 +211,18 @@ __device__ __forceinline__ void d_rot(RegsD &r, double k) {
     }
 }
 
+// The amplitudes with register bit J set times 1 or -1, `sg` the sign bit:
+// integer operations only, the FP64 pipe has none of it.
+template <int J>
+__device__ __forceinline__ void d_sign(RegsD &r, uint32_t sg) {
+#pragma unroll
+    for (int g = 0; g < 16; g++) {
+        const int b = lo_of<J>(g) | (1 << J);
+        r.re[b] = __hiloint2double(__double2hiint(r.re[b]) ^ (int)sg, __double2loint(r.re[b]));
+        r.im[b] = __hiloint2double(__double2hiint(r.im[b]) ^ (int)sg, __double2loint(r.im[b]));
+    }
+}
+
 // General 2x2 on register bit J for the pairs whose packed-pair index (r >> 1
 // of the lower register) is in `pm`, and with `odd` only for odd registers
 // (a control on register bit 0).
@@ -402,6 +414,24 @@ __device__ __forceinline__ void t2d_run(const T2Args &a, Ins ins, double2 *gstat
         if (hd == kT2HdFactor) {
             const int j = (w.x >> 16) & 0xff;
             d_factor_bit(r, j ? 1 << (j - 1) : 0, thread_factor(w));
+            continue;
+        }
+        if (hd == kT2HdSigns) {
+            const uint32_t mask = (uint32_t)w.y & 31u;
+            const int *words = reinterpret_cast<const int *>(mrec);
+#define SV_SIGN(J)                                                                        \
+    if (mask & (1u << J)) {                                                               \
+        const int v = words[J], sl = v >> 16;                                             \
+        uint32_t sg = (uint32_t)__popc(tid & v & 0xffff) << 31;                           \
+        if (sl >= 0) sg ^= (uint32_t)__double2hiint(slotc[sl].x) & 0x80000000u;           \
+        d_sign<J>(r, sg);                                                                 \
+    }
+            SV_SIGN(0)
+            SV_SIGN(1)
+            SV_SIGN(2)
+            SV_SIGN(3)
+            SV_SIGN(4)
+#undef SV_SIGN
             continue;
         }
         switch (hd) {

@@ -370,6 +370,22 @@ __device__ __forceinline__ void reg_u2(RegsN<NP> &r, uint32_t qm, const float *m
     }
 }
 
+// The amplitudes with register bit J set times g (1 or -1).
+template <int J, int NP>
+__device__ __forceinline__ void reg_sign(RegsN<NP> &r, float g) {
+#pragma unroll
+    for (int i = 0; i < (J >= 1 ? NP / 2 : NP); i++) {
+        if constexpr (J >= 1) {
+            const int q1 = bfly_q<J>(i) | (1 << (J - 1));
+            r.re[q1] = mul2(r.re[q1], f2(g));
+            r.im[q1] = mul2(r.im[q1], f2(g));
+        } else {
+            r.re[i].y *= g;
+            r.im[i].y *= g;
+        }
+    }
+}
+
 // Rotation [[c, -s], [s, c]] (c >= 0) on register bit J as three in-place
 // shears: a += t b, b += s a, a += t b with t = -s / (1 + c) = (c - 1) / s
 // (exactly the rotation); each shear is one multiply-add per plane and no

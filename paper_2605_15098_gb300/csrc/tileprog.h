@@ -224,6 +224,10 @@ constexpr int kT2HdStage = 1, kT2HdScale = 2, kT2HdDiag = 3;
 //    Factor (idx = 1 + register bit or 0, cidx = slot, e0 = static row,
 //    e1 = slot of the lowest dynamic thread bit, aux = dynamic thread bits;
 //    -1 = none);
+//  * Signs: the run's factors on register bits that are signs (CZ terms): cidx =
+//    their register bits, aux = a record of one word per register bit, bits
+//    0..15 the thread bits whose parity is the sign, bits 16..31 the slot whose
+//    sign joins it (-1 = none);
 //  * Stage: cidx = 1: the change stays within the warps (the layouts before and
 //    after have the same warp bits);
 //  * Scale holds its factor: complex64 hi in aux and lo in (e0, e1) as FP32
@@ -232,7 +236,7 @@ constexpr int kT2HdStage = 1, kT2HdScale = 2, kT2HdDiag = 3;
 // [[k, -1], [1, k]] with k = c / s, whichever has |k| <= 1: two multiply-adds
 // per pair and component instead of three (the FP64 pipe bounds that kernel);
 // the product of the divisors joins the closing scale.
-constexpr int kT2HdRots = 4, kT2HdTable = 5, kT2HdFactor = 6, kT2HdRots4 = 7;
+constexpr int kT2HdRots = 4, kT2HdTable = 5, kT2HdFactor = 6, kT2HdRots4 = 7, kT2HdSigns = 8;
 constexpr int kT2DevIns = 256;  // at most kT2SmemIns steps and kT2SmemFactors factors
 
 // Write-back offsets of the final layout in the global state (amplitudes),
