@@ -519,76 +519,112 @@ k_normalise(double *__restrict__ p, uint64_t len, const ReadResult *__restrict__
     }
 }
 
-// CDF, step 1: the running sums of each block of 1024 outcomes, in index
-// order: one lane per block, 32 blocks per warp.  The warp loads 32 outcomes
-// of each of its blocks at a time (whole 256-byte rows, the next ones while it
-// adds), and each lane keeps its running sum at every 32nd outcome (chk)
-// and at the end (btot).  One addition after the other bounds it: 70 us for
-// 2^20 outcomes; reading them from each lane's own row and writing the whole
-// CDF took 160 us.
-constexpr int kCdfBlock = 1024, kCdfStep = 32;
-__global__ void __launch_bounds__(32)
-k_cdf_blocks(const double *__restrict__ p, uint64_t len, double *__restrict__ chk, double *__restrict__ btot) {
-    __shared__ double sh[32][33];
-    const int lane = threadIdx.x;
-    const uint64_t b0 = (uint64_t)blockIdx.x * 32;
-    double nxt[32];
-    auto load = [&](int c) {
-#pragma unroll
-        for (int k = 0; k < 32; k++) {
-            const uint64_t i = (b0 + k) * kCdfBlock + c * kCdfStep + lane;
-            nxt[k] = i < len ? p[i] : 0.0;
+// Running FP64 sums of non-negative values in order, 32 at a time: lane k adds
+// x to the sum of everything before it, every addition rounded to nearest as
+// one addition after the other rounds it.  While the sum stays in one binade
+// a value adds a whole number of the sum's last places, whatever the sum is,
+// so the 32 steps are a prefix sum of integers on the sum's bit pattern.  The
+// exceptions take an FP64 addition of their own, and the lanes after it start
+// again from its result: a tie (its direction depends on the sum), a value
+// above the sum's binade, a step out of the binade, a sum that is not a
+// normal number.  Zeros change nothing and are never exceptions.
+//
+// total: the sum so far, the same in every lane, on return the sum with all
+// 32 values; returns the sum up to and including the lane's own value.
+__device__ __forceinline__ double warp_run(double &total, double x, int lane) {
+    uint64_t c = (uint64_t)__double_as_longlong(total), mine = c;
+    const uint64_t xb = (uint64_t)__double_as_longlong(x);
+    const int ex = (int)(xb >> 52);
+    const uint64_t m = (xb & ((UINT64_C(1) << 52) - 1)) | (ex ? UINT64_C(1) << 52 : 0);
+    for (int pos = 0; pos < 32;) {
+        const int e = (int)(c >> 52);
+        const int de = e - (ex ? ex : 1);
+        bool bad = false;
+        uint64_t s = 0;
+        if (lane >= pos && xb) {
+            const int d = de < 0 ? 0 : de > 63 ? 63 : de;
+            const uint64_t q = m >> d, rest = (m - (q << d)) << 1, one = UINT64_C(1) << d;
+            bad = e < 1 || e > 0x7fe || de < 0 || rest == one;
+            s = bad ? 0 : q + (rest > one);
         }
-    };
-    load(0);
-    double run = 0.0;
-    const uint64_t b = b0 + lane;
-    const bool mine = b * kCdfBlock < len;
-    for (int c = 0; c < kCdfBlock / kCdfStep; c++) {
 #pragma unroll
-        for (int k = 0; k < 32; k++) sh[k][lane] = nxt[k];
-        __syncwarp();
-        if (c + 1 < kCdfBlock / kCdfStep) load(c + 1);
-        if (mine) chk[b * (kCdfBlock / kCdfStep) + c] = run;
-        double x[32];
-#pragma unroll
-        for (int k = 0; k < 32; k++) x[k] = sh[lane][k];
-#pragma unroll
-        for (int k = 0; k < 32; k++) run += x[k];  // outcomes beyond len are 0
-        __syncwarp();
+        for (int w = 1; w < 32; w <<= 1) {
+            const uint64_t y = __shfl_up_sync(0xffffffffu, s, w);
+            if (lane >= w) s += y;
+        }
+        const uint64_t after = c + s;
+        bad = bad || (lane >= pos && (int)(after >> 52) != e);
+        const unsigned stop = __ballot_sync(0xffffffffu, bad);
+        const int first = stop ? __ffs((int)stop) - 1 : 32;
+        if (lane >= pos && lane < first) mine = after;
+        // lanes below pos add nothing, so lane first - 1 has the sum before
+        // the exception (c itself when that is the first lane of this round)
+        const uint64_t last = __shfl_sync(0xffffffffu, after, first ? first - 1 : 0);
+        c = first > pos ? last : c;
+        if (first < 32) {
+            const double xf = __shfl_sync(0xffffffffu, x, first);
+            c = (uint64_t)__double_as_longlong(__dadd_rn(__longlong_as_double((long long)c), xf));
+            if (lane == first) mine = c;
+        }
+        pos = first + 1;
     }
-    if (mine) btot[b] = run;
+    total = __longlong_as_double((long long)c);
+    return __longlong_as_double((long long)mine);
+}
+
+// CDF, step 1: running sums of blocks of 1024 outcomes in index order.  One
+// warp takes a block, 32 consecutive outcomes at a time (warp_run), and keeps
+// the running sum at every 32nd outcome (chk) and at the end (btot).  The
+// latency of the shuffles bounds it, about 45 prefix sums per block: 18 us for
+// 2^20 outcomes.  With one FP64 addition after the other (about 90 cycles
+// each) a lane per block took 70 us.
+constexpr int kCdfBlock = 1024, kCdfStep = 32, kCdfAhead = 4;
+__global__ void __launch_bounds__(kRedThreads)
+k_cdf_blocks(const double *__restrict__ p, uint64_t len, double *__restrict__ chk, double *__restrict__ btot) {
+    constexpr int steps = kCdfBlock / kCdfStep;
+    const int lane = threadIdx.x & 31;
+    const uint64_t b = (uint64_t)blockIdx.x * (kRedThreads / 32) + (threadIdx.x >> 5);
+    if (b * kCdfBlock >= len) return;  // the whole warp
+    auto value = [&](int c) {
+        const uint64_t i = b * kCdfBlock + c * kCdfStep + lane;
+        return c < steps && i < len ? p[i] : 0.0;  // outcomes beyond len add nothing
+    };
+    double run = 0.0, nxt[kCdfAhead];
+#pragma unroll
+    for (int k = 0; k < kCdfAhead; k++) nxt[k] = value(k);
+    for (int c = 0; c < steps; c += kCdfAhead) {
+#pragma unroll
+        for (int k = 0; k < kCdfAhead; k++) {
+            const double x = nxt[k];
+            nxt[k] = value(c + kCdfAhead + k);
+            if (lane == 0) chk[b * steps + c + k] = run;
+            warp_run(run, x, lane);
+        }
+    }
+    if (lane == 0) btot[b] = run;
 }
 
 // CDF, step 2: before[b] = running total of the blocks before b, in block
-// order; before[nb] = C_last.  One addition after the other (about 90 cycles
-// each: 48 us for 1024 blocks, 107 us when each waited for its load too); the
-// loads and stores go through shared memory, 1024 blocks at a time.
-__global__ void __launch_bounds__(kRedThreads)
+// order; before[nb] = C_last: one warp, 32 blocks at a time: 15 us for 1024
+// blocks, against 48 us with one addition after the other.
+__global__ void __launch_bounds__(32)
 k_cdf_scan(const double *__restrict__ btot, uint64_t nb, double *__restrict__ before) {
-    __shared__ double in[1024], out[1024];
-    double run = 0.0;
-    for (uint64_t c = 0; c < nb; c += 1024) {
-        const int m = (int)(nb - c < 1024 ? nb - c : 1024);
-        for (int i = threadIdx.x; i < 1024; i += kRedThreads) in[i] = i < m ? btot[c + i] : 0.0;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            for (int i = 0; i < m; i += 16) {
-                double x[16];
+    const int lane = threadIdx.x;
+    auto value = [&](uint64_t i) { return i + lane < nb ? btot[i + lane] : 0.0; };
+    double run = 0.0, nxt[kCdfAhead];
+    if (lane == 0) before[0] = 0.0;
 #pragma unroll
-                for (int k = 0; k < 16; k++) x[k] = in[i + k];  // zeros beyond m
+    for (int k = 0; k < kCdfAhead; k++) nxt[k] = value(32 * k);
+    for (uint64_t c = 0; c < nb; c += 32 * kCdfAhead) {
 #pragma unroll
-                for (int k = 0; k < 16; k++) {
-                    out[i + k] = run;
-                    run += x[k];
-                }
-            }
+        for (int k = 0; k < kCdfAhead; k++) {
+            const uint64_t i = c + 32 * k;
+            const double x = nxt[k];
+            nxt[k] = value(i + 32 * kCdfAhead);
+            const double after = warp_run(run, x, lane);
+            if (i + lane < nb) before[i + lane + 1] = after;
         }
-        __syncthreads();
-        for (int i = threadIdx.x; i < m; i += kRedThreads) before[c + i] = out[i];
-        __syncthreads();
     }
-    if (threadIdx.x == 0) before[nb] = run;
 }
 
 // CDF, step 3: the smallest i with C_i > u * C_last, where C_i = (total before
@@ -837,9 +873,9 @@ sv_status sample_device(sv_state *h, const double *dev_p, uint64_t len, const do
     double *before = reinterpret_cast<double *>(base + off_be);
     double *du = reinterpret_cast<double *>(base + off_u);
     uint64_t *dout = reinterpret_cast<uint64_t *>(base + off_o);
-    k_cdf_blocks<<<blocks_for(nb, 32), 32, 0, h->stream>>>(dev_p, len, chk, bt);
+    k_cdf_blocks<<<blocks_for(nb, kRedThreads / 32), kRedThreads, 0, h->stream>>>(dev_p, len, chk, bt);
     SV_CUDA(cudaGetLastError());
-    k_cdf_scan<<<1, kRedThreads, 0, h->stream>>>(bt, nb, before);
+    k_cdf_scan<<<1, 32, 0, h->stream>>>(bt, nb, before);
     SV_CUDA(cudaGetLastError());
     SV_CUDA(cudaMemcpyAsync(du, host_u, shots * sizeof(double), cudaMemcpyHostToDevice, h->stream));
     k_sample<<<blocks_for(shots, 64), 64, 0, h->stream>>>(dev_p, len, before, chk, du, shots, dout);

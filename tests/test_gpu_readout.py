@@ -56,3 +56,30 @@ def test_ties_take_the_lowest_index(sv):
             s.apply(C.gates([C.h(q) for q in range(n)]))
             idx, p = s.argmax(mask)
         assert idx == 0 and p == 2.0 ** -bin(mask).count("1")
+
+
+@pytest.mark.parametrize("n", [5, 10, 12, 15, 21])
+@pytest.mark.parametrize("kind", ["uniform", "sparse", "binades", "dyadic", "growing", "tiny"])
+def test_samples_follow_the_running_sums(sv, orc, n, kind):
+    """Running sums with ties, steps out of the binade at many places, zeros, and
+    values above the sum so far: samples equal the oracle's, also at the CDF's own values."""
+    rng = np.random.default_rng(n)
+    size = 1 << n
+    a = {"uniform": lambda: np.ones(size),
+         "sparse": lambda: (rng.random(size) < 0.01) * rng.random(size),
+         "binades": lambda: np.ldexp(rng.random(size), rng.integers(-60, 60, size)),
+         "dyadic": lambda: np.ldexp(1.0, rng.integers(0, 12, size)),
+         "growing": lambda: np.ldexp(1.0 + rng.random(size), np.arange(size) * 200 // size),
+         "tiny": lambda: np.where(np.arange(size) < size // 2, 1e-160, 1.0)}[kind]()
+    a[-1] = max(a[-1], 1e-3)
+    psi = (a / np.linalg.norm(a)).astype(np.complex128)
+    mask = size - 1
+    with sv.State(n, sv.SV_C128) as s:
+        sv.sv_copy_in(s.h, psi)
+        p = s.probabilities(mask)
+        c = np.cumsum(p)
+        at = c[rng.integers(0, size, 200)] / c[-1]
+        u = np.minimum(np.concatenate([rng.random(300), at, np.nextafter(at, 0.0)]), np.nextafter(1.0, 0.0))
+        got = s.sample(mask, u)
+    want, _ = orc.sample(p, u)
+    assert np.array_equal(got, want)
