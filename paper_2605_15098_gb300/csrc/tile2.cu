@@ -1015,6 +1015,7 @@ __global__ void __launch_bounds__(kT2Threads, 2) k_batch(float *__restrict__ sta
         // straight from registers
         if (!ga.gen && tid < 32) {
             fence_async_global();
+            fence_tensor_map(ga.map);  // for all copies of this pass: warp 0 issues them
             issue_tile_load<kT2Qubits>(ga, ga.map, sm, t0, tile_base(ga, t0), bar, tid);
         }
         load_programme<kT2Qubits>(ga, sm, tid, blockDim.x);

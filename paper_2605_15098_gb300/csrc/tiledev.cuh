@@ -72,6 +72,12 @@ __device__ __forceinline__ void tensor_g2s(void *dst, const CUtensorMap *map, co
         "l"(map), "r"(x[0]), "r"(x[1]), "r"(x[2]), "r"(x[3]), "r"(x[4]), "r"(saddr(bar))
         : "memory");
 }
+// Before the first copy through a tensor map that lies in global memory: the
+// copy engine keeps descriptors it has read, and an earlier allocation at this
+// address may have held another map.  (Maps in the parameter block need none.)
+__device__ __forceinline__ void fence_tensor_map(const CUtensorMap *map) {
+    asm volatile("fence.proxy.tensormap::generic.acquire.sys [%0], 128;" ::"l"(map) : "memory");
+}
 // The copies of the tile whose global bits are `wbase` (8-byte words), by the
 // lanes of one warp: one tensor copy for each value of the bits beyond the
 // box's dimensions.  One copy of the whole tile instead of one per chunk of
