@@ -152,9 +152,14 @@ k_u2q(R *__restrict__ s, uint64_t units, Ins in, uint64_t ma, uint64_t mb, C4<R>
     }
 }
 
-// Sums of squares of one value of the measured qubit.  complex64: exact FP32
-// squares in a double-float pair (product and fmaf remainder, error-free
-// sums), moved to FP64 every few amplitudes; complex128: FP64.
+// Sum of squares of one value of the measured qubit.  complex128: FP64.
+// complex64: summed in FP32 without error (exact squares as product and fmaf
+// remainder; sums and their remainders as an unevaluated sum of three), which
+// is good to the FP64 it becomes; FP64 issues at 1/64 of the FP32 rate, so
+// that its conversions and additions are made once per thread.  Where the sum
+// lies outside [2^-90, 2^120] this does not hold: a square's remainder goes
+// below 2^-149, or a square above the FP32 range.  keep() then takes the last
+// vectors out again and is false, and the caller adds them in FP64.
 template <typename R>
 struct Squares {
     double sr = 0.0, si = 0.0;
@@ -162,30 +167,46 @@ struct Squares {
         sr = fma(re, re, sr);
         si = fma(im, im, si);
     }
-    __device__ void flush() {}
+    __device__ bool keep(const Squares &) { return true; }
+    __device__ void add_wide(R, R) {}
     __device__ double value() const { return sr + si; }
 };
 template <>
 struct Squares<float> {
-    double acc = 0.0;
-    float hi = 0.f, lo = 0.f;
-    __device__ void sum(float b) {
-        const float t = hi + b, bb = t - hi;
-        lo += (hi - (t - bb)) + (b - bb);
-        hi = t;
+    double wide = 0.0;
+    float s0 = 0.f, s1 = 0.f, s2 = 0.f;
+    // s <- fl(s + b); returns the rounding's remainder
+    __device__ static float two_sum(float &s, float b) {
+        const float t = s + b, bb = t - s;
+        const float e = (s - (t - bb)) + (b - bb);
+        s = t;
+        return e;
+    }
+    __device__ void square(float x) {
+        const float p = __fmul_rn(x, x);  // not contracted into the sum
+        const float e = two_sum(s1, two_sum(s0, p));
+        s2 += e + two_sum(s1, fmaf(x, x, -p));
     }
     __device__ void add(float re, float im) {
-        const float pr = re * re, pi = im * im;
-        lo += fmaf(re, re, -pr) + fmaf(im, im, -pi);
-        sum(pr);
-        sum(pi);
+        square(re);
+        square(im);
     }
-    __device__ void flush() {
-        acc += (double)hi + (double)lo;
-        hi = lo = 0.f;
+    // `before`: the sum before the vectors since the last call
+    __device__ bool keep(const Squares &before) {
+        if (s0 >= 0x1p-90f && s0 <= 0x1p120f) return true;
+        *this = before;
+        return false;
     }
-    __device__ double value() const { return acc; }
+    __device__ void add_wide(float re, float im) {
+        wide = fma((double)re, (double)re, wide);
+        wide = fma((double)im, (double)im, wide);
+    }
+    __device__ double value() const { return wide + ((double)s0 + ((double)s1 + (double)s2)); }
 };
+
+// Whether a vector has a component other than zero.
+__device__ __forceinline__ bool nonzero(float4 v) { return v.x != 0.f || v.y != 0.f || v.z != 0.f || v.w != 0.f; }
+__device__ __forceinline__ bool nonzero(double2) { return false; }  // FP64 sums are always kept
 
 // Sum over a block by a fixed tree; the result in thread 0.
 __device__ __forceinline__ double block_sum(double x) {
@@ -216,6 +237,7 @@ k_meas_decide(const R *__restrict__ s, uint64_t units, int pos, uint64_t tbit, b
     using T = typename Vec<R, VB>::T;
     __shared__ bool last;
     const T *v = reinterpret_cast<const T *>(s);
+    auto at = [&](uint64_t i) { return intra ? i : ((i >> pos) << (pos + 1)) | (i & ((UINT64_C(1) << pos) - 1)); };
     Squares<R> s0, s1;
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
     for (uint64_t u0 = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; u0 < units; u0 += stride * kItems) {
@@ -225,10 +247,11 @@ k_meas_decide(const R *__restrict__ s, uint64_t units, int pos, uint64_t tbit, b
             const uint64_t i = u0 + k * stride;
             a[k] = b[k] = T{};
             if (i >= units) continue;
-            const uint64_t x = intra ? i : ((i >> pos) << (pos + 1)) | (i & ((UINT64_C(1) << pos) - 1));
+            const uint64_t x = at(i);
             a[k] = v[x];
             if (!intra) b[k] = v[x | tbit];
         }
+        const Squares<R> was0 = s0, was1 = s1;
 #pragma unroll
         for (int k = 0; k < kItems; k++) {
             const R *pa = reinterpret_cast<const R *>(&a[k]), *pb = reinterpret_cast<const R *>(&b[k]);
@@ -243,8 +266,29 @@ k_meas_decide(const R *__restrict__ s, uint64_t units, int pos, uint64_t tbit, b
                 }
             }
         }
-        s0.flush();
-        s1.flush();
+        const bool ok0 = s0.keep(was0), ok1 = s1.keep(was1);
+        if (ok0 && ok1) continue;
+        // (a vector of zeros, in the half an earlier measurement cleared, adds
+        // nothing; the vectors are read again: kept, they cost a resident block)
+#pragma unroll 1
+        for (int k = 0; k < kItems; k++) {
+            const uint64_t i = u0 + k * stride;
+            if (i >= units) break;
+            const uint64_t x = at(i);
+            const T wa = v[x], wb = intra ? T{} : v[x | tbit];
+            const R *pa = reinterpret_cast<const R *>(&wa), *pb = reinterpret_cast<const R *>(&wb);
+            if (intra) {
+                if (!nonzero(wa)) continue;
+                if (!ok0) s0.add_wide(pa[0], pa[1]);
+                if (VB && !ok1) s1.add_wide(pa[VB * 2], pa[VB * 2 + 1]);
+                continue;
+            }
+#pragma unroll
+            for (int e = 0; e < (1 << VB); e++) {
+                if (!ok0 && nonzero(wa)) s0.add_wide(pa[2 * e], pa[2 * e + 1]);
+                if (!ok1 && nonzero(wb)) s1.add_wide(pb[2 * e], pb[2 * e + 1]);
+            }
+        }
     }
     double p0 = block_sum(s0.value()), p1 = block_sum(s1.value());
     if (threadIdx.x == 0) {
