@@ -98,6 +98,8 @@ struct PlanOptions {
 
 // Planner options of a configuration (library defaults filled in).
 PlanOptions plan_options(int n, sv_dtype dt, const sv_config &cfg);
+// The same for a gate list.
+PlanOptions plan_options(int n, sv_dtype dt, const sv_config &cfg, const std::vector<sv_gate> &gates);
 
 struct Plan {
     std::vector<TilePass> passes;

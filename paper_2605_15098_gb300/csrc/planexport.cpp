@@ -151,13 +151,13 @@ extern "C" sv_status sv_plan_export(int n, sv_dtype dt, const int *host_phys_of_
     sv_config c{};
     if (cfg) c = *cfg;
     const bool dbl = dt == SV_C128;
-    PlanOptions opt = plan_options(n, dt, c);
+    std::vector<sv_gate> gl(host_gates, host_gates + m);
+    PlanOptions opt = plan_options(n, dt, c, gl);
     int phys[64];
     for (int q = 0; q < 64; q++) phys[q] = q;
     if (host_phys_of_logical)
         for (int q = 0; q < n; q++) phys[q] = host_phys_of_logical[q];
     Plan plan;
-    std::vector<sv_gate> gl(host_gates, host_gates + m);
     std::string err = build_plan(gl, opt, phys, &plan);
     if (!err.empty()) return fail(SV_ERR_ARG, "planner: %s", err.c_str());
     const bool allow_t2 = !dbl && !(c.flags & SV_FLAG_GENERIC_TILE);
@@ -169,7 +169,16 @@ extern "C" sv_status sv_plan_export(int n, sv_dtype dt, const int *host_phys_of_
     j.raw(",\"passes\":[");
     bool first = true, first_pass = true;
     std::vector<char> eligible;  // register-stage, format 2, 2^13 tiles: may join an L2 block group
-    for (const TilePass &p : plan.passes) {
+    for (size_t pi = 0; pi < plan.passes.size(); pi++) {
+        T2Pass t2;
+        std::string why = "disabled";
+        if (dbl && !(c.flags & SV_FLAG_GENERIC_TILE) && opt.k == kT2Qubits && !plan.passes[pi].ops.empty()) {
+            // complex128 on 2^13-amplitude tiles: the FP64 register-stage
+            // kernel (its programme is the emulator's business only through the ops)
+            do why = compile_t2v2_c128(plan.passes[pi], &t2, false);
+            while (!why.empty() && opt.split_u3 && cut_pass(&plan.passes, pi));
+        }
+        const TilePass &p = plan.passes[pi];
         eligible.push_back(0);
         if (!first) j.raw(",");
         first = false;
@@ -230,9 +239,7 @@ extern "C" sv_status sv_plan_export(int n, sv_dtype dt, const int *host_phys_of_
             j.raw("]}");
             continue;
         }
-        T2Pass t2;
         const bool fused = c.mode == SV_MODE_FUSED;
-        std::string why = "disabled";
         const char *kname = "t2";
         if (allow_t2 && !p.ops.empty()) {
             why = fused ? compile_t2(p, &t2, true) : "not fused";
@@ -247,23 +254,18 @@ extern "C" sv_status sv_plan_export(int n, sv_dtype dt, const int *host_phys_of_
                 kname = "t2";
             }
         }
-        if (dbl && !(c.flags & SV_FLAG_GENERIC_TILE) && p.k == kT2Qubits && !p.ops.empty()) {
-            // complex128 on 2^13-amplitude tiles: the FP64 register-stage kernel
-            // (its programme is the emulator's business only through the ops)
-            why = compile_t2v2_c128(p, &t2, false);
-            if (why.empty()) {
-                j.raw(",\"kernel\":\"t2d\",\"t2d\":");
-                put_t2(j, t2);
-                if (first_ops) {
-                    T2Pass g;
-                    if (compile_t2v2_c128(p, &g, true).empty()) {
-                        j.raw(",\"t2dgen\":");
-                        put_t2(j, g);
-                    }
+        if (dbl && why.empty()) {
+            j.raw(",\"kernel\":\"t2d\",\"t2d\":");
+            put_t2(j, t2);
+            if (first_ops) {
+                T2Pass g;
+                if (compile_t2v2_c128(p, &g, true).empty()) {
+                    j.raw(",\"t2dgen\":");
+                    put_t2(j, g);
                 }
-                j.raw("}");
-                continue;
             }
+            j.raw("}");
+            continue;
         }
         if (why.empty()) {
             eligible.back() = t2.format == 2 && p.k == kT2Qubits;

@@ -345,13 +345,12 @@ std::string build_plan_paper(const std::vector<sv_gate> &gates, const std::vecto
 
 }  // namespace
 
-// Whether the passes of a complex128 plan run on the register-stage kernel.
-// There a split U3 is two FP64 operations per amplitude and its phases join
-// the diagonal runs, against eight for the complex 2x2 (random circuit
-// n = 21, depth 10: 8.35 -> 3.38 ms); the generic tile kernel's diagonal runs
-// cost more than they save.  The error against a reference that does not round
-// phi + lambda halves (n = 20, depth 12: 4.7e-15 -> 1.7e-15).
-bool c128_register_stage(const PlanOptions &opt, int flags) {
+// Whether the passes of a complex128 plan run on the register-stage kernel (a
+// pass too long for it is cut, cut_pass).  There a split U3 is two FP64
+// operations per amplitude and its phases join the diagonal runs, against
+// eight for the complex 2x2 (random circuit n = 21, depth 10: 8.35 -> 3.38
+// ms); the generic tile kernel's diagonal runs cost more than they save.
+static bool c128_register_stage(const PlanOptions &opt, int flags) {
     return opt.n >= 13 && opt.k == 13 && opt.c >= 4 && opt.merge_diag && !(flags & SV_FLAG_GENERIC_TILE);
 }
 
@@ -371,6 +370,15 @@ PlanOptions plan_options(int n, sv_dtype dt, const sv_config &cfg) {
     if (opt.paper) opt.c = opt.k;  // the block is contiguous
     if ((cfg.flags & SV_FLAG_NARROW_FIRST) && !opt.paper) opt.first_c = 4;
     opt.split_u3 = !dbl || c128_register_stage(opt, cfg.flags);
+    return opt;
+}
+
+PlanOptions plan_options(int n, sv_dtype dt, const sv_config &cfg, const std::vector<sv_gate> &gates) {
+    PlanOptions opt = plan_options(n, dt, cfg);
+    // a SWAP executed in the tile keeps its pass on the generic tile kernel
+    if (dt == SV_C128 && !opt.relabel)
+        for (const sv_gate &g : gates)
+            if (g.kind == SV_SWAP) opt.split_u3 = false;
     return opt;
 }
 

@@ -1165,4 +1165,21 @@ std::string compile_t2v2_c128(const TilePass &tp, T2Pass *out, bool gen) {
     return compile_fmt2<P64>(tp, out, gen);
 }
 
+bool cut_pass(std::vector<TilePass> *passes, size_t i) {
+    const TilePass &whole = (*passes)[i];
+    const size_t steps = whole.ops.size(), half = steps / 2;
+    if (steps < 2) return false;
+    for (const TileOp &op : whole.ops)
+        if (op.type == TOP_SWAP) return false;
+    TilePass rest = whole;
+    rest.remap_before.clear();
+    rest.ops.erase(rest.ops.begin(), rest.ops.begin() + (long)half);
+    rest.ngates = (int)((size_t)whole.ngates * (steps - half) / steps);
+    TilePass &head = (*passes)[i];
+    head.ops.resize(half);
+    head.ngates -= rest.ngates;
+    passes->insert(passes->begin() + (long)i + 1, std::move(rest));
+    return true;
+}
+
 }  // namespace sv

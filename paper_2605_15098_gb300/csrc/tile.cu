@@ -485,7 +485,7 @@ static std::string plan_key(const sv_state *h, const std::vector<sv_gate> &gates
 static sv_status compiled_plan(sv_state *h, const std::vector<sv_gate> &gates, const sv_config &cfg,
                                const PlanOverride *ov, std::shared_ptr<CompiledPlan> *out) {
     const bool dbl = h->dt == SV_C128;
-    PlanOptions opt = ov ? ov->opt : plan_options(h->n, h->dt, cfg);
+    PlanOptions opt = ov ? ov->opt : plan_options(h->n, h->dt, cfg, gates);
     if (dbl && opt.k > 13) return fail(SV_ERR_ARG, "complex128 tiles hold at most 2^13 amplitudes");
     std::string key = plan_key(h, gates, cfg, opt, ov);
     const uint64_t hash = key_hash(key.data(), key.size());
@@ -522,6 +522,15 @@ static sv_status compiled_plan(sv_state *h, const std::vector<sv_gate> &gates, c
         return fail(SV_ERR_STATE, "internal: learned plan does not match the planner's passes");
     bool first_pass = true;  // the pass that may start from a recorded basis state
     for (size_t i = 0; i < plan.passes.size(); i++) {
+        std::string why;  // complex128: why the pass does not compile
+        if (dbl && allow_t2 && !ov && !plan.passes[i].ops.empty()) {
+            why = compile_t2v2_c128(plan.passes[i], &t2[i], false);
+            while (!why.empty() && opt.split_u3 && cut_pass(&plan.passes, i)) {
+                t2.emplace(t2.begin() + (long)i + 1);
+                up.emplace(up.begin() + (long)i + 1);
+                why = compile_t2v2_c128(plan.passes[i], &t2[i], false);
+            }
+        }
         const TilePass &p = plan.passes[i];
         if (!p.general.empty()) first_pass = false;  // the step writes the state first
         if (p.ops.empty()) continue;
@@ -530,7 +539,8 @@ static sv_status compiled_plan(sv_state *h, const std::vector<sv_gate> &gates, c
         const int want = ov ? ov->kernel[i] : (!allow_t2 ? PK_GENERIC : fused && !dbl ? PK_T3 : PK_T2);
         bool ok = false;
         if (dbl) {
-            if (want != PK_GENERIC && allow_t2 && compile_t2v2_c128(p, &t2[i], false).empty()) {
+            if (ov && want != PK_GENERIC && allow_t2) why = compile_t2v2_c128(p, &t2[i], false);
+            if (want != PK_GENERIC && allow_t2 && why.empty()) {
                 ok = true;
                 if (first_ops) {
                     auto g = std::make_shared<T2Pass>();
