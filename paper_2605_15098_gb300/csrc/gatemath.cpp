@@ -123,16 +123,16 @@ uint64_t diag_turns64(const sv_gate &g, bool *exact) {
         case SV_CP: {
             *exact = false;
             // p / (2 pi) as an unevaluated sum (the product, its exact
-            // remainder and the tail of 1 / (2 pi)), so that the phase is
-            // good to 2^-64 of a turn whatever the angle's size
+            // remainder and the tail of 1 / (2 pi)), each part reduced
+            // exactly and rounded to 2^-64 of a turn: good to 2^-63 of a turn
+            // for |p| < 2^40 (beyond, the two words of 1 / (2 pi) end)
             const double inv_hi = 0x1.45f306dc9c883p-3, inv_lo = -0x1.6b01ec5417056p-57;
             const double hi = g.p[0] * inv_hi;
             const double lo = std::fma(g.p[0], inv_hi, -hi) + g.p[0] * inv_lo;
             if (!std::isfinite(hi)) return 0;
             auto turns = [](double x) -> uint64_t {  // x mod 1
-                if (std::fabs(x) < 0.25) return (uint64_t)(int64_t)std::llrint(std::ldexp(x, 64));
-                const double f = x - std::floor(x);
-                return f >= 1.0 ? 0 : (uint64_t)std::ldexp(f, 64);
+                const double f = std::rint(std::ldexp(x - std::rint(x), 64));
+                return std::fabs(f) < 0x1p63 ? (uint64_t)(int64_t)f : UINT64_C(1) << 63;  // +-1/2: the same
             };
             return turns(hi) + turns(lo);
         }
