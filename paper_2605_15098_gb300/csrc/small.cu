@@ -25,6 +25,7 @@
 #include <cooperative_groups.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstring>
 #include <vector>
@@ -254,12 +255,6 @@ sv_status launch_small(sv_state *h, int most, const std::vector<SmallGroup> &gro
     std::copy(groups.begin(), groups.end(), a.group);
     std::copy(ops.begin(), ops.end(), a.op);
     const size_t smem = (2 * sizeof(R) << a.nl) + sizeof(SmallGroup) * NO + sizeof(SmallOp<R>) * ops.size();
-    static bool configured = false;
-    if (!configured) {
-        SV_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * 1024));
-        SV_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-        configured = true;
-    }
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(1u << cl);
     cfg.blockDim = dim3(std::max(32, 1 << (a.nl - 3)));
@@ -292,35 +287,46 @@ constexpr int kManyOps = sizeof(R) == 4 ? 512 : 320;
 static_assert(sizeof(SmallArgs<float, kManyOps<float>>) <= 32000, "launch parameters");
 static_assert(sizeof(SmallArgs<double, kManyOps<double>>) <= 32000, "launch parameters");
 
-// log2 of the largest cluster the device can place with these resources.
+// Prepare the kernels for the current device (their attributes are the
+// device's own) and return the log2 of the largest cluster it can place with
+// these resources in *most.  Once per device: a second thread that comes at
+// the same time sets the same.
 template <typename R>
-int most_ctas() {
-    static const int most = [] {
-        auto kern = k_small<R, kManyOps<R>>;
-        const int smem = 128 * 1024;
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-        cudaLaunchConfig_t cfg{};
-        cfg.gridDim = dim3(1u << kMaxClusterLog);
-        cfg.blockDim = dim3(512);
-        cfg.dynamicSmemBytes = smem;
-        cudaLaunchAttribute at{};
-        at.id = cudaLaunchAttributeClusterDimension;
-        at.val.clusterDim.x = 1u << kMaxClusterLog;
-        at.val.clusterDim.y = at.val.clusterDim.z = 1;
-        cfg.attrs = &at;
-        cfg.numAttrs = 1;
-        int count = 0;
-        const bool ok = cudaOccupancyMaxActiveClusters(&count, kern, &cfg) == cudaSuccess && count > 0;
-        cudaGetLastError();
-        return ok ? kMaxClusterLog : 3;
-    }();
-    return most;
+sv_status prepare_small(int device, int *most) {
+    constexpr int kDevices = 64, kSmem = 128 * 1024;
+    static std::atomic<int8_t> known[kDevices];  // 0: not yet
+    if (device < kDevices && (*most = known[device].load(std::memory_order_acquire)) > 0) return SV_OK;
+    auto prepare = [](auto kern) -> sv_status {
+        SV_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem));
+        SV_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+        return SV_OK;
+    };
+    auto kern = k_small<R, kManyOps<R>>;
+    SV_TRY(prepare(kern));
+    SV_TRY(prepare(k_small<R, kFewOps<R>>));
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(1u << kMaxClusterLog);
+    cfg.blockDim = dim3(512);
+    cfg.dynamicSmemBytes = kSmem;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = 1u << kMaxClusterLog;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    int count = 0;
+    const bool ok = cudaOccupancyMaxActiveClusters(&count, kern, &cfg) == cudaSuccess && count > 0;
+    cudaGetLastError();
+    *most = ok ? kMaxClusterLog : 3;
+    if (device < kDevices) known[device].store((int8_t)*most, std::memory_order_release);
+    return SV_OK;
 }
 
 template <typename R>
 sv_status run_small(sv_state *h, const std::vector<sv_gate> &g) {
-    const int n = h->n, most = most_ctas<R>();
+    const int n = h->n;
+    int most = 0;
+    SV_TRY(prepare_small<R>(h->device, &most));
     const int nl = n - cluster_log(n, most);
     size_t i = 0;
     std::vector<SmallGroup> groups;
