@@ -46,14 +46,14 @@ uint64_t plan_key(const sv_state *h, const std::vector<sv_gate> &g, const sv_con
 
 struct Option {
     int family;
-    int rec;
+    std::vector<int> recs;  // its launches
 };
 
 struct Candidate {
     PlanOptions opt;
     std::vector<std::vector<Option>> pass_opts;  // per pass of the plan
     std::vector<int> remap_recs;
-    int passes = 0, remaps = 0;
+    int remaps = 0;
 };
 
 // The kernel partitioned_apply picks for a pass without an override.
@@ -82,10 +82,9 @@ sv_status learned_entry(sv_state *h, const std::vector<sv_gate> &gates, const sv
         return SV_OK;
     }
     const bool dbl = h->dt == SV_C128;
-    const bool allow_t2 = !dbl && !(cfg.flags & SV_FLAG_GENERIC_TILE);
-    const bool fused = cfg.mode == SV_MODE_FUSED;
-    PlanOptions base = plan_options(h->n, h->dt, cfg);
-    if (dbl) base.split_u3 = false;  // its candidates run on the generic tile kernel
+    const bool allow_t2 = !(cfg.flags & SV_FLAG_GENERIC_TILE);
+    const bool fused = cfg.mode == SV_MODE_FUSED && !dbl;
+    const PlanOptions base = plan_options(h->n, h->dt, cfg, gates);
     if (dbl && base.k > 13) return fail(SV_ERR_ARG, "complex128 tiles hold at most 2^13 amplitudes");
 
     // candidate planner options; the configuration's own options come first
@@ -97,12 +96,19 @@ sv_status learned_entry(sv_state *h, const std::vector<sv_gate> &gates, const sv
         o.paper = paper;
         o.late_diag = late;
         o.first_c = paper ? 0 : first_c;
+        o.split_u3 = u3_splits(o, h->dt, cfg.flags, gates);
         for (const PlanOptions &e : opts)
             if (e.k == o.k && e.c == o.c && e.paper == o.paper && e.late_diag == o.late_diag &&
                 e.first_c == o.first_c)
                 return;
         opts.push_back(o);
     };
+    // complex128: whether 2^13 tiles run on the FP64 register-stage kernel
+    PlanOptions wide = base;
+    wide.paper = false;
+    wide.k = kT2Qubits;
+    wide.c = 5;
+    const bool register_stage = dbl && allow_t2 && u3_splits(wide, h->dt, cfg.flags, gates);
     // every (k, c) with diagonal gates in their successors' passes and in
     // the first pass where they are ready
     auto add = [&](int k, int c, bool paper) {
@@ -114,6 +120,13 @@ sv_status learned_entry(sv_state *h, const std::vector<sv_gate> &gates, const sv
         for (int c : {6, 7, 8, 9}) add1(13, c, false, true, 4);  // a narrow first pass
         for (int c : {4, 5, 7}) add(14, c, false);
         add(13, 13, true);
+    } else if (register_stage) {
+        // The register-stage kernel can run it, two and a half to four times as
+        // fast as the generic one (QPE n = 20: 0.19 ms and 0.50 at the best
+        // tile, random n = 20 1.2 and 4.1, n = 22 12.4 and 39): no other
+        // candidates, because the model knows a generic pass by its number of
+        // gates only and takes 150 U3 gates of n = 23 (18.9 ms) for 3.1 ms.
+        for (int c : {4, 5}) add(13, c, false);
     } else {
         for (int k : {11, 12, 13})
             for (int c : {3, 4, 5}) add(k, c, false);
@@ -143,10 +156,32 @@ sv_status learned_entry(sv_state *h, const std::vector<sv_gate> &gates, const sv
             }
             std::vector<Option> po;
             if (!p.ops.empty()) {
-                cd.passes++;
-                po.push_back({PK_GENERIC, (int)recs.size()});
+                const Option generic{PK_GENERIC, {(int)recs.size()}};
                 recs.push_back(describe_pass(h->n, h->dt, p, nullptr, PK_GENERIC));
-                if (allow_t2) {
+                if (allow_t2 && dbl && o.k == kT2Qubits) {
+                    // the FP64 register-stage kernel, the pass cut as the library cuts it
+                    std::vector<TilePass> piece{p};
+                    std::vector<int> at;
+                    bool any = false;
+                    for (size_t j = 0; j < piece.size(); j++) {
+                        T2Pass a, g;
+                        const bool ok = compile_pass_c128(&piece, j, o.split_u3, &a).empty();
+                        const bool gen = ok && gen_next && !j && compile_t2v2_c128(piece[j], &g, true).empty();
+                        sv_launch_record rec =
+                            describe_pass(h->n, h->dt, piece[j], gen ? &g : &a, ok ? PK_T2 : PK_GENERIC);
+                        if (gen) {  // written only
+                            rec.bytes *= 0.5;
+                            rec.generated = 1;
+                        }
+                        any |= ok;
+                        at.push_back((int)recs.size());
+                        recs.push_back(rec);
+                    }
+                    po.push_back(any ? Option{PK_T2, at} : generic);
+                } else {
+                    po.push_back(generic);
+                }
+                if (allow_t2 && !dbl) {
                     T2Pass a, g;
                     if (compile_t2(p, &a, false).empty()) {
                         const bool gen = gen_next && a.format == 2 && compile_t2v2(p, &g, true).empty();
@@ -155,12 +190,12 @@ sv_status learned_entry(sv_state *h, const std::vector<sv_gate> &gates, const sv
                             rec.bytes *= 0.5;
                             rec.generated = 1;
                         }
-                        po.push_back({PK_T2, (int)recs.size()});
+                        po.push_back({PK_T2, {(int)recs.size()}});
                         recs.push_back(rec);
                     }
                     T2Pass b;
                     if (compile_t2(p, &b, true).empty()) {
-                        po.push_back({PK_T3, (int)recs.size()});
+                        po.push_back({PK_T3, {(int)recs.size()}});
                         recs.push_back(describe_pass(h->n, h->dt, p, &b, PK_T3));
                     }
                 }
@@ -180,13 +215,19 @@ sv_status learned_entry(sv_state *h, const std::vector<sv_gate> &gates, const sv
     for (size_t r = 0; r < recs.size(); r++)
         ms[r] = std::exp((double)y[r]) * recs[r].bytes * 1e-9;
 
+    auto time = [&](const Option &o) {
+        double t = 0.0;
+        for (int r : o.recs) t += ms[r];
+        return t;
+    };
+
     sv_state::Learned L;
     double best = 1e300, greedy = 0.0;
     for (size_t ci = 0; ci < cands.size(); ci++) {
         const Candidate &cd = cands[ci];
         double tot = 0.0, tot_rule = 0.0;
         std::vector<int8_t> kern, kern_rule;
-        int nfused = 0;
+        int nfused = 0, passes = 0;
         for (int r : cd.remap_recs) {
             tot += ms[r];
             tot_rule += ms[r];
@@ -199,14 +240,15 @@ sv_status learned_entry(sv_state *h, const std::vector<sv_gate> &gates, const sv
             }
             const Option *bo = &po[0];
             for (const Option &o : po)
-                if (ms[o.rec] < ms[bo->rec]) bo = &o;
-            tot += ms[bo->rec];
+                if (time(o) < time(*bo)) bo = &o;
+            tot += time(*bo);
+            passes += (int)bo->recs.size();
             kern.push_back((int8_t)bo->family);
             nfused += bo->family == PK_T3;
             const int rf = rule_family(po, allow_t2, fused);
             kern_rule.push_back((int8_t)rf);
             for (const Option &o : po)
-                if (o.family == rf) tot_rule += ms[o.rec];
+                if (o.family == rf) tot_rule += time(o);
         }
         if (ci == 0) greedy = tot_rule;
         if (tot < best) {
@@ -218,7 +260,7 @@ sv_status learned_entry(sv_state *h, const std::vector<sv_gate> &gates, const sv
             L.info.paper_swap = cd.opt.paper ? 1 : 0;
             L.info.early_diag = cd.opt.late_diag ? 0 : 1;
             L.info.narrow_first = cd.opt.first_c > 0 ? 1 : 0;
-            L.info.passes = cd.passes;
+            L.info.passes = passes;
             L.info.remaps = cd.remaps;
             L.info.fused_passes = nfused;
         }

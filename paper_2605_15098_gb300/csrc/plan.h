@@ -96,10 +96,11 @@ struct PlanOptions {
     int first_c = 0;        // chunk qubits of the list's first pass (0: c); SV_FLAG_NARROW_FIRST
 };
 
-// Planner options of a configuration (library defaults filled in).
-PlanOptions plan_options(int n, sv_dtype dt, const sv_config &cfg);
-// The same for a gate list.
+// Planner options of a configuration for a gate list (library defaults filled in).
 PlanOptions plan_options(int n, sv_dtype dt, const sv_config &cfg, const std::vector<sv_gate> &gates);
+// Their split_u3: always in complex64; in complex128 where the passes run on
+// the register-stage kernel.
+bool u3_splits(const PlanOptions &opt, sv_dtype dt, int flags, const std::vector<sv_gate> &gates);
 
 struct Plan {
     std::vector<TilePass> passes;

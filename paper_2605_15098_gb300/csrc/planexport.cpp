@@ -175,8 +175,7 @@ extern "C" sv_status sv_plan_export(int n, sv_dtype dt, const int *host_phys_of_
         if (dbl && !(c.flags & SV_FLAG_GENERIC_TILE) && opt.k == kT2Qubits && !plan.passes[pi].ops.empty()) {
             // complex128 on 2^13-amplitude tiles: the FP64 register-stage
             // kernel (its programme is the emulator's business only through the ops)
-            do why = compile_t2v2_c128(plan.passes[pi], &t2, false);
-            while (!why.empty() && opt.split_u3 && cut_pass(&plan.passes, pi));
+            why = compile_pass_c128(&plan.passes, pi, opt.split_u3, &t2);
         }
         const TilePass &p = plan.passes[pi];
         eligible.push_back(0);

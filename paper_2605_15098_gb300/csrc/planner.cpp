@@ -354,7 +354,16 @@ static bool c128_register_stage(const PlanOptions &opt, int flags) {
     return opt.n >= 13 && opt.k == 13 && opt.c >= 4 && opt.merge_diag && !(flags & SV_FLAG_GENERIC_TILE);
 }
 
-PlanOptions plan_options(int n, sv_dtype dt, const sv_config &cfg) {
+bool u3_splits(const PlanOptions &opt, sv_dtype dt, int flags, const std::vector<sv_gate> &gates) {
+    if (dt != SV_C128) return true;
+    // a SWAP executed in the tile keeps its pass on the generic tile kernel
+    if (!opt.relabel)
+        for (const sv_gate &g : gates)
+            if (g.kind == SV_SWAP) return false;
+    return c128_register_stage(opt, flags);
+}
+
+PlanOptions plan_options(int n, sv_dtype dt, const sv_config &cfg, const std::vector<sv_gate> &gates) {
     PlanOptions opt;
     opt.n = n;
     const bool dbl = dt == SV_C128;
@@ -369,16 +378,7 @@ PlanOptions plan_options(int n, sv_dtype dt, const sv_config &cfg) {
     opt.search = !(cfg.flags & SV_FLAG_GREEDY_ONLY);
     if (opt.paper) opt.c = opt.k;  // the block is contiguous
     if ((cfg.flags & SV_FLAG_NARROW_FIRST) && !opt.paper) opt.first_c = 4;
-    opt.split_u3 = !dbl || c128_register_stage(opt, cfg.flags);
-    return opt;
-}
-
-PlanOptions plan_options(int n, sv_dtype dt, const sv_config &cfg, const std::vector<sv_gate> &gates) {
-    PlanOptions opt = plan_options(n, dt, cfg);
-    // a SWAP executed in the tile keeps its pass on the generic tile kernel
-    if (dt == SV_C128 && !opt.relabel)
-        for (const sv_gate &g : gates)
-            if (g.kind == SV_SWAP) opt.split_u3 = false;
+    opt.split_u3 = u3_splits(opt, dt, cfg.flags, gates);
     return opt;
 }
 

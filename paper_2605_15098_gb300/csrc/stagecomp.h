@@ -236,13 +236,13 @@ std::string compile_t2v2(const TilePass &tp, T2Pass *out, bool gen);
 // 64-bit phases, FP64 matrices, tables and rows; 2^13-amplitude tiles.
 std::string compile_t2v2_c128(const TilePass &tp, T2Pass *out, bool gen);
 
-// Cut pass i of a plan in two at the middle of its steps, both on the same
-// tiles: for a complex128 pass with more steps, factors, records or runs than
-// a programme holds.  One more sweep of the state costs less than the generic
-// tile kernel, to which the pass would go (ten layers of U3 on ten of 20
-// qubits: 2860 -> 670 us; n = 16, 40 layers: 17.8 -> 3.9 ms).  False (nothing
-// changed) if it has a single step, or an in-tile SWAP, which only that kernel
-// runs.
-bool cut_pass(std::vector<TilePass> *passes, size_t i);
+// The same for pass i of a plan.  With `cut`, a pass with more steps, factors,
+// records or runs than a programme holds is cut in two at the middle of its
+// steps, both on the same tiles, until the first piece compiles (the rest is
+// inserted behind it).  One more sweep of the state costs less than the
+// generic tile kernel, to which the pass would go (ten layers of U3 on ten of
+// 20 qubits: 2860 -> 670 us; n = 16, 40 layers: 17.8 -> 3.9 ms).  A pass with
+// an in-tile SWAP, which only that kernel runs, stays whole.
+std::string compile_pass_c128(std::vector<TilePass> *passes, size_t i, bool cut, T2Pass *out);
 
 }  // namespace sv

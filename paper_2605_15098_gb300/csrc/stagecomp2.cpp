@@ -1165,7 +1165,9 @@ std::string compile_t2v2_c128(const TilePass &tp, T2Pass *out, bool gen) {
     return compile_fmt2<P64>(tp, out, gen);
 }
 
-bool cut_pass(std::vector<TilePass> *passes, size_t i) {
+// Cut pass i at the middle of its steps; false (nothing changed) if it has a
+// single step or an in-tile SWAP.
+static bool cut_pass(std::vector<TilePass> *passes, size_t i) {
     const TilePass &whole = (*passes)[i];
     const size_t steps = whole.ops.size(), half = steps / 2;
     if (steps < 2) return false;
@@ -1180,6 +1182,13 @@ bool cut_pass(std::vector<TilePass> *passes, size_t i) {
     head.ngates -= rest.ngates;
     passes->insert(passes->begin() + (long)i + 1, std::move(rest));
     return true;
+}
+
+std::string compile_pass_c128(std::vector<TilePass> *passes, size_t i, bool cut, T2Pass *out) {
+    for (;;) {
+        const std::string why = compile_t2v2_c128((*passes)[i], out, false);
+        if (why.empty() || !cut || !cut_pass(passes, i)) return why;
+    }
 }
 
 }  // namespace sv

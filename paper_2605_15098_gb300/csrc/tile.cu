@@ -521,25 +521,26 @@ static sv_status compiled_plan(sv_state *h, const std::vector<sv_gate> &gates, c
     if (ov && ov->kernel.size() != plan.passes.size())
         return fail(SV_ERR_STATE, "internal: learned plan does not match the planner's passes");
     bool first_pass = true;  // the pass that may start from a recorded basis state
+    // the kernel each pass is to run on; the pieces of a cut pass share one
+    std::vector<int8_t> kernel(plan.passes.size(),
+                               (int8_t)(!allow_t2 ? PK_GENERIC : fused && !dbl ? PK_T3 : PK_T2));
+    if (ov) kernel = ov->kernel;
     for (size_t i = 0; i < plan.passes.size(); i++) {
+        const int want = kernel[i];
         std::string why;  // complex128: why the pass does not compile
-        if (dbl && allow_t2 && !ov && !plan.passes[i].ops.empty()) {
-            why = compile_t2v2_c128(plan.passes[i], &t2[i], false);
-            while (!why.empty() && opt.split_u3 && cut_pass(&plan.passes, i)) {
-                t2.emplace(t2.begin() + (long)i + 1);
-                up.emplace(up.begin() + (long)i + 1);
-                why = compile_t2v2_c128(plan.passes[i], &t2[i], false);
-            }
+        if (dbl && allow_t2 && want != PK_GENERIC && !plan.passes[i].ops.empty()) {
+            why = compile_pass_c128(&plan.passes, i, opt.split_u3, &t2[i]);
+            kernel.insert(kernel.begin() + (long)i, plan.passes.size() - kernel.size(), (int8_t)want);
+            t2.resize(plan.passes.size());
+            up.resize(plan.passes.size());
         }
         const TilePass &p = plan.passes[i];
         if (!p.general.empty()) first_pass = false;  // the step writes the state first
         if (p.ops.empty()) continue;
         const bool first_ops = first_pass && p.remap_before.empty();
         first_pass = false;
-        const int want = ov ? ov->kernel[i] : (!allow_t2 ? PK_GENERIC : fused && !dbl ? PK_T3 : PK_T2);
         bool ok = false;
         if (dbl) {
-            if (ov && want != PK_GENERIC && allow_t2) why = compile_t2v2_c128(p, &t2[i], false);
             if (want != PK_GENERIC && allow_t2 && why.empty()) {
                 ok = true;
                 if (first_ops) {
