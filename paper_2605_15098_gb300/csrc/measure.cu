@@ -806,14 +806,15 @@ sv_status marginal(sv_state *h, const int *pos, int m, double *dev_out, bool nor
         return SV_OK;
     }
     uint64_t rows = fold ? blocks : UINT64_C(1) << gl;
-    SV_TRY(ensure_scratch(h, (rows + kFoldRows) * outcomes * sizeof(double)));
+    // many partials of few outcomes: one block would read them all (8
+    // outcomes, 2048 rows: 18 us), so more blocks add most of them
+    const bool fold_rows = rows > 4 * kFoldRows && outcomes * kFoldRows <= 8192;
+    SV_TRY(ensure_scratch(h, (rows + (fold_rows ? kFoldRows : 0)) * outcomes * sizeof(double)));
     double *partial = reinterpret_cast<double *>(h->scratch);
     launch_marginal<MARG_PART>(h, a, layout_r, pairs, blocks, partial, st, perm);
     SV_CUDA(cudaGetLastError());
     note_launch();
-    if (rows > 4 * kFoldRows && outcomes * kFoldRows <= 8192) {
-        // many partials of few outcomes: one block would read them all
-        // (8 outcomes, 2048 rows: 18 us), so more blocks add most of them
+    if (fold_rows) {
         double *folded = partial + rows * outcomes;
         const int to = (int)std::min<uint64_t>(outcomes, 32);
         k_fold_rows<<<dim3((unsigned)(outcomes / to), kFoldRows), kRedThreads, 0, h->stream>>>(
