@@ -156,7 +156,8 @@ __device__ __forceinline__ void better(double &v, uint64_t &i, double v2, uint64
 // best so far.
 __device__ __forceinline__ bool may_beat(double v, double best) {
     const long long b = __double_as_longlong(v);
-    return b >= __double_as_longlong(best) && b <= 0x7ff0000000000000ll;
+    // (unsigned: a NaN of either sign is above infinity)
+    return b >= __double_as_longlong(best) && (unsigned long long)b <= 0x7ff0000000000000ull;
 }
 
 // Output index of the entry at position i of a marginal ordered as p says.
