@@ -2,6 +2,7 @@
 // Host only (no CUDA call), for inspection and for host-side tests that
 // execute the exported programme and compare it with the oracle.
 #include <cinttypes>
+#include <cmath>
 #include <cstdio>
 #include <cstring>
 #include <string>
@@ -33,6 +34,73 @@ struct J {
         s += "]";
     }
 };
+
+// The device form (tileprog.h) of a format-2 programme, which the kernels
+// run: steps, matrix records, the terms of every slot, and the factor of a
+// generated state.
+void put_dev(J &j, const T2Pass &t) {
+    j.raw(",\"dev\":[");
+    for (size_t i = 0; i < t.dev.size(); i++) {
+        const T2Ins &in = t.dev[i];
+        if (i) j.raw(",");
+        j.raw("{\"hd\":"); j.num(in.hd);
+        j.raw(",\"op\":"); j.num(in.op);
+        j.raw(",\"idx\":"); j.num(in.idx);
+        j.raw(",\"ccls\":"); j.num(in.ccls);
+        j.raw(",\"cidx\":"); j.num(in.cidx);
+        j.raw(",\"e0\":"); j.num(in.e0);
+        j.raw(",\"e1\":"); j.num(in.e1);
+        j.raw(",\"aux\":"); j.num(in.aux);
+        if (in.hd == kT2HdSigns) {  // one word per register bit
+            int32_t w[8];
+            if (t.wide) std::memcpy(w, &t.dev_mats64[8 * (size_t)in.aux], sizeof w);
+            else std::memcpy(w, t.dev_mats[in.aux].m, sizeof w);
+            j.raw(",\"words\":");
+            j.arr(w, 5);
+        } else if (in.hd == kT2HdScale) {
+            const uint32_t low = (uint32_t)(uint16_t)in.e0 | ((uint32_t)(uint16_t)in.e1 << 16);
+            j.raw(",\"scale\":");
+            if (t.wide) {
+                const uint64_t bits = low | ((uint64_t)(uint32_t)in.aux << 32);
+                double v;
+                std::memcpy(&v, &bits, sizeof v);
+                j.dbl(v);
+            } else {
+                float hi, lo;
+                std::memcpy(&hi, &in.aux, sizeof hi);
+                std::memcpy(&lo, &low, sizeof lo);
+                j.dbl((double)hi + (double)lo);
+            }
+        }
+        j.raw("}");
+    }
+    j.raw("],\"dev_mats\":[");
+    const size_t nm = t.wide ? t.dev_mats64.size() / 8 : t.dev_mats.size();
+    for (size_t i = 0; i < nm; i++) {
+        if (i) j.raw(",");
+        j.raw("[");
+        for (int e = 0; e < 8; e++) {
+            const double v = t.wide ? t.dev_mats64[8 * i + e] : (double)t.dev_mats[i].m[e];
+            if (e) j.raw(",");
+            j.dbl(std::isfinite(v) ? v : 0.0);  // the words of a Signs step
+        }
+        j.raw("]");
+    }
+    j.raw("],\"slot_terms\":[");
+    for (size_t s = 0; s < t.slots.size(); s++) {
+        if (s) j.raw(",");
+        j.raw("[");
+        for (int32_t e = t.soff[s]; e < t.soff[s + 1]; e++) {
+            if (e > t.soff[s]) j.raw(",");
+            j.raw("["); j.num(t.wide ? t.sterms64[e].g0 : t.sterms[e].g0);
+            j.raw(","); j.num(t.wide ? t.sterms64[e].g1 : t.sterms[e].g1);
+            j.raw(","); j.u64(t.wide ? t.sterms64[e].theta : t.sterms[e].theta);
+            j.raw("]");
+        }
+        j.raw("]");
+    }
+    j.raw("],\"dev_gen_scale\":"); j.dbl(t.dev_gen_scale);
+}
 
 void put_t2(J &j, const T2Pass &t) {
     j.raw("{\"ins\":[");
@@ -129,6 +197,7 @@ void put_t2(J &j, const T2Pass &t) {
     }
     j.raw("],\"nruns\":"); j.num(t.nruns);
     j.raw(",\"n_h\":"); j.num(t.n_h);
+    if (t.format == 2) put_dev(j, t);
     j.raw("}");
 }
 
@@ -173,8 +242,7 @@ extern "C" sv_status sv_plan_export(int n, sv_dtype dt, const int *host_phys_of_
         T2Pass t2;
         std::string why = "disabled";
         if (dbl && !(c.flags & SV_FLAG_GENERIC_TILE) && opt.k == kT2Qubits && !plan.passes[pi].ops.empty()) {
-            // complex128 on 2^13-amplitude tiles: the FP64 register-stage
-            // kernel (its programme is the emulator's business only through the ops)
+            // complex128 on 2^13-amplitude tiles: the FP64 register-stage kernel
             why = compile_pass_c128(&plan.passes, pi, opt.split_u3, &t2);
         }
         const TilePass &p = plan.passes[pi];
