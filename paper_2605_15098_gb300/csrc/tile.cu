@@ -763,6 +763,7 @@ sv_status partitioned_apply(sv_state *h, const std::vector<sv_gate> &gates, cons
             slots_together += (most + 255) & ~(size_t)255;
             need = std::max(need, most);
         }
+        const size_t one_pass = need;
         if (slots_together <= kSlotvTogether) need = slots_together;
         else slots_together = 0;
         if (need > h->slotv_cap) {
@@ -772,11 +773,19 @@ sv_status partitioned_apply(sv_state *h, const std::vector<sv_gate> &gates, cons
             }
             h->slotv = nullptr;
             h->slotv_cap = 0;
-            if (dev_malloc(&h->slotv, need) != cudaSuccess) {
+            auto allocate = [&]() {
+                if (dev_malloc(&h->slotv, need) == cudaSuccess) return true;
                 cudaGetLastError();
                 h->slotv = nullptr;
-                return fail(SV_ERR_OOM, "cannot allocate the per-tile slot values (%zu bytes)", need);
+                return false;
+            };
+            bool ok = allocate();
+            if (!ok && one_pass < need) {  // no room for all passes: one at a time
+                need = one_pass;
+                slots_together = 0;
+                ok = allocate();
             }
+            if (!ok) return fail(SV_ERR_OOM, "cannot allocate the per-tile slot values (%zu bytes)", need);
             h->slotv_cap = need;
         }
     }

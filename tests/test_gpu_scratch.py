@@ -34,3 +34,34 @@ def test_marginal_scratch(sv, m):
             # 2 MiB of sums, in 2 MiB pages
             assert free - torch.cuda.mem_get_info()[0] <= 4 << 20
         assert abs(float(out.sum()) - 1.0) < 1e-12
+
+
+def test_slot_values_one_pass_at_a_time(sv, orc):
+    """Without room for the slot values of all passes the call computes them
+    pass by pass: one refused allocation is survived, and the amplitudes are
+    those of an undisturbed call."""
+    import numpy as np
+
+    from paper_2605_15098_gb300 import circuits as C
+
+    n = 19
+    g = C.random_circuit(n, 8, 4)
+    cfg = sv.make_config(sv.SV_MODE_PARTITIONED)
+    with sv.State(n, sv.SV_C64) as s:
+        s.apply(g, cfg)
+        want = s.amplitudes()
+    survived = 0
+    for after in range(5):  # three allocations of the apply, two of a new handle
+        with sv.State(n, sv.SV_C64) as s:
+            sv.sv_fault_inject(sv.SV_FAULT_ALLOC, after)
+            try:
+                s.apply(g, cfg)
+                sv.sv_destroy(sv.sv_create(3, sv.SV_C64))  # refused if the fault is still to come
+            except sv.SvError as e:
+                assert e.code == sv.SV_ERR_OOM
+                continue
+            finally:
+                sv.sv_fault_inject(sv.SV_FAULT_ALLOC, -1)
+            survived += 1
+            assert np.array_equal(s.amplitudes(), want)
+    assert survived == 1
