@@ -32,11 +32,11 @@ struct MargArgs {
     int n;
     int m;                    // outcome bits
     uint64_t mask;            // physical bits of the outcome
-    uint64_t rest;            // physical bits summed over (within n)
+    uint64_t rest;            // physical bits summed over (within n; RB: without bit 0)
     uint64_t upper;           // layout R: rest bits above the 5 lane bits
     int spos[34];             // outcome physical bits, ascending
     int out_bit[34];          // logical output bit of spos[k]
-    uint64_t per_group;       // enumerated rest values per group
+    uint64_t per_group;       // enumerated rest values (RB: pairs of them) per group
     int groups_log2;
     int in_order;             // the output order is the physical one
     uint64_t flush;           // values a thread sums before it adds them to its FP64 sum
@@ -104,12 +104,41 @@ struct ProbAcc<float> {
     __device__ double value() const { return (double)hi + (double)lo; }
 };
 
-__device__ __forceinline__ void add_vec(ProbAcc<float> &a, ProbAcc<float> &b, float4 v) {
+// complex64 sums without rounding errors down to FP64's: the remainders' sum
+// keeps its own remainders.  Twice the pair's instructions, for a thread that
+// sums a whole outcome, where the pair's error (rms 1.8e-15 after 32 amplitudes,
+// against 2e-16) would show and FP64 additions in between cost more.
+struct ExactAcc {
+    float s0 = 0.f, s1 = 0.f, s2 = 0.f;
+    __device__ static float two_sum(float &s, float b) {
+        const float t = s + b, bb = t - s;
+        const float e = (s - (t - bb)) + (b - bb);
+        s = t;
+        return e;
+    }
+    __device__ void square(float x) {
+        const float p = __fmul_rn(x, x);  // not contracted into the sum
+        const float e = two_sum(s1, two_sum(s0, p));
+        s2 += e + two_sum(s1, fmaf(x, x, -p));
+    }
+    __device__ void add(float2 v) {
+        square(v.x);
+        square(v.y);
+    }
+    __device__ double value() const { return (double)s0 + ((double)s1 + (double)s2); }
+};
+
+// A load's amplitudes: two outcomes (PB = 1), or one or two of one outcome.
+template <int PB, typename A>
+__device__ __forceinline__ void add_vec(A &a, A &b, float4 v) {
     a.add(make_float2(v.x, v.y));
-    b.add(make_float2(v.z, v.w));
+    if (PB) b.add(make_float2(v.z, v.w));
+    else a.add(make_float2(v.z, v.w));
 }
-__device__ __forceinline__ void add_vec(ProbAcc<float> &a, ProbAcc<float> &, float2 v) { a.add(v); }
-__device__ __forceinline__ void add_vec(ProbAcc<double> &a, ProbAcc<double> &, double2 v) { a.add(v); }
+template <int PB, typename A>
+__device__ __forceinline__ void add_vec(A &a, A &, float2 v) { a.add(v); }
+template <int PB, typename A>
+__device__ __forceinline__ void add_vec(A &a, A &, double2 v) { a.add(v); }
 
 // What a read-out leaves besides the marginal itself.
 struct ReadResult {
@@ -244,16 +273,26 @@ enum { MARG_PART = 0, MARG_SUM = 1, MARG_ARG = 2 };
 
 // Layout M: consecutive threads take consecutive physical-order outcomes.
 // PB = 1 (complex64 with physical bit 0 an outcome bit): the two outcomes that
-// differ in it, whose amplitudes one 16-byte load covers.  With fewer outcomes than
+// differ in it, whose amplitudes one 16-byte load covers.  RB (complex64 with
+// bit 0 summed over): such a load covers two amplitudes of one outcome.  RB = 2:
+// where a warp per outcome used to sum, with no larger error: exactly
+// (ExactAcc), or in complex128 in shorter chains.
+// With fewer outcomes than
 // a block has threads, the block's slices of one outcome are added here, so
 // that a marginal of a few qubits leaves a thousand partials per outcome
 // instead of up to 2^18.  HBM bounds it: 512 MiB in 86 us (0.93 of the
 // measured rate); QPE n = 28's argmax, 2 GiB, 376 us against 470 us for the
 // marginal, its block sums and its argmax as kernels of their own.
-template <typename R, int PB, int MODE>
+template <typename R, int PB, int RB, int MODE>
 __global__ void __launch_bounds__(kRedThreads, kRedBlocks)
 k_marg_m(const R *__restrict__ s, MargArgs a, double *__restrict__ partial, const Stats st, const OutPerm perm) {
-    using V = typename std::conditional<PB == 1, float4, typename ProbAcc<R>::V>::type;
+    constexpr bool kWide = sizeof(R) == 8;
+    using V = typename std::conditional<!kWide && (PB || RB), float4, typename ProbAcc<R>::V>::type;
+    using Acc = typename std::conditional<!kWide && RB == 2, ExactAcc, ProbAcc<R>>::type;
+    constexpr int kShift = !kWide && (PB || RB) ? 1 : 0;
+    // complex128 sums that a warp's lanes used to share: even and odd loads
+    // apart, so that no addition has more before it than there
+    constexpr int kAlt = kWide && RB == 2 ? 1 : 0;
     __shared__ double sh[MODE == MARG_PART ? 2 * kRedThreads : 1];
     const uint64_t outcomes = UINT64_C(1) << a.m;
     const uint64_t per = outcomes >> PB;  // threads per slice
@@ -279,21 +318,19 @@ k_marg_m(const R *__restrict__ s, MargArgs a, double *__restrict__ partial, cons
         }
         const uint64_t ml1 = PB ? ml | (UINT64_C(1) << a.out_bit[0]) : ml;
         uint64_t xr = pdep_mask(g * a.per_group, a.rest);
-        ProbAcc<R> acc0, acc1;
+        Acc acc0, acc1;
         double p0 = 0.0, p1 = 0.0;
         auto flush = [&](uint64_t done) {
             if (done & (a.flush - 1)) return;
             if (a.flush == a.per_group) {  // one sum: nothing to add it to
-                p0 = acc0.value();
+                p0 = kAlt ? acc0.value() + acc1.value() : acc0.value();
                 if (PB) p1 = acc1.value();
                 return;
             }
-            p0 += acc0.value();
-            acc0 = ProbAcc<R>();
-            if (PB) {
-                p1 += acc1.value();
-                acc1 = ProbAcc<R>();
-            }
+            p0 += kAlt ? acc0.value() + acc1.value() : acc0.value();
+            acc0 = Acc();
+            if (PB) p1 += acc1.value();
+            if (PB || kAlt) acc1 = Acc();
         };
         uint64_t i = in ? 0 : a.per_group;
         // kLoadBatch loads in flight per thread, then accumulated in order
@@ -301,24 +338,24 @@ k_marg_m(const R *__restrict__ s, MargArgs a, double *__restrict__ partial, cons
             V v[kLoadBatch];
 #pragma unroll
             for (int k = 0; k < kLoadBatch; k++) {
-                v[k] = sv_[(xm | xr) >> PB];
+                v[k] = sv_[(xm | xr) >> kShift];
                 xr = ((xr | ~a.rest) + 1) & a.rest;
             }
             if (a.flush >= kLoadBatch) {
 #pragma unroll
-                for (int k = 0; k < kLoadBatch; k++) add_vec(acc0, acc1, v[k]);
+                for (int k = 0; k < kLoadBatch; k++) add_vec<PB>(kAlt && (k & 1) ? acc1 : acc0, acc1, v[k]);
                 flush(i + kLoadBatch);
             } else {
 #pragma unroll
                 for (int k = 0; k < kLoadBatch; k++) {
-                    add_vec(acc0, acc1, v[k]);
+                    add_vec<PB>(acc0, acc1, v[k]);
                     flush(k + 1);
                 }
             }
         }
         for (; i < a.per_group; i++) {
-            const V v = sv_[(xm | xr) >> PB];
-            add_vec(acc0, acc1, v);
+            const V v = sv_[(xm | xr) >> kShift];
+            add_vec<PB>(acc0, acc1, v);
             flush(i + 1);
             xr = ((xr | ~a.rest) + 1) & a.rest;
         }
@@ -359,20 +396,26 @@ k_marg_m(const R *__restrict__ s, MargArgs a, double *__restrict__ partial, cons
     if constexpr (MODE != MARG_PART) finish_stats<MODE == MARG_ARG>(tot, best, bidx, st);
 }
 
-// Layout R: the lowest physical bits are summed over; one warp per
-// (group, outcome), lanes take the five lowest rest bits.
-template <typename R, int MODE>
+// Layout R: physical bit 0 is summed over; 2^J lanes per (group, outcome) take
+// the J lowest rest bits (RB: above bit 0, which is inside a load).  J = 5 for
+// few outcomes: with many, the five FP64 additions over the lanes and the
+// start of each sum are most of the work (see marginal).
+template <typename R, int J, int RB, int MODE>
 __global__ void __launch_bounds__(kRedThreads, kRedBlocks)
 k_marg_r(const R *__restrict__ s, MargArgs a, double *__restrict__ partial, const Stats st, const OutPerm perm) {
+    using V = typename std::conditional<RB == 1, float4, typename ProbAcc<R>::V>::type;
+    const V *sv_ = reinterpret_cast<const V *>(s);
     const uint64_t outcomes = UINT64_C(1) << a.m;
-    const int lane = threadIdx.x & 31;
+    const int sub = threadIdx.x & ((1 << J) - 1);
+    const uint64_t xl = pdep_mask((uint64_t)sub, a.rest & ~a.upper);
     const uint64_t items = outcomes << a.groups_log2;
     double tot = 0.0, best = -1.0;
     uint64_t bidx = ~UINT64_C(0);
-    for (uint64_t warp = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; warp < items;
-         warp += ((uint64_t)gridDim.x * blockDim.x) >> 5) {
-        const uint64_t mp = warp & (outcomes - 1);
-        const uint64_t g = warp >> a.m;
+    // (items: a multiple of the warp's, so that its lanes leave together)
+    for (uint64_t item = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> J; item < items;
+         item += ((uint64_t)gridDim.x * blockDim.x) >> J) {
+        const uint64_t mp = item & (outcomes - 1);
+        const uint64_t g = item >> a.m;
         uint64_t xm = 0, ml = 0;
         for (int k = 0; k < a.m; k++) {
             if ((mp >> k) & 1) {
@@ -380,8 +423,6 @@ k_marg_r(const R *__restrict__ s, MargArgs a, double *__restrict__ partial, cons
                 ml |= UINT64_C(1) << a.out_bit[k];
             }
         }
-        const uint64_t lane_bits = a.rest & ~a.upper;
-        const uint64_t xl = pdep_mask((uint64_t)lane, lane_bits);
         uint64_t xo = pdep_mask(g * a.per_group, a.upper);
         ProbAcc<R> pa;
         double acc = 0.0;
@@ -392,32 +433,32 @@ k_marg_r(const R *__restrict__ s, MargArgs a, double *__restrict__ partial, cons
         };
         uint64_t i = 0;
         for (; i + kLoadBatch <= a.per_group; i += kLoadBatch) {
-            typename ProbAcc<R>::V v[kLoadBatch];
+            V v[kLoadBatch];
 #pragma unroll
             for (int k = 0; k < kLoadBatch; k++) {
-                v[k] = ProbAcc<R>::load(s, xm | xo | xl);
+                v[k] = sv_[(xm | xo | xl) >> RB];
                 xo = ((xo | ~a.upper) + 1) & a.upper;
             }
             if (a.flush >= kLoadBatch) {
 #pragma unroll
-                for (int k = 0; k < kLoadBatch; k++) pa.add(v[k]);
+                for (int k = 0; k < kLoadBatch; k++) add_vec<0>(pa, pa, v[k]);
                 flush(i + kLoadBatch);
             } else {
 #pragma unroll
                 for (int k = 0; k < kLoadBatch; k++) {
-                    pa.add(v[k]);
+                    add_vec<0>(pa, pa, v[k]);
                     flush(k + 1);
                 }
             }
         }
         for (; i < a.per_group; i++) {
-            pa.add(s, xm | xo | xl);
+            add_vec<0>(pa, pa, sv_[(xm | xo | xl) >> RB]);
             flush(i + 1);
             xo = ((xo | ~a.upper) + 1) & a.upper;
         }
 #pragma unroll
-        for (int off = 16; off; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-        if (lane == 0) {
+        for (int off = 1 << (J - 1); off; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
+        if (sub == 0) {
             if (MODE != MARG_ARG) partial[g * outcomes + ml] = acc;
             if (MODE != MARG_PART) tot += acc;
             if (MODE == MARG_ARG && may_beat(acc, best)) better(best, bidx, acc, output_index(mp, perm));
@@ -714,22 +755,30 @@ sv_status ensure_probs(sv_state *h, size_t bytes) {
 namespace {
 
 template <int MODE>
-void launch_marginal(sv_state *h, const MargArgs &a, bool layout_r, bool pairs, unsigned grid, double *partial, const Stats &st,
-                     const OutPerm &perm) {
+void launch_marginal(sv_state *h, const MargArgs &a, int lanes_log2, bool pairs, bool rest_pairs, bool exact, unsigned grid,
+                     double *partial, const Stats &st, const OutPerm &perm) {
     if (h->dt == SV_C128) {
         const double *s = reinterpret_cast<const double *>(h->amps);
-        if (layout_r)
-            k_marg_r<double, MODE><<<grid, kRedThreads, 0, h->stream>>>(s, a, partial, st, perm);
+        if (lanes_log2)
+            k_marg_r<double, 5, 0, MODE><<<grid, kRedThreads, 0, h->stream>>>(s, a, partial, st, perm);
+        else if (exact)
+            k_marg_m<double, 0, 2, MODE><<<grid, kRedThreads, 0, h->stream>>>(s, a, partial, st, perm);
         else
-            k_marg_m<double, 0, MODE><<<grid, kRedThreads, 0, h->stream>>>(s, a, partial, st, perm);
+            k_marg_m<double, 0, 0, MODE><<<grid, kRedThreads, 0, h->stream>>>(s, a, partial, st, perm);
     } else {
         const float *s = reinterpret_cast<const float *>(h->amps);
-        if (layout_r)
-            k_marg_r<float, MODE><<<grid, kRedThreads, 0, h->stream>>>(s, a, partial, st, perm);
+        if (lanes_log2 == 5)
+            k_marg_r<float, 5, 0, MODE><<<grid, kRedThreads, 0, h->stream>>>(s, a, partial, st, perm);
+        else if (lanes_log2)
+            k_marg_r<float, 1, 1, MODE><<<grid, kRedThreads, 0, h->stream>>>(s, a, partial, st, perm);
         else if (pairs)
-            k_marg_m<float, 1, MODE><<<grid, kRedThreads, 0, h->stream>>>(s, a, partial, st, perm);
+            k_marg_m<float, 1, 0, MODE><<<grid, kRedThreads, 0, h->stream>>>(s, a, partial, st, perm);
+        else if (exact)
+            k_marg_m<float, 0, 2, MODE><<<grid, kRedThreads, 0, h->stream>>>(s, a, partial, st, perm);
+        else if (rest_pairs)
+            k_marg_m<float, 0, 1, MODE><<<grid, kRedThreads, 0, h->stream>>>(s, a, partial, st, perm);
         else
-            k_marg_m<float, 0, MODE><<<grid, kRedThreads, 0, h->stream>>>(s, a, partial, st, perm);
+            k_marg_m<float, 0, 0, MODE><<<grid, kRedThreads, 0, h->stream>>>(s, a, partial, st, perm);
     }
 }
 
@@ -766,42 +815,68 @@ sv_status marginal(sv_state *h, const int *pos, int m, double *dev_out, bool nor
     const int rbits = n - m;
     const uint64_t outcomes = UINT64_C(1) << m;
     const bool bit0 = (a.mask & 1) != 0;
-    const bool layout_r = !bit0 && rbits >= 5;
+    // Where physical bit 0 is summed over, a warp per outcome below 2^15 of them
+    // (layout R).  Above, the five FP64 additions over its lanes and the start
+    // of each sum are most of the work: one thread per outcome (layout M), in
+    // complex64 with exact sums (ExactAcc), or, where a lane of that warp would
+    // hold 16 amplitudes or more, FP32 pairs of as many, and two lanes with 32
+    // contiguous bytes if bit 1 is summed over too.  n = 26, complex64, the 2^m
+    // outcomes of the highest qubits, a warp against this: m = 14 104 against
+    // 107 us, m = 15 121 and 110, m = 17 197 and 105, m = 18 281 and 144, m = 20
+    // 985 and 140; n = 22: m = 14 27 and 33, m = 15 60 and 25, m = 17 110 and 23.
+    // complex128, where the sums themselves fill the FP64 pipe, keeps the warp
+    // for 2^10 amplitudes or more per outcome, unless bit 1 is an outcome bit and
+    // half of each 64 bytes that it reads another outcome's (n = 26: m = 15 292
+    // and 320, m = 16 with bit 1 558 and 320, m = 17 339 and 322).
+    const bool many_rest = !bit0 && rbits >= 5 && m >= 15 && (h->dt == SV_C64 || rbits < 10 || (a.mask & 2));
+    const bool exact = many_rest && (h->dt == SV_C128 || rbits < 9);
+    const int lanes_log2 = bit0 || rbits < 5 ? 0 : !many_rest ? 5 : exact || (a.mask & 2) ? 0 : 1;
+    const bool layout_r = lanes_log2 > 0;
+    // complex64 with bit 0 summed over: two amplitudes per load where two share
+    // an FP32 sum (a.flush below)
+    const bool rest_pairs = lanes_log2 < 5 && !bit0 && h->dt == SV_C64 && n >= 20;
+    if (rest_pairs) a.rest &= ~UINT64_C(1);
+    const int bits = rbits - rest_pairs;
     // complex64 with physical bit 0 an outcome bit: two outcomes per thread
     const bool pairs = bit0 && h->dt == SV_C64;
     // slices per outcome: enough threads (layout M) or lanes (layout R) for the
-    // device, but at least 16 (8) vectors per thread, so that a marginal with
+    // device, but at least 16 (8) loads per thread, so that a marginal with
     // many outcomes, or a small state's, is one launch
     const int target_log2 = 18;
     int gl;
     if (layout_r) {
         uint64_t up = a.rest;
-        for (int i = 0; i < 5; i++) up &= up - 1;  // drop the 5 lowest rest bits
+        for (int i = 0; i < lanes_log2; i++) up &= up - 1;  // drop the lanes' rest bits
         a.upper = up;
-        int ubits = rbits - 5;
-        gl = std::max(0, std::min(ubits - 3, target_log2 - 5 - m));
+        int ubits = bits - lanes_log2;
+        gl = std::max(0, std::min(ubits - 3, target_log2 - lanes_log2 - m));
         a.per_group = UINT64_C(1) << (ubits - gl);
     } else {
-        gl = std::max(0, std::min(rbits - 4, target_log2 - m));
-        a.per_group = UINT64_C(1) << (rbits - gl);
+        gl = std::max(0, std::min(bits - 4, target_log2 - rest_pairs - m));
+        a.per_group = UINT64_C(1) << (bits - gl);
     }
     a.groups_log2 = gl;
     // FP32 pairs carry about 2^-48 of their sum's size per addition: short
     // sums, added up in FP64, keep the marginal's error below 1e-15 on small
     // and mid-sized states, where the conversions cost nothing (2^19 of them
     // or one per amplitude, whichever is less)
-    const int short_log2 = layout_r ? std::max(0, rbits - 5 - std::max(0, 14 - m)) : std::max(0, rbits - std::max(0, 19 - m));
-    a.flush = std::min(a.per_group, UINT64_C(1) << short_log2);
+    int short_log2 = std::max(0, rbits - lanes_log2 - std::max(0, 19 - lanes_log2 - m));
+    if (many_rest) short_log2 = !exact ? rbits - 5 : rest_pairs ? rbits : 4;
+    a.flush = std::min(a.per_group, UINT64_C(1) << (short_log2 - rest_pairs));
     const int pb = pairs ? 1 : 0;
     const Stats st = stats_of(h);
     const unsigned most = (unsigned)std::min(kMaxStatBlocks, h->sm_count * kRedBlocks);
-    const uint64_t threads = layout_r ? (outcomes << gl) * 32 : (outcomes >> pb) << gl;
+    const uint64_t threads = layout_r ? (outcomes << gl) << lanes_log2 : (outcomes >> pb) << gl;
     const unsigned blocks = blocks_for(threads, kRedThreads);
     const bool fold = !layout_r && (outcomes >> pb) < kRedThreads;  // the block adds its slices
     *divided = false;
     if (gl == 0) {  // every thread (warp) holds whole outcomes
-        const unsigned grid = std::min(blocks, most);
-        launch_marginal<MODE>(h, a, layout_r, pairs, grid, dev_out, st, perm);
+        // layout R's items are few and large: a block for each of them where
+        // that is at most two waves of blocks (n = 26, m = 13: 105 against 116
+        // us), with two lanes per outcome at all sizes
+        const unsigned cap = lanes_log2 == 5 ? 2 * most : lanes_log2 ? (unsigned)kMaxStatBlocks : most;
+        const unsigned grid = blocks <= cap ? blocks : most;
+        launch_marginal<MODE>(h, a, lanes_log2, pairs, rest_pairs, exact, grid, dev_out, st, perm);
         SV_CUDA(cudaGetLastError());
         note_launch();
         return SV_OK;
@@ -812,7 +887,7 @@ sv_status marginal(sv_state *h, const int *pos, int m, double *dev_out, bool nor
     const bool fold_rows = rows > 4 * kFoldRows && outcomes * kFoldRows <= 8192;
     SV_TRY(ensure_scratch(h, (rows + (fold_rows ? kFoldRows : 0)) * outcomes * sizeof(double)));
     double *partial = reinterpret_cast<double *>(h->scratch);
-    launch_marginal<MARG_PART>(h, a, layout_r, pairs, blocks, partial, st, perm);
+    launch_marginal<MARG_PART>(h, a, lanes_log2, pairs, rest_pairs, exact, blocks, partial, st, perm);
     SV_CUDA(cudaGetLastError());
     note_launch();
     if (fold_rows) {
