@@ -571,14 +571,31 @@ k_normalise(double *__restrict__ p, uint64_t len, const ReadResult *__restrict__
 // above the sum's binade, a step out of the binade, a sum that is not a
 // normal number.  Zeros change nothing and are never exceptions.
 //
+// An exception costs a prefix sum, about eight additions' time.  Sums of
+// similar values have about two per doubling of the sum; but all 32 values of
+// a step can be exceptions, so after kRunRounds of them the rest is added one
+// after the other.  sv_sample of 2^20 outcomes, the call: Gaussian amplitudes
+// 120 us without this, 117 with it; every value a tie 503 and 224; values
+// that grow by 2^2000 in all 530 and 240.  (kRunRounds 1, 2, 4, 6: Gaussian 129, 126,
+// 119, 125; ties 214, 211, 232, 254.)
+//
 // total: the sum so far, the same in every lane, on return the sum with all
 // 32 values; returns the sum up to and including the lane's own value.
+constexpr int kRunRounds = 3;
 __device__ __forceinline__ double warp_run(double &total, double x, int lane) {
     uint64_t c = (uint64_t)__double_as_longlong(total), mine = c;
     const uint64_t xb = (uint64_t)__double_as_longlong(x);
     const int ex = (int)(xb >> 52);
     const uint64_t m = (xb & ((UINT64_C(1) << 52) - 1)) | (ex ? UINT64_C(1) << 52 : 0);
-    for (int pos = 0; pos < 32;) {
+    for (int pos = 0, rounds = 0; pos < 32; rounds++) {
+        if (rounds == kRunRounds) {
+            for (; pos < 32; pos++) {
+                const double xf = __shfl_sync(0xffffffffu, x, pos);
+                c = (uint64_t)__double_as_longlong(__dadd_rn(__longlong_as_double((long long)c), xf));
+                if (lane == pos) mine = c;
+            }
+            break;
+        }
         const int e = (int)(c >> 52);
         const int de = e - (ex ? ex : 1);
         bool bad = false;
