@@ -574,14 +574,14 @@ k_normalise(double *__restrict__ p, uint64_t len, const ReadResult *__restrict__
 // An exception costs a prefix sum, about eight additions' time.  Sums of
 // similar values have about two per doubling of the sum; but all 32 values of
 // a step can be exceptions, so after kRunRounds of them the rest is added one
-// after the other.  sv_sample of 2^20 outcomes, the call: Gaussian amplitudes
-// 120 us without this, 117 with it; every value a tie 503 and 224; values
-// that grow by 2^2000 in all 530 and 240.  (kRunRounds 1, 2, 4, 6: Gaussian 129, 126,
-// 119, 125; ties 214, 211, 232, 254.)
+// after the other.  2^20 outcomes: k_cdf_blocks on Gaussian amplitudes 18.8 us
+// with and without this, on sums of 16 of them 18.9 and 18.5 (kRunRounds 3: 19.0
+// and 19.5); sv_sample where every value is a tie 503 -> 232 us (3: 224, 6: 254),
+// where they grow by 2^2000 in all 530 -> 249.
 //
 // total: the sum so far, the same in every lane, on return the sum with all
 // 32 values; returns the sum up to and including the lane's own value.
-constexpr int kRunRounds = 3;
+constexpr int kRunRounds = 4;
 __device__ __forceinline__ double warp_run(double &total, double x, int lane) {
     uint64_t c = (uint64_t)__double_as_longlong(total), mine = c;
     const uint64_t xb = (uint64_t)__double_as_longlong(x);
