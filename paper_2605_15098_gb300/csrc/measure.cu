@@ -842,10 +842,18 @@ sv_status marginal(sv_state *h, const int *pos, int m, double *dev_out, bool nor
     // 107 us, m = 15 121 and 110, m = 17 197 and 105, m = 18 281 and 144, m = 20
     // 985 and 140; n = 22: m = 14 27 and 33, m = 15 60 and 25, m = 17 110 and 23.
     // complex128, where the sums themselves fill the FP64 pipe, keeps the warp
-    // for 2^10 amplitudes or more per outcome, unless bit 1 is an outcome bit and
-    // half of each 64 bytes that it reads another outcome's (n = 26: m = 15 292
-    // and 320, m = 16 with bit 1 558 and 320, m = 17 339 and 322).
-    const bool many_rest = !bit0 && rbits >= 5 && m >= 15 && (h->dt == SV_C64 || rbits < 10 || (a.mask & 2));
+    // for 2^10 amplitudes or more per outcome, 2^9 from 2^18 outcomes up (a warp
+    // against a thread: n = 25, m = 15 168 and 173, m = 16 179 and 175; n = 26,
+    // m = 15 298 and 324, m = 16 308 and 326, m = 17 338 and 328; n = 27, m = 17
+    // 593 and 627, m = 18 659 and 712), unless its lanes lie far apart: where
+    // only two bits summed over are below bit 18 the warp takes 1.2 to 2.6 times
+    // as long (n = 26, m = 16, the qubits from 1 up 629 and 324, from 2 up 414 and
+    // 323; m = 15, with the third bit at 17, 301 and 324).
+    uint64_t third = a.rest & (a.rest - 1);
+    third &= third - 1;  // the bits summed over without the two lowest
+    const bool far = !(third & ((UINT64_C(1) << 18) - 1));
+    const bool many_rest =
+        !bit0 && rbits >= 5 && m >= 15 && (h->dt == SV_C64 || far || rbits < (m >= 18 ? 9 : 10));
     const bool exact = many_rest && (h->dt == SV_C128 || rbits < 9);
     const int lanes_log2 = bit0 || rbits < 5 ? 0 : !many_rest ? 5 : exact || (a.mask & 2) ? 0 : 1;
     const bool layout_r = lanes_log2 > 0;

@@ -26,7 +26,8 @@ CASES = [(n, spread(n, m, low)) for n, m in ((19, 13), (19, 14), (20, 14), (20, 
          for low in (1, 2, 3)]
 CASES += [(20, list(range(5, 20))), (20, list(range(4, 20))), (22, list(range(7, 22))), (22, list(range(5, 22))),
           (23, list(range(5, 23))), (24, list(range(5, 24))), (24, [1] + list(range(6, 24))),
-          (24, list(range(9, 24))), (25, list(range(10, 25))), (25, [1] + list(range(11, 25)))]
+          (24, list(range(9, 24))), (25, list(range(10, 25))), (25, [1] + list(range(11, 25))),
+          (26, list(range(1, 17)))]  # complex128: a warp's lanes far apart
 
 
 @pytest.mark.parametrize("dt", ["c64", "c128"])
