@@ -799,11 +799,27 @@ void launch_marginal(sv_state *h, const MargArgs &a, int lanes_log2, bool pairs,
     }
 }
 
+// Whether the handle has this much scratch, or can get it now: not while the
+// stream is being captured, where an allocation would end the capture.
+bool scratch_at_hand(sv_state *h, size_t bytes) {
+    if (bytes <= h->scratch_cap) return true;
+    cudaStreamCaptureStatus cs;
+    if (cudaStreamIsCapturing(h->stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
+        return false;
+    }
+    if (ensure_scratch(h, bytes) == SV_OK) return true;
+    clear_error();
+    return false;
+}
+
 // pos[j]: physical bit of output bit j.  MODE MARG_SUM: the marginal and its
 // total, in dev_out; MARG_ARG: its total and largest entry only (dev_out may
 // be NULL).  *divided: the marginal was divided by its total already.
+// no_scratch: a marginal of 2^15 outcomes or more without partial sums.
 template <int MODE>
-sv_status marginal(sv_state *h, const int *pos, int m, double *dev_out, bool norm, bool *divided) {
+sv_status marginal(sv_state *h, const int *pos, int m, double *dev_out, bool norm, bool *divided,
+                   bool no_scratch = false) {
     SV_TRY(materialize(h));
     const int n = h->n;
     MargArgs a{};
@@ -853,7 +869,7 @@ sv_status marginal(sv_state *h, const int *pos, int m, double *dev_out, bool nor
     third &= third - 1;  // the bits summed over without the two lowest
     const bool far = !(third & ((UINT64_C(1) << 18) - 1));
     const bool many_rest =
-        !bit0 && rbits >= 5 && m >= 15 && (h->dt == SV_C64 || far || rbits < (m >= 18 ? 9 : 10));
+        !no_scratch && !bit0 && rbits >= 5 && m >= 15 && (h->dt == SV_C64 || far || rbits < (m >= 18 ? 9 : 10));
     const bool exact = many_rest && (h->dt == SV_C128 || rbits < 9);
     const int lanes_log2 = bit0 || rbits < 5 ? 0 : !many_rest ? 5 : exact || (a.mask & 2) ? 0 : 1;
     const bool layout_r = lanes_log2 > 0;
@@ -910,7 +926,10 @@ sv_status marginal(sv_state *h, const int *pos, int m, double *dev_out, bool nor
     // many partials of few outcomes: one block would read them all (8
     // outcomes, 2048 rows: 18 us), so more blocks add most of them
     const bool fold_rows = rows > 4 * kFoldRows && outcomes * kFoldRows <= 8192;
-    SV_TRY(ensure_scratch(h, (rows + (fold_rows ? kFoldRows : 0)) * outcomes * sizeof(double)));
+    const size_t bytes = (rows + (fold_rows ? kFoldRows : 0)) * outcomes * sizeof(double);
+    // (up to 2 MiB for 2^15 to 2^17 outcomes; the warp per outcome needs none)
+    if (many_rest && !scratch_at_hand(h, bytes)) return marginal<MODE>(h, pos, m, dev_out, norm, divided, true);
+    SV_TRY(ensure_scratch(h, bytes));
     double *partial = reinterpret_cast<double *>(h->scratch);
     launch_marginal<MARG_PART>(h, a, lanes_log2, pairs, rest_pairs, exact, blocks, partial, st, perm);
     SV_CUDA(cudaGetLastError());

@@ -65,3 +65,48 @@ def test_slot_values_one_pass_at_a_time(sv, orc):
             survived += 1
             assert np.array_equal(s.amplitudes(), want)
     assert survived == 1
+
+
+@pytest.mark.parametrize("dt,n,m", [("c64", 20, 15), ("c64", 24, 15), ("c64", 24, 16), ("c128", 21, 16)])
+def test_many_outcomes_without_scratch(sv, orc, dt, n, m):
+    """A marginal of 2^15 outcomes or more without physical bit 0 needs no device
+    memory but its result: it survives a refused allocation, and it can be
+    captured into a graph on a handle that has not run one before."""
+    import numpy as np
+    import torch
+
+    rng = np.random.default_rng(n + m)
+    psi = rng.normal(size=1 << n) + 1j * rng.normal(size=1 << n)
+    psi = (psi / np.linalg.norm(psi)).astype(np.complex64 if dt == "c64" else np.complex128)
+    mask = ((1 << m) - 1) << (n - m)
+    ref = orc.marginal(n, psi.astype(np.complex128), mask)
+    code = sv.SV_C64 if dt == "c64" else sv.SV_C128
+    out = torch.empty(1 << m, dtype=torch.float64, device="cuda")
+
+    def check():
+        torch.cuda.synchronize()
+        assert np.max(np.abs(out.cpu().numpy() - ref)) <= 2e-13 * np.max(ref)  # as tests/test_gpu_readout.py
+        out.zero_()
+        torch.cuda.synchronize()
+
+    with sv.State(n, code) as s:
+        sv.sv_copy_in(s.h, psi)
+        sv.sv_fault_inject(sv.SV_FAULT_ALLOC, 0)
+        try:
+            sv.sv_probabilities_device(s.h, mask, out.data_ptr())
+        finally:
+            sv.sv_fault_inject(sv.SV_FAULT_ALLOC, -1)
+        check()
+
+    amps = torch.from_numpy(psi).cuda()
+    stream = torch.cuda.Stream()
+    with sv.State(n, code, tensor=amps, stream=stream) as s:
+        sv.sv_info(s.h)
+        torch.cuda.synchronize()
+        amps.copy_(torch.from_numpy(psi))
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=stream):
+            sv.sv_probabilities_device(s.h, mask, out.data_ptr())
+        g.replay()
+        check()
