@@ -85,7 +85,9 @@ typedef enum {
  *               SV_MAT with the same target and control, rows 1..3
  *   SV_MAT      a row of the preceding SV_U2Q (valid only there)
  *   SV_MEASURE  projective measurement of `target` with the caller's uniform
- *               u = p[0] in [0,1): p0 and p1 are the FP64 sums of |amp|^2 over
+ *               u = p[0] in [0,1): p0 and p1 are the sums of |amp|^2, to
+ *               FP64 accuracy in both dtypes and over the whole range
+ *               of the amplitudes' type, over
  *               the amplitudes with that qubit 0 and 1; the outcome is the
  *               smallest i with C_i > u * C_last for C = (p0, p0 + p1) (as
  *               sv_sample); the other half of the state becomes 0 and the kept

@@ -6,7 +6,7 @@
 // controls: the pair (x, x + 2^t) is updated only when every control bit of
 // x is 1, so the kernel enumerates exactly those pairs (2^(n-1-k) of them).
 // U2Q updates the four amplitudes that agree off its two qubits.  MEASURE
-// sums |amp|^2 over each value of its qubit in FP64 (per-block partials in a
+// sums |amp|^2 over each value of its qubit to FP64 accuracy (partials in a
 // fixed tree, then the blocks in a fixed tree), picks the outcome on the
 // device as the smallest i with C_i > u C_last for C = (p0, p0 + p1), and
 // collapses the state: the other half is zeroed and the kept one divided by
