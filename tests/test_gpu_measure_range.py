@@ -55,3 +55,18 @@ def test_a_small_half(sv, orc, n, q, small):
     psi /= np.linalg.norm(psi)
     psi[((np.arange(1 << n) >> q) & 1) == 0] *= small
     check(sv, orc, n, psi, q, 0.0)
+
+
+@pytest.mark.parametrize("n,q,q0", [(3, 1, 0), (5, 4, 0), (14, 0, 5), (14, 6, 0), (17, 9, 16), (17, 9, 9)])
+@pytest.mark.parametrize("scale", [1e-30, 1.0])
+def test_zeros_of_both_signs(sv, orc, n, q, q0, scale):
+    """A qubit q0 cleared by an earlier measurement, its zeros of either sign, and
+    few amplitudes left in the other half: zeros add nothing, the rest counts."""
+    rng = np.random.default_rng(n + q)
+    psi = (rng.normal(size=1 << n) + 1j * rng.normal(size=1 << n)) * scale
+    i = np.arange(1 << n)
+    psi[(((i >> q0) & 1) == 1) | (rng.random(1 << n) < 0.7)] = 0.0
+    psi[i[psi == 0][::2]] = complex(-0.0, -0.0)
+    psi[0] = scale
+    for u in (0.0, 0.999):
+        check(sv, orc, n, psi, q, u)
