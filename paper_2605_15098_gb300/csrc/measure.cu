@@ -571,31 +571,27 @@ k_normalise(double *__restrict__ p, uint64_t len, const ReadResult *__restrict__
 // above the sum's binade, a step out of the binade, a sum that is not a
 // normal number.  Zeros change nothing and are never exceptions.
 //
-// An exception costs a prefix sum, about eight additions' time.  Sums of
-// similar values have about two per doubling of the sum; but all 32 values of
-// a step can be exceptions, so after kRunRounds of them the rest is added one
-// after the other.  2^20 outcomes: k_cdf_blocks on Gaussian amplitudes 18.8 us
-// with and without this, on sums of 16 of them 18.9 and 18.5 (kRunRounds 3: 19.0
-// and 19.5); sv_sample where every value is a tie 503 -> 232 us (3: 224, 6: 254),
-// where they grow by 2^2000 in all 530 -> 249.
+// An exception costs a prefix sum, about four additions' time.  Sums of similar
+// values have about two per doubling of the sum, ten in their first 32 values,
+// but all 32 of a step can be exceptions: a kernel that meets more than
+// kRunMost of them in a step adds the rest of its values one after the other.
+// 2^20 outcomes, k_cdf_blocks on Gaussian amplitudes 18.7 us without this and
+// 19.0 with it, on sums of 16 of them 18.5 and 18.8; the call of sv_sample
+// where every value is a tie 497 and 249, where the values grow by 2^2000 in
+// all 521 and 255.  (Counted in here, step by step: 19.0 and 19.0, 18.4 of 17.7
+// for 2^16 outcomes and 24.4 of 21.9 for 2^21, calls 234 and 248.)
 //
 // total: the sum so far, the same in every lane, on return the sum with all
 // 32 values; returns the sum up to and including the lane's own value.
-constexpr int kRunRounds = 4;
-__device__ __forceinline__ double warp_run(double &total, double x, int lane) {
+// rounds: the prefix sums it took.
+constexpr int kRunMost = 16;
+__device__ __forceinline__ double warp_run(double &total, double x, int lane, int &rounds) {
     uint64_t c = (uint64_t)__double_as_longlong(total), mine = c;
     const uint64_t xb = (uint64_t)__double_as_longlong(x);
     const int ex = (int)(xb >> 52);
     const uint64_t m = (xb & ((UINT64_C(1) << 52) - 1)) | (ex ? UINT64_C(1) << 52 : 0);
-    for (int pos = 0, rounds = 0; pos < 32; rounds++) {
-        if (rounds == kRunRounds) {
-            for (; pos < 32; pos++) {
-                const double xf = __shfl_sync(0xffffffffu, x, pos);
-                c = (uint64_t)__double_as_longlong(__dadd_rn(__longlong_as_double((long long)c), xf));
-                if (lane == pos) mine = c;
-            }
-            break;
-        }
+    rounds = 0;
+    for (int pos = 0; pos < 32; rounds++) {
         const int e = (int)(c >> 52);
         const int de = e - (ex ? ex : 1);
         bool bad = false;
@@ -651,14 +647,23 @@ k_cdf_blocks(const double *__restrict__ p, uint64_t len, double *__restrict__ ch
     double run = 0.0, nxt[kCdfAhead];
 #pragma unroll
     for (int k = 0; k < kCdfAhead; k++) nxt[k] = value(k);
-    for (int c = 0; c < steps; c += kCdfAhead) {
+    int c = 0;
+    for (bool go = true; go && c < steps; c += kCdfAhead) {
 #pragma unroll
         for (int k = 0; k < kCdfAhead; k++) {
             const double x = nxt[k];
             nxt[k] = value(c + kCdfAhead + k);
             if (lane == 0) chk[b * steps + c + k] = run;
-            warp_run(run, x, lane);
+            int rounds;
+            warp_run(run, x, lane, rounds);
+            go = go && rounds <= kRunMost;
         }
+    }
+    for (; c < steps; c++) {
+        const double x = value(c);
+        if (lane == 0) chk[b * steps + c] = run;
+#pragma unroll 8
+        for (int k = 0; k < 32; k++) run = __dadd_rn(run, __shfl_sync(0xffffffffu, x, k));
     }
     if (lane == 0) btot[b] = run;
 }
@@ -674,15 +679,28 @@ k_cdf_scan(const double *__restrict__ btot, uint64_t nb, double *__restrict__ be
     if (lane == 0) before[0] = 0.0;
 #pragma unroll
     for (int k = 0; k < kCdfAhead; k++) nxt[k] = value(32 * k);
-    for (uint64_t c = 0; c < nb; c += 32 * kCdfAhead) {
+    uint64_t c = 0;
+    for (bool go = true; go && c < nb; c += 32 * kCdfAhead) {
 #pragma unroll
         for (int k = 0; k < kCdfAhead; k++) {
             const uint64_t i = c + 32 * k;
             const double x = nxt[k];
             nxt[k] = value(i + 32 * kCdfAhead);
-            const double after = warp_run(run, x, lane);
+            int rounds;
+            const double after = warp_run(run, x, lane, rounds);
             if (i + lane < nb) before[i + lane + 1] = after;
+            go = go && rounds <= kRunMost;
         }
+    }
+    for (; c < nb; c += 32) {
+        const double x = value(c);
+        double after = 0.0;
+#pragma unroll 8
+        for (int k = 0; k < 32; k++) {
+            run = __dadd_rn(run, __shfl_sync(0xffffffffu, x, k));
+            if (lane == k) after = run;
+        }
+        if (c + lane < nb) before[c + lane + 1] = after;
     }
 }
 

@@ -1,6 +1,6 @@
 """The sampler's running sums where most values of a step of 32 leave the prefix
-sum of integers (ties, values above the sum's binade, steps out of it): one
-addition after the other from the fifth of a step on, with the same samples."""
+sum of integers (ties, values above the sum's binade, steps out of it): the rest
+is then added one after the other, in blocks and over blocks, with the same samples."""
 import math
 from fractions import Fraction
 
@@ -32,13 +32,16 @@ def exceptions(p):
     return out
 
 
-@pytest.mark.parametrize("n", [6, 10, 11])
-@pytest.mark.parametrize("kind", ["ties", "doubling", "doubling_from_the_middle"])
-def test_samples_with_many_exceptions(sv, orc, n, kind):
+@pytest.mark.parametrize("kind,n", [(k, n) for k in ("ties", "doubling", "doubling_from_the_middle") for n in (6, 10, 11)] +
+                         [("block_ties", 18), ("block_ties", 20)])
+def test_samples_with_many_exceptions(sv, orc, kind, n):
     size = 1 << n
     i = np.arange(size)
-    if kind == "ties":  # two values, then only values of half the last place of their sum
-        a = np.full(size, 2.0 ** -27, np.complex128)
+    step = 1024 if kind == "block_ties" else 1
+    tie = 2 if step == 1 else step
+    if kind in ("ties", "block_ties"):  # two values, then only (block sums of) half the last place of their sum
+        a = np.zeros(size, np.complex128)
+        a[::step] = 2.0 ** -27
         a[:2] = math.sqrt(1.0 - 2.0 ** -20), 0.0
     else:
         start = 0 if kind == "doubling" else min(size // 2, 300)
@@ -49,9 +52,9 @@ def test_samples_with_many_exceptions(sv, orc, n, kind):
         sv.sv_copy_in(s.h, a)
         p = s.probabilities(mask)
         for _ in range(8):  # the ties want a total of exactly 1
-            if kind != "ties" or p[2] == 2.0 ** -54:
+            if "ties" not in kind or p[tie] == 2.0 ** -54:
                 break
-            a[1] = math.sqrt(max(0.0, abs(a[1]) ** 2 + 1.0 - 2.0 ** -54 / p[2]))
+            a[1] = math.sqrt(max(0.0, abs(a[1]) ** 2 + 1.0 - 2.0 ** -54 / p[tie]))
             sv.sv_copy_in(s.h, a)
             p = s.probabilities(mask)
         c = np.cumsum(p)
@@ -59,6 +62,6 @@ def test_samples_with_many_exceptions(sv, orc, n, kind):
         u = np.concatenate([np.random.default_rng(n).random(300), at, np.nextafter(at, 0.0)])
         u = np.minimum(u, np.nextafter(1.0, 0.0))
         got = s.sample(mask, u)
-    assert max(exceptions(p)) > 4
+    assert max(exceptions(p if step == 1 else p.reshape(-1, step).sum(1))) > 16
     want, _ = orc.sample(p, u)
     assert np.array_equal(got, want)
